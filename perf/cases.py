@@ -242,8 +242,8 @@ class Scene:
             pix = torch.gather(order[node], 1, torch.minimum(k, masked[node][:, None] - 1))
             return torch.gather(surface[node], 1, pix[..., None].expand(-1, -1, 3))
 
-        T = torch.tensor(self.true, device="cuda", dtype=torch.float32)
-        M = T[j] @ torch.linalg.inv(T[i])
+        M = np.stack([self.true[q] @ np.linalg.inv(self.true[p]) for p, q in self.pairs])
+        M = torch.tensor(M, device="cuda", dtype=torch.float32)
         pi = points(i)
         pj = pi @ M[:, :3, :3].transpose(1, 2) + M[:, None, :3, 3]
         u, v = (pj[..., 0] / pj[..., 2] * fx + cx).round().long(), (pj[..., 1] / pj[..., 2] * fy + cy).round().long()
