@@ -330,7 +330,6 @@ int bthost::build_topology(bt_graph* g, int tile)
     a.n_upairs = U;
     a.tile = tile;
     a.precision = g->cfg.precision;
-    a.stage_blocks = bt::reduce_stage_fits(nfree, N) ? 1 : 0;
     const bt_config& c = g->cfg;
     a.dmax2 = (float)(c.dense_max_dist * c.dense_max_dist);
     a.cmin = (float)std::cos(c.dense_max_normal_deg * 3.14159265358979323846 / 180.0);
@@ -879,7 +878,7 @@ int batch_build(bt_batch* b, int shape)
         for (int t = 0; t < a.n_tiles; ++t) wres.push_back(make_int2((int)k, a.n_edges + t));
         for (int u = 0; u < a.n_upairs; ++u) wpair.push_back(make_int2((int)k, u));
         b->max_N = std::max(b->max_N, a.N);
-        b->solve_smem = std::max(b->solve_smem, bt::reduce_smem_bytes(a.n_free, a.N));
+        b->solve_smem = std::max(b->solve_smem, bt::reduce_smem_bytes(a.n_free));
         b->pixels_per_pass += g->pixels_per_pass;
     }
     cudaStream_t s = b->stream;

@@ -89,7 +89,6 @@ struct SolveArgs {
     int N, n_tiles, n_pairs, n_edges, n_free, n_upairs;
     int precision;          // storage precision of the per-pixel maps (BT_FP32 / BT_BF16 / BT_FP16)
     int tile;               // source pixels per dense tile (CTA shape product)
-    int stage_blocks;       // 1: the last CTA copies the pair blocks to shared memory
     float dmax2, cmin, huber_dense, huber_sparse;
     double lambda_dense, lambda_sparse;
     int solver;             // BT_SOLVER_CHOLESKY / BT_SOLVER_PCG
@@ -195,8 +194,7 @@ cudaError_t launch_reduce(const SolveArgs& a, bool full, int iter, cudaStream_t 
 // against node j at the current transforms (out: device, nodes[i].M ints).
 cudaError_t launch_assoc_debug(const SolveArgs& a, int i, int j, int M, int* out, cudaStream_t s);
 
-size_t reduce_smem_bytes(int n_free, int N);
-bool reduce_stage_fits(int n_free, int N);
+size_t reduce_smem_bytes(int n_free);
 size_t residual_smem_bytes(int N, int shape);
 inline int shape_tile(int shape) { return kShapeThreads[shape] * kShapePix[shape]; }
 

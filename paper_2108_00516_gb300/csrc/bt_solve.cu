@@ -1,7 +1,7 @@
 // bt_solve.cu -- sm_103a kernels of the pose-graph solve (BundleTrack, Sec. IV-D):
 // single-precision transforms of the FP64 poses, the reduction of the residual
 // pass's FP32 partials into FP64 6x6 blocks, the assembly of the normal
-// equations, the FP64 Cholesky (LDL^T) solve and the FP64 se(3) update, for one
+// equations, the Cholesky (LDL^T) solve and the FP64 se(3) update, for one
 // graph (reduce_kernel) or a batch of graphs (batch_*_kernel).
 //
 //   reduce_kernel   one CTA per unordered node pair turns the FP32 partials of
@@ -366,8 +366,8 @@ __device__ double se3_exp_entry(const double* xi, const double* cf, int r, int c
 }
 
 // Last CTA: energies, then (full) assembly of H and g over the free nodes,
-// the FP64 solve of H dx = -g (square-root-free Cholesky with a one-column
-// look-ahead, bt_ldlt.h; or PCG, the paper's inner solver), and finally
+// the solve of H dx = -g (square-root-free Cholesky in double-float
+// arithmetic, bt_ldlt.h; or PCG, the paper's inner solver, in FP64), and finally
 // T <- T exp(dx).
 // The first global reads of the last CTA, issued by every CTA of the reduce
 // kernel before its pair stage: the last CTA is only known after the
@@ -403,16 +403,16 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x;
     const int nf = a.n_free, n = 6 * nf;
     const int status0 = kFull ? pf.status : 0;
-    // energies of the iteration: from the staged pair blocks when a full
-    // solve stages them, else straight from global memory
-    const bool staged_costs = kFull && n > 0 && status0 == 0 && a.stage_blocks != 0;
-    auto write_costs = [&](const double* blocks, bool shared) {
+    // energies of the iteration, by one warp: at once when there is no
+    // system to solve, else while warp 0 is busy alone
+    const bool solves = kFull && n > 0 && status0 == 0;
+    auto write_costs = [&]() {
         double ed = 0.0, es = 0.0, cnt = 0.0;
         for (int u = lane; u < U; u += 32) {
-            const double* o = blocks + (size_t)u * kUPairBlk;
-            ed += shared ? o[90] : __ldcg(o + 90);
-            es += shared ? o[91] : __ldcg(o + 91);
-            cnt += shared ? o[92] : __ldcg(o + 92);
+            const double* o = a.upairblk + (size_t)u * kUPairBlk;
+            ed += __ldcg(o + 90);
+            es += __ldcg(o + 91);
+            cnt += __ldcg(o + 92);
         }
 #pragma unroll
         for (int off = 16; off >= 1; off >>= 1) {
@@ -427,55 +427,62 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
             a.costs[iter * 4 + 3] = cnt;
         }
     };
-    if (!staged_costs && tid < 32) write_costs(a.upairblk, false);
-    if (!kFull || n == 0 || status0 != 0) return;
+    if (!solves) {
+        if (tid < 32) write_costs();
+        return;
+    }
     unsigned long long t0 = clock64();
     const int ld = n + 1;        // odd leading dimension: conflict-free FP64 rows
     double* H = sm;              // n*ld: lower triangle H, then L^T in the upper triangle
     double* y = H + n * ld;      // n
-    double* rD = y + n;          // n: 1 / D_k
+    double* rD = y + n;          // n: scratch (PCG, the update)
     double* ps = rD + n;         // 12 * N poses
     double* tinv = ps + 12 * kMaxNodes;   // 12 * N
-    // tinv + 12 * kMaxNodes: [2][n] scaled columns, then the triangle index
-    // table (n (n+1) / 2 ints, rounded up to whole doubles), then the staged
-    // pair blocks
-    const size_t tab_dbl = ((size_t)n * (n + 1) / 2 + 1) / 2;
-    double* stage = tinv + 12 * kMaxNodes + 2 * n + tab_dbl;
-    if (((size_t)(stage - sm)) & 1) ++stage;               // 16-byte alignment for double2
-    const size_t stage_len = a.stage_blocks ? (size_t)U * kUPairBlk : 0;
-    int* node_of = reinterpret_cast<int*>(stage + stage_len);
+    // tinv + 12 * kMaxNodes: the solve's panels and scaling exponents (bt_ldlt.h)
+    double* colb = tinv + 12 * kMaxNodes;    // 16-byte aligned: n is even
+    double* shift = colb + ldlt_pan_doubles(n);
+    int* node_of = reinterpret_cast<int*>(shift + ldlt_shift_doubles(n));
+    double* scratch = reinterpret_cast<double*>(node_of + kMaxNodes);      // 264 doubles
     __shared__ int s_fail;
     if (tid < N && pf.free_idx >= 0) node_of[pf.free_idx] = tid;
     if (tid < 12 * N) ps[tid] = pf.pose0;
     if (tid + nt < 12 * N) ps[tid + nt] = pf.pose1;
     if (tid == 0) s_fail = 0;
-    {   // pair blocks to shared memory, up to twelve independent loads in
-        // flight per thread (one round for ten nodes: each round costs an
-        // L2 round trip)
-        const double2* src = reinterpret_cast<const double2*>(a.upairblk);
-        double2* dst = reinterpret_cast<double2*>(stage);
-        const int n2 = (int)(stage_len / 2);
-        for (int q0 = tid; q0 < n2; q0 += 12 * nt) {
-            double2 v[12];
-#pragma unroll
-            for (int k = 0; k < 12; ++k) {
-                const int q = q0 + k * nt;
-                if (q < n2) v[k] = __ldcg(src + q);
-            }
-#pragma unroll
-            for (int k = 0; k < 12; ++k) {
-                const int q = q0 + k * nt;
-                if (q < n2) dst[q] = v[k];
-            }
-        }
-    }
     __syncthreads();
-    // (with staged blocks the energies are added up during the update, by a
-    // warp that has no other work there: here their FP64 adds would hold
-    // one sub-partition's DP unit beside its share of the diagonal sums)
+    // Assembly straight from the pair blocks in L2.  What it costs is L2
+    // round trips and FP64 adds, so each thread has up to twelve loads in
+    // flight (cycles, against staging the blocks in shared memory first: ten
+    // nodes 7.4 k -> 7.5 k; twenty nodes, whose blocks do not fit there,
+    // 59.6 k -> 28.6 k, and no staging room is needed).
     const int cost_warp = (nt >> 5) - 1;
-    const bool staged = a.stage_blocks != 0;
-    auto blk = [&](size_t q) { return staged ? stage[q] : __ldcg(a.upairblk + q); };
+    constexpr int kFly = 12;
+    const double* blk = a.upairblk;
+    // off-diagonal blocks (fa > fb)
+    const int nob = nf * (nf - 1) / 2;
+    for (int q0 = tid; q0 < nob * 36; q0 += kFly * nt) {
+        double v[kFly];
+        int at[kFly];
+#pragma unroll
+        for (int x = 0; x < kFly; ++x) {
+            const int q = q0 + x * nt;
+            at[x] = -1;
+            if (q >= nob * 36) continue;
+            const int b = q / 36, e = q % 36, rr = e / 6, cc = e % 6;
+            // b = fa (fa - 1) / 2 + fb with fb < fa: fa from the square root,
+            // corrected by one step either way (b < 253, exact in FP32)
+            int fa = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)b)) * 0.5f);
+            if (fa * (fa - 1) / 2 > b) --fa;
+            if (fa * (fa + 1) / 2 <= b) ++fa;
+            const int fb = b - fa * (fa - 1) / 2;
+            const int A = node_of[fa], B = node_of[fb];
+            const int u = A < B ? upair_index(A, B, N) : upair_index(B, A, N);
+            at[x] = (6 * fa + rr) * ld + 6 * fb + cc;
+            v[x] = __ldcg(blk + (size_t)u * kUPairBlk + 42 + (A < B ? rr * 6 + cc : cc * 6 + rr));
+        }
+#pragma unroll
+        for (int x = 0; x < kFly; ++x)
+            if (at[x] >= 0) H[at[x]] = v[x];
+    }
     // diagonal blocks and gradient: one thread per (free node, value), values
     // 0-20 the unique block entries, 21-26 the gradient entries (all the
     // warps' FP64 pipes at once rather than one warp per node)
@@ -483,11 +490,21 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
         const int f = q / 27, v = q - 27 * f;
         const int A = node_of[f];
         double s0 = 0.0, s1 = 0.0;
-        for (int k = 0; k < N; ++k) {
-            if (k == A) continue;
-            const int u = A < k ? upair_index(A, k, N) : upair_index(k, A, N);
-            const size_t off = (size_t)u * kUPairBlk + (v < 21 ? (A < k ? 0 : 21) + v : (A < k ? 78 : 84) + v - 21);
-            if (k & 1) s1 += blk(off); else s0 += blk(off);
+        for (int k0 = 0; k0 < N; k0 += kFly) {
+            double x[kFly];
+#pragma unroll
+            for (int y2 = 0; y2 < kFly; ++y2) {
+                const int k = k0 + y2;
+                x[y2] = 0.0;
+                if (k >= N || k == A) continue;
+                const int u = A < k ? upair_index(A, k, N) : upair_index(k, A, N);
+                x[y2] = __ldcg(blk + (size_t)u * kUPairBlk + (v < 21 ? (A < k ? 0 : 21) + v : (A < k ? 78 : 84) + v - 21));
+            }
+#pragma unroll
+            for (int y2 = 0; y2 < kFly; ++y2) {
+                if (k0 + y2 >= N) break;
+                if (y2 & 1) s1 += x[y2]; else s0 += x[y2];
+            }
         }
         const double s = s0 + s1;
         if (v < 21) {
@@ -499,20 +516,6 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
             y[6 * f + v - 21] = -s;   // right-hand side of H dx = -g
         }
     }
-    // off-diagonal blocks (fa > fb)
-    const int nob = nf * (nf - 1) / 2;
-    for (int q = tid; q < nob * 36; q += nt) {
-        const int b = q / 36, e = q % 36, rr = e / 6, cc = e % 6;
-        // b = fa (fa - 1) / 2 + fb with fb < fa: fa from the square root,
-        // corrected by one step either way (b < 253, exact in FP32)
-        int fa = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)b)) * 0.5f);
-        if (fa * (fa - 1) / 2 > b) --fa;
-        if (fa * (fa + 1) / 2 <= b) ++fa;
-        const int fb = b - fa * (fa - 1) / 2;
-        const int A = node_of[fa], B = node_of[fb];
-        const int u = A < B ? upair_index(A, B, N) : upair_index(B, A, N);
-        H[(6 * fa + rr) * ld + 6 * fb + cc] = blk((size_t)u * kUPairBlk + 42 + (A < B ? rr * 6 + cc : cc * 6 + rr));
-    }
     __syncthreads();
     if (a.ne_out != nullptr) {
         // diagnostic export of the assembled system (symmetric H, g = -y);
@@ -522,11 +525,10 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
             a.ne_out[q] = r >= c ? H[r * ld + c] : H[c * ld + r];
         }
         for (int q = tid; q < n; q += nt) a.ne_out[n * n + q] = -y[q];
-        if (staged_costs && warp == cost_warp) write_costs(stage, true);
+        if (warp == cost_warp) write_costs();
         return;
     }
     unsigned long long t1 = clock64();
-    double* colb = tinv + 12 * kMaxNodes;   // [2][n]
     unsigned long long t2, t3;
     if (a.solver == 1) {
         // Conjugate gradients with the diagonal preconditioner (the paper's
@@ -539,7 +541,7 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
         double* rv = y;              // residual, starts as -g
         double* zv = rD;             // preconditioned residual
         double* qv = tinv;           // H p
-        double* part = reinterpret_cast<double*>(node_of + kMaxNodes);   // [n * C]
+        double* part = scratch;      // [n * C]
         double* red = part + 256;    // [8]
         const int C = nt / n > 0 ? nt / n : 1;
         const int w = (n + C - 1) / C;
@@ -606,28 +608,27 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
         }
         if (s_fail) {
             if (tid == 0) a.ctrl->status = -4;
-            if (staged_costs && warp == cost_warp) write_costs(stage, true);
+            if (warp == cost_warp) write_costs();
             return;
         }
         for (int i = tid; i < n; i += nt) y[i] = xv[i];
         __syncthreads();
         t2 = t3 = clock64();
     } else {
-    // LDL^T with a one-column look-ahead, D w = z, blocked L^T dx = w
+    // LDL^T in panels of six columns, D w = z, blocked L^T dx = w
     // (bt_ldlt.h); the forward substitution of -g is carried along
     LdltScratch sc;
-    sc.rD = rD;
-    sc.colb = colb;
-    sc.tab = reinterpret_cast<int*>(colb + 2 * n);
-    sc.part = reinterpret_cast<double*>(node_of + kMaxNodes);
+    sc.pan = colb;
+    sc.shift = reinterpret_cast<int*>(shift);
+    sc.part = scratch;
     // the energies are added up by the last warp while warp 0 runs the
     // first block of the back substitution alone
     ldlt_solve(H, ld, n, y, sc, &s_fail, t2, [&](int w) {
-        if (staged_costs && w == cost_warp) write_costs(stage, true);
+        if (w == cost_warp) write_costs();
     });
     if (s_fail) {
         if (tid == 0) a.ctrl->status = -4;
-        if (staged_costs && warp == cost_warp) write_costs(stage, true);
+        if (warp == cost_warp) write_costs();
         return;
     }
     __syncthreads();
@@ -636,7 +637,7 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
     // T_A <- T_A exp(dx_A) in three steps: the coefficients of exp per node
     // (warps 0-2, one coefficient each, so the three FP64 chains run on
     // three sub-partitions), the entries of exp(dx_A) (one thread each), the
-    // products T_A exp(dx_A) (one thread each).  The look-ahead columns, rD
+    // products T_A exp(dx_A) (one thread each).  The solve's scratch, rD
     // and tinv are free now (after PCG the last warp adds up the energies
     // meanwhile; the Cholesky path has done so during its back substitution).
     {
@@ -649,7 +650,7 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
             cf[4 * lane + 1 + warp] = c;
             if (warp == 0) cf[4 * lane] = fma(xi[5], xi[5], fma(xi[4], xi[4], xi[3] * xi[3]));
         }
-        if (a.solver == 1 && staged_costs && warp == cost_warp) write_costs(stage, true);
+        if (a.solver == 1 && warp == cost_warp) write_costs();
         __syncthreads();
         for (int q = tid; q < 12 * nf; q += nt) {
             // rotation entries (f, r, c < 3) first, then the translations
@@ -681,8 +682,8 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
     }
     __syncthreads();
     for (int q = tid; q < 12 * N; q += nt) a.pose[q] = ps[q];
-    // split scratch from tinv on (32 N floats: tinv, the look-ahead columns,
-    // the triangle table and the staged blocks are free now)
+    // split scratch from tinv on (32 N floats: tinv, the solve's scratch
+    // is free now)
     write_xforms(a, reinterpret_cast<float*>(tinv), ps);
     if (tid == 0) {
         unsigned long long t4 = clock64();
@@ -717,24 +718,15 @@ __global__ void __launch_bounds__(kThreads, 1) reduce_kernel(SolveArgs a, int it
     final_phase<kFull>(a, iter, sm, pf);
 }
 
-static size_t reduce_smem_bytes_for(int n_free, int N, bool stage)
+size_t reduce_smem_bytes(int n_free)
 {
     const size_t n = 6 * (size_t)n_free;
-    const size_t U = (size_t)N * (N - 1) / 2;
-    const size_t sl = stage ? U * kUPairBlk : 0;
-    const size_t tab_dbl = (n * (n + 1) / 2 + 1) / 2;
-    // ... + the PCG scratch after node_of: 256 partial sums + 8 warp sums
-    size_t fin = (n * (n + 1) + 4 * n + 24 * (size_t)kMaxNodes + tab_dbl + 1 + sl + 264) * sizeof(double) +
-                 kMaxNodes * sizeof(int);
-    size_t ph1 = kPairSmemDoubles * sizeof(double);
+    // H, y, two poses' worth a node, the solve's panels and exponents, the
+    // node table, 256 partial sums + 8 warp sums
+    const size_t fin = (n * (n + 1) + 2 * n + 24 * (size_t)kMaxNodes + ldlt_pan_doubles(n) + ldlt_shift_doubles(n) + 264) *
+                           sizeof(double) + kMaxNodes * sizeof(int);
+    const size_t ph1 = kPairSmemDoubles * sizeof(double);
     return fin > ph1 ? fin : ph1;
-}
-
-bool reduce_stage_fits(int n_free, int N) { return reduce_smem_bytes_for(n_free, N, true) <= kReduceSmemMax; }
-
-size_t reduce_smem_bytes(int n_free, int N)
-{
-    return reduce_smem_bytes_for(n_free, N, reduce_stage_fits(n_free, N));
 }
 
 cudaError_t launch_reduce(const SolveArgs& a, bool full, int iter, cudaStream_t s)
@@ -746,7 +738,7 @@ cudaError_t launch_reduce(const SolveArgs& a, bool full, int iter, cudaStream_t 
     }();
     (void)attr_set;
     const int grid = a.n_upairs > 0 ? a.n_upairs : 1;
-    const size_t smem = reduce_smem_bytes(a.n_free, a.N);
+    const size_t smem = reduce_smem_bytes(a.n_free);
     if (full)
         return launch_chained(reduce_kernel<true>, dim3(grid), dim3(kThreads), smem, s, a, iter);
     return launch_chained(reduce_kernel<false>, dim3(grid), dim3(kThreads), smem, s, a, iter);

@@ -934,12 +934,11 @@ __global__ void __launch_bounds__(kAvgThreads) average_kernel(const AvgGraph* __
     double* H = sT + 12 * N;                 // [n][ld]
     double* b = H + (size_t)n * ld;          // [n]
     LdltScratch sc;                          // the solve's scratch (bt_ldlt.h)
-    sc.rD = b + n;                           // [n]
-    sc.colb = sc.rD + n;                     // [2n]
-    sc.part = sc.colb + 2 * n;               // [256]
+    sc.pan = b + n;                          // 16-byte aligned: n is even
+    sc.part = sc.pan + ldlt_pan_doubles(n);  // [256]
     int* eof = reinterpret_cast<int*>(sc.part + 256);   // [N][N]
     int* freenode = eof + N * N;             // [nf]
-    sc.tab = freenode + nf;                  // [n (n + 1) / 2]
+    sc.shift = freenode + nf;
     const double Wd[6] = {1.0 / (kSU * kSU), 1.0 / (kSU * kSU), 1.0 / (kSU * kSU),
                           1.0 / (kSW * kSW), 1.0 / (kSW * kSW), 1.0 / (kSW * kSW)};
     if (tid == 0) s_sing = 0;
@@ -1075,7 +1074,7 @@ __global__ void __launch_bounds__(kAvgThreads) average_kernel(const AvgGraph* __
         b[r] = v;
     }
     __syncthreads();
-    // 4-5. H d = b by LDL^T with a one-column look-ahead (bt_ldlt.h); a
+    // 4-5. H d = b by LDL^T in double-float arithmetic (bt_ldlt.h); a
     // pivot that is not positive, or a solution that is not finite, leaves
     // the poses as they were
     if (n > 0) {
@@ -1158,8 +1157,8 @@ cudaError_t launch_adam(Net net, const float* grad, float lr, float beta1, float
 size_t average_smem_bytes(int max_free, int max_N)
 {
     const size_t n = 6 * (size_t)max_free;
-    return sizeof(double) * (24 * (size_t)max_N + n * (n + 1) + 4 * n + 256) +
-           sizeof(int) * ((size_t)max_N * max_N + max_free + n * (n + 1) / 2) + 16;
+    return sizeof(double) * (24 * (size_t)max_N + n * (n + 1) + n + ldlt_pan_doubles(n) + 256 + ldlt_shift_doubles(n)) +
+           sizeof(int) * ((size_t)max_N * max_N + max_free) + 16;
 }
 
 cudaError_t launch_average(const AvgGraph* graphs, int n_graphs, int max_free, cudaStream_t s)
