@@ -491,7 +491,7 @@ int64_t bt_debug_tensor_wait_ns(int64_t ns);
  * k-th: see bt_profile_enable); the pixel-pair and correspondence counts
  * below cover the same timed launches. */
 typedef struct {
-    int64_t prep_launches;      /* frame-preparation kernels (3 per frame) */
+    int64_t prep_launches;      /* frame-preparation kernels (2 per frame) */
     int64_t xform_launches;     /* transform kernels: always 0 (a solve's first
                                  * transforms are formed on the host, the later
                                  * ones by the update in the reduce kernel);

@@ -622,7 +622,7 @@ int bt_add_frame(bt_graph* g, const float* depth, const float* normals, const ui
             f.slot = -1;
         }
     }
-    g->prof.prep_launches += 3;
+    g->prof.prep_launches += 2;
     if (e != cudaSuccess) {
         g->pool.put(f.tgt, f.tgt_bytes);
         g->pool.put(f.src_p, f.src_bytes);

@@ -44,42 +44,29 @@ namespace bt {
 // K0: frame preparation
 // ---------------------------------------------------------------------------
 
-__device__ __forceinline__ bool pixel_valid(const float* depth, const float* normals,
-                                            const uint8_t* mask, int pix, float& z, float3& n)
-{
-    if (!mask[pix]) return false;
-    z = depth[pix];
-    if (!(z > 0.f) || !isfinite(z)) return false;
-    n = make_float3(normals[3 * pix], normals[3 * pix + 1], normals[3 * pix + 2]);
-    return isfinite(n.x) && isfinite(n.y) && isfinite(n.z);
-}
+// A warp takes kPixPerThread groups of 32 consecutive pixels, one pixel a
+// lane, so that every load and store of a group is contiguous and a pixel's
+// rank among the valid ones follows from ballots.
+struct Pixel {
+    float z;
+    float3 n;
+    bool ok;
+};
 
-__device__ __forceinline__ int block_exclusive_scan(int v, int* total, int* sm /* >= 33 */)
+// The pixel's mask, depth and normal, all loads issued together (gating the
+// normal on the mask and the depth would make them a chain of three).
+__device__ __forceinline__ Pixel load_pixel(const float* depth, const float* normals, const uint8_t* mask, int pix,
+                                            int HW)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
+    Pixel x{0.f, make_float3(0.f, 0.f, 0.f), false};
+    if (pix < HW) {
+        const uint8_t m = __ldg(mask + pix);
+        x.z = __ldg(depth + pix);
+        const float* n = normals + 3 * (size_t)pix;
+        x.n = make_float3(__ldg(n), __ldg(n + 1), __ldg(n + 2));
+        x.ok = m != 0 && x.z > 0.f && isfinite(x.z) && isfinite(x.n.x) && isfinite(x.n.y) && isfinite(x.n.z);
     }
-    if (lane == 31) sm[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-        const int nw = blockDim.x >> 5;
-        int w = lane < nw ? sm[lane] : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int y = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += y;
-        }
-        if (lane < nw) sm[lane] = w;       // inclusive warp totals
-        if (lane == nw - 1) sm[32] = w;
-    }
-    __syncthreads();
-    const int before = warp > 0 ? sm[warp - 1] : 0;
-    *total = sm[32];
-    return before + x - v;
+    return x;
 }
 
 // 16-bit storage helpers (BF16 / FP16 as raw bits)
@@ -107,121 +94,183 @@ size_t prep_scratch_bytes(int HW)
     return (nblk + 1) * (sizeof(int) + sizeof(double)) + 16;
 }
 
-// Validity, count and depth sum of each block of kPrepPix pixels.
+// Count of valid pixels of each block of kPrepPix pixels and, for the 16-bit
+// encodings (kSum), the sum of their depths.
+template <bool kSum>
 __global__ void __launch_bounds__(kThreads) prep_count_kernel(
     const float* __restrict__ depth, const float* __restrict__ normals,
     const uint8_t* __restrict__ mask, int HW, int* __restrict__ blockcnt, double* __restrict__ blocksum)
 {
-    __shared__ int sm[33];
+    __shared__ int sc[kThreads / 32];
     __shared__ double sz[kThreads / 32];
-    const int base = blockIdx.x * kPrepPix + threadIdx.x * kPixPerThread;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int base = blockIdx.x * kPrepPix + warp * (32 * kPixPerThread) + lane;
+    Pixel px[kPixPerThread];
+#pragma unroll
+    for (int k = 0; k < kPixPerThread; ++k) px[k] = load_pixel(depth, normals, mask, base + 32 * k, HW);
     int c = 0;
-    float zs = 0.f;
+    double dz = 0.0;
 #pragma unroll
     for (int k = 0; k < kPixPerThread; ++k) {
-        const int pix = base + k;
-        if (pix < HW) {
-            float z;
-            float3 n;
-            if (pixel_valid(depth, normals, mask, pix, z, n)) {
-                ++c;
-                zs += z;
-            }
+        c += __popc(__ballot_sync(0xffffffffu, px[k].ok));
+        if constexpr (kSum) {      // four neighbours in FP32, then FP64
+            const float z = px[k].ok ? px[k].z : 0.f;
+            float q = z + __shfl_down_sync(0xffffffffu, z, 1);
+            q += __shfl_down_sync(0xffffffffu, z, 2);
+            q += __shfl_down_sync(0xffffffffu, z, 3);
+            if ((lane & 3) == 0) dz += (double)q;
         }
     }
-    int total;
-    block_exclusive_scan(c, &total, sm);
-    double dz = zs;
+    if constexpr (kSum) {
 #pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) dz += __shfl_xor_sync(0xffffffffu, dz, o);
-    if ((threadIdx.x & 31) == 0) sz[threadIdx.x >> 5] = dz;
+        for (int o = 16; o >= 4; o >>= 1) dz += __shfl_xor_sync(0xffffffffu, dz, o);
+    }
+    if (lane == 0) {
+        sc[warp] = c;
+        sz[warp] = dz;
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
+        int total = 0;
         double t = 0.0;
-        for (int w = 0; w < kThreads / 32; ++w) t += sz[w];
+        for (int w = 0; w < kThreads / 32; ++w) {
+            total += sc[w];
+            t += sz[w];
+        }
         blockcnt[blockIdx.x] = total;
-        blocksum[blockIdx.x] = t;
-    }
-}
-
-// Exclusive scan of the block counts; M and the reference depth (mean valid
-// depth, used by the 16-bit encodings).
-__global__ void prep_scan_kernel(int* __restrict__ blockcnt, const double* __restrict__ blocksum, int nblk,
-                                 int* __restrict__ out2, int* __restrict__ host_out2)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        int s = 0;
-        double z = 0.0;
-        for (int b = 0; b < nblk; ++b) {
-            const int c = blockcnt[b];
-            blockcnt[b] = s;
-            s += c;
-            z += blocksum[b];
-        }
-        out2[0] = s;
-        out2[1] = __float_as_int(s > 0 ? (float)(z / s) : 0.f);
-        if (host_out2) {      // the host's read-back slot (mapped pinned memory)
-            host_out2[0] = out2[0];
-            host_out2[1] = out2[1];
-        }
+        if constexpr (kSum) blocksum[blockIdx.x] = t;
     }
 }
 
 // Target map of every pixel and the compacted source list of the valid ones.
+// A CTA takes a run of consecutive blocks.  It adds up the counts of all
+// blocks before its own for itself (a scan kernel between the two would be
+// one more launch; the serial one this replaced took 28 us of a VGA frame's
+// 42); the last CTA writes the valid count M, and every CTA of a 16-bit
+// encoding forms the reference depth, the mean valid depth.
 template <int P>
 __global__ void __launch_bounds__(kThreads) prep_write_kernel(
     const float* __restrict__ depth, const float* __restrict__ normals,
     const uint8_t* __restrict__ mask, int W, int HW, float cx, float cy, float ifx, float ify,
-    const int* __restrict__ blockoff, const int* __restrict__ out2, void* __restrict__ tgt_v,
-    void* __restrict__ src_p_v, void* __restrict__ src_n_v)
+    const int* __restrict__ blockcnt, const double* __restrict__ blocksum, int nblk, int* __restrict__ out2,
+    int* __restrict__ host_out2, void* __restrict__ tgt_v, void* __restrict__ src_p_v, void* __restrict__ src_n_v)
 {
-    __shared__ int sm[33];
-    const int base = blockIdx.x * kPrepPix + threadIdx.x * kPixPerThread;
-    const float zref = P == 0 ? 0.f : __int_as_float(out2[1]);
-    bool ok[kPixPerThread];
-    float zz[kPixPerThread];
-    float3 nn[kPixPerThread];
-    int c = 0;
+    constexpr int kWarps = kThreads / 32;
+    __shared__ int sc[2][kWarps], sw[kWarps];
+    __shared__ double sz[kWarps];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int b0 = (int)((long long)blockIdx.x * nblk / gridDim.x), b1 = (int)((long long)(blockIdx.x + 1) * nblk / gridDim.x);
+    int before = 0, all = 0;
+    double z = 0.0;
+    for (int b = tid; b < nblk; b += kThreads) {
+        const int c = __ldg(blockcnt + b);
+        all += c;
+        before += b < b0 ? c : 0;
+        if constexpr (P != 0) z += __ldg(blocksum + b);
+    }
 #pragma unroll
-    for (int k = 0; k < kPixPerThread; ++k) {
-        const int pix = base + k;
-        ok[k] = pix < HW && pixel_valid(depth, normals, mask, pix, zz[k], nn[k]);
-        c += ok[k];
-        if (pix < HW) {
-            if constexpr (P == 0) {
-                reinterpret_cast<float4*>(tgt_v)[pix] =
-                    ok[k] ? make_float4(zz[k], nn[k].x, nn[k].y, nn[k].z) : make_float4(0.f, 0.f, 0.f, 0.f);
-            } else {
-                ushort4 t;
-                t.x = ok[k] ? to16<P>(zz[k] - zref) : nan16<P>();
-                t.y = ok[k] ? to16<P>(nn[k].x) : (unsigned short)0;
-                t.z = ok[k] ? to16<P>(nn[k].y) : (unsigned short)0;
-                t.w = ok[k] ? to16<P>(nn[k].z) : (unsigned short)0;
-                reinterpret_cast<ushort4*>(tgt_v)[pix] = t;
+    for (int o = 16; o >= 1; o >>= 1) {
+        before += __shfl_xor_sync(0xffffffffu, before, o);
+        all += __shfl_xor_sync(0xffffffffu, all, o);
+        if constexpr (P != 0) z += __shfl_xor_sync(0xffffffffu, z, o);
+    }
+    if (lane == 0) {
+        sc[0][warp] = before;
+        sc[1][warp] = all;
+        sz[warp] = z;
+    }
+    __syncthreads();
+    int off = 0, M = 0;
+    z = 0.0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+        off += sc[0][w];
+        M += sc[1][w];
+        if constexpr (P != 0) z += sz[w];
+    }
+    const float zref = P == 0 || M == 0 ? 0.f : (float)(z / M);
+    if (blockIdx.x == gridDim.x - 1 && tid == 0) {
+        out2[0] = M;
+        out2[1] = __float_as_int(zref);
+        if (host_out2) {      // the host's read-back slot (mapped pinned memory)
+            host_out2[0] = M;
+            host_out2[1] = __float_as_int(zref);
+        }
+    }
+    for (int b = b0; b < b1; ++b) {
+        const int base = b * kPrepPix + warp * (32 * kPixPerThread) + lane;
+        Pixel px[kPixPerThread];
+#pragma unroll
+        for (int k = 0; k < kPixPerThread; ++k) px[k] = load_pixel(depth, normals, mask, base + 32 * k, HW);
+        unsigned bits[kPixPerThread];
+        int c = 0;
+#pragma unroll
+        for (int k = 0; k < kPixPerThread; ++k) {
+            bits[k] = __ballot_sync(0xffffffffu, px[k].ok);
+            c += __popc(bits[k]);
+        }
+        if (lane == 0) sw[warp] = c;
+        __syncthreads();
+        int at = off;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+            const int cw = sw[w];
+            at += w < warp ? cw : 0;
+            off += cw;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kPixPerThread; ++k) {
+            const int pix = base + 32 * k;
+            const bool ok = px[k].ok;
+            const float zz = px[k].z;
+            const float3 nn = px[k].n;
+            if (pix < HW) {
+                // NaN depth where the pixel cannot be a target: no distance gate accepts it
+                if constexpr (P == 0) {
+                    reinterpret_cast<float4*>(tgt_v)[pix] =
+                        ok ? make_float4(zz, nn.x, nn.y, nn.z) : make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
+                } else {
+                    ushort4 t;
+                    t.x = ok ? to16<P>(zz - zref) : nan16<P>();
+                    t.y = ok ? to16<P>(nn.x) : (unsigned short)0;
+                    t.z = ok ? to16<P>(nn.y) : (unsigned short)0;
+                    t.w = ok ? to16<P>(nn.z) : (unsigned short)0;
+                    reinterpret_cast<ushort4*>(tgt_v)[pix] = t;
+                }
             }
+            if (ok) {
+                const int o = at + __popc(bits[k] & ((1u << lane) - 1u));
+                const int u = pix % W, v = pix / W;
+                // pi_D^-1(x): (u - cx) z / fx, (v - cy) z / fy, z
+                const float px_ = ((float)u - cx) * zz * ifx;
+                const float py_ = ((float)v - cy) * zz * ify;
+                if constexpr (P == 0) {
+                    reinterpret_cast<float4*>(src_p_v)[o] = make_float4(px_, py_, zz, 0.f);
+                    reinterpret_cast<float4*>(src_n_v)[o] = make_float4(nn.x, nn.y, nn.z, 0.f);
+                } else {
+                    reinterpret_cast<ushort4*>(src_p_v)[o] =
+                        make_ushort4(to16<P>(px_), to16<P>(py_), to16<P>(zz - zref), 0);
+                    reinterpret_cast<ushort4*>(src_n_v)[o] =
+                        make_ushort4(to16<P>(nn.x), to16<P>(nn.y), to16<P>(nn.z), 0);
+                }
+            }
+            at += __popc(bits[k]);
         }
     }
-    int total;
-    int off = blockoff[blockIdx.x] + block_exclusive_scan(c, &total, sm);
-#pragma unroll
-    for (int k = 0; k < kPixPerThread; ++k) {
-        if (!ok[k]) continue;
-        const int pix = base + k;
-        const int u = pix % W, v = pix / W;
-        const float z = zz[k];
-        // pi_D^-1(x): (u - cx) z / fx, (v - cy) z / fy, z
-        const float px = ((float)u - cx) * z * ifx;
-        const float py = ((float)v - cy) * z * ify;
-        if constexpr (P == 0) {
-            reinterpret_cast<float4*>(src_p_v)[off] = make_float4(px, py, z, 0.f);
-            reinterpret_cast<float4*>(src_n_v)[off] = make_float4(nn[k].x, nn[k].y, nn[k].z, 0.f);
-        } else {
-            reinterpret_cast<ushort4*>(src_p_v)[off] = make_ushort4(to16<P>(px), to16<P>(py), to16<P>(z - zref), 0);
-            reinterpret_cast<ushort4*>(src_n_v)[off] =
-                make_ushort4(to16<P>(nn[k].x), to16<P>(nn[k].y), to16<P>(nn[k].z), 0);
-        }
-        ++off;
-    }
+}
+
+template <int P>
+static void launch_prep_p(const float* depth, const float* normals, const uint8_t* mask, int W, int HW, float cx, float cy,
+                          float ifx, float ify, void* tgt, void* src_p, void* src_n, int* blockcnt, double* blocksum,
+                          int nblk, int* out2, int* host_out2, cudaStream_t s)
+{
+    // at most eight CTAs an SM: each reads every block's count once
+    constexpr int kMaxCtas = 8 * 152;
+    prep_count_kernel<P != 0><<<nblk, kThreads, 0, s>>>(depth, normals, mask, HW, blockcnt, blocksum);
+    prep_write_kernel<P><<<std::min(nblk, kMaxCtas), kThreads, 0, s>>>(depth, normals, mask, W, HW, cx, cy, ifx, ify,
+                                                                       blockcnt, blocksum, nblk, out2, host_out2, tgt,
+                                                                       src_p, src_n);
 }
 
 cudaError_t launch_prep(const float* depth, const float* normals, const uint8_t* mask, int W, int H, float cx,
@@ -233,17 +282,8 @@ cudaError_t launch_prep(const float* depth, const float* normals, const uint8_t*
     int* blockcnt = static_cast<int*>(block_scratch);
     double* blocksum = reinterpret_cast<double*>(
         (reinterpret_cast<uintptr_t>(blockcnt + nblk + 1) + 15) & ~static_cast<uintptr_t>(15));
-    prep_count_kernel<<<nblk, kThreads, 0, s>>>(depth, normals, mask, HW, blockcnt, blocksum);
-    prep_scan_kernel<<<1, 32, 0, s>>>(blockcnt, blocksum, nblk, out2, host_out2);
-    if (precision == 1)
-        prep_write_kernel<1><<<nblk, kThreads, 0, s>>>(depth, normals, mask, W, HW, cx, cy, ifx, ify, blockcnt, out2,
-                                                       tgt, src_p, src_n);
-    else if (precision == 2)
-        prep_write_kernel<2><<<nblk, kThreads, 0, s>>>(depth, normals, mask, W, HW, cx, cy, ifx, ify, blockcnt, out2,
-                                                       tgt, src_p, src_n);
-    else
-        prep_write_kernel<0><<<nblk, kThreads, 0, s>>>(depth, normals, mask, W, HW, cx, cy, ifx, ify, blockcnt, out2,
-                                                       tgt, src_p, src_n);
+    auto run = precision == 1 ? launch_prep_p<1> : precision == 2 ? launch_prep_p<2> : launch_prep_p<0>;
+    run(depth, normals, mask, W, HW, cx, cy, ifx, ify, tgt, src_p, src_n, blockcnt, blocksum, nblk, out2, host_out2, s);
     return cudaGetLastError();
 }
 
