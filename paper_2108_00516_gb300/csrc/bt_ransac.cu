@@ -12,8 +12,9 @@
 //                      then the FP64 fit in quaternion form (Horn 1987: the
 //                      eigenvector of the largest eigenvalue of a symmetric
 //                      4x4 matrix built from the cross-covariance, here by
-//                      cyclic Jacobi rotations), the same optimum as the SVD
-//                      form of Arun et al. 1987.
+//                      single-precision Jacobi rotations corrected from FP64
+//                      residuals), the same optimum as the SVD form of Arun
+//                      et al. 1987.
 //   score_kernel       one warp per (set, sample): the inlier test in IEEE
 //                      single precision with a fixed operation order
 //                      (u = ((R00 px + R01 py) + R02 pz) + tx, each product
@@ -106,6 +107,138 @@ __device__ void top_eigenvector4(double (&A)[4][4], double (&v)[4])
     for (int k = 0; k < 4; ++k) v[k] = V[k][best];
 }
 
+// Single-precision eigenvectors of a symmetric 4x4 matrix (scaled to entries of
+// order one), largest eigenvalue first, by cyclic Jacobi rotations.
+__device__ void eigenvectors4_f32(float (&A)[4][4], float (&V)[4][4])
+{
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) V[r][c] = r == c ? 1.f : 0.f;
+    for (int sweep = 0; sweep < 6; ++sweep) {
+        float off = 0.f;
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+            for (int c = r + 1; c < 4; ++c) off = fmaxf(off, fabsf(A[r][c]));
+        if (!(off > 1e-8f)) break;
+#pragma unroll
+        for (int p = 0; p < 3; ++p) {
+#pragma unroll
+            for (int q = p + 1; q < 4; ++q) {
+                const float apq = A[p][q];
+                if (fabsf(apq) < 1e-12f) continue;
+                const float theta = (A[q][q] - A[p][p]) / (2.f * apq);
+                const float t = copysignf(1.f, theta) / (fabsf(theta) + sqrtf(fmaf(theta, theta, 1.f)));
+                const float c = rsqrtf(fmaf(t, t, 1.f)), s = t * c;
+                A[p][p] = fmaf(-t, apq, A[p][p]);
+                A[q][q] = fmaf(t, apq, A[q][q]);
+                A[p][q] = A[q][p] = 0.f;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if (k != p && k != q) {
+                        const float akp = A[k][p], akq = A[k][q];
+                        A[k][p] = A[p][k] = c * akp - s * akq;
+                        A[k][q] = A[q][k] = s * akp + c * akq;
+                    }
+                    const float vkp = V[k][p], vkq = V[k][q];
+                    V[k][p] = c * vkp - s * vkq;
+                    V[k][q] = s * vkp + c * vkq;
+                }
+            }
+        }
+    }
+    // largest eigenvalue into column 0, then the second largest into column 1
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = i + 1; j < 4; ++j)
+            if (A[j][j] > A[i][i]) {
+                const float t = A[i][i];
+                A[i][i] = A[j][j];
+                A[j][j] = t;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float x = V[k][i];
+                    V[k][i] = V[k][j];
+                    V[k][j] = x;
+                }
+            }
+}
+
+// Largest-eigenvalue eigenvector of a symmetric 4x4 matrix N to FP64 accuracy:
+// single-precision eigenvectors V, then corrections of the first from its FP64
+// residual r = N v - (v.N v) v, v += sum_k V_k (V_k.r) / (lambda - lambda_k),
+// each of which shrinks the error by the single-precision error of V over the
+// gap to the next eigenvalue (about 1e-6: three corrections).  A correction is
+// ~46 FP64 instructions; the all-FP64 Jacobi iteration is ~9000, and on this
+// part a warp-wide FP64 instruction takes 64 cycles of its sub-partition.
+// Returns false, v unset, where the gap is below 2e-6 of the largest entry or
+// the corrections do not settle: the caller then runs the FP64 iteration.
+__device__ bool top_eigenvector4_refined(const double (&N)[4][4], double (&v)[4])
+{
+    float A[4][4], V[4][4], big = 0.f;
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = r; c < 4; ++c) {
+            A[r][c] = (float)N[r][c];
+            big = fmaxf(big, fabsf(A[r][c]));
+        }
+    if (!(big > 1e-30f && big < 1e30f)) return false;
+    const float scale = 1.f / big;
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = r; c < 4; ++c) A[r][c] = A[c][r] = A[r][c] * scale;
+    eigenvectors4_f32(A, V);
+    if (!(A[0][0] - A[1][1] > 2e-6f)) return false;
+    // the second eigenvalue, whose distance from the first may be small, from
+    // its FP64 Rayleigh quotient
+    double l1;
+    {
+        double u[4], num = 0.0, den = 0.0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) u[k] = (double)V[k][1];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            num = fma(u[r], fma(N[r][0], u[0], fma(N[r][1], u[1], fma(N[r][2], u[2], N[r][3] * u[3]))), num);
+            den = fma(u[r], u[r], den);
+        }
+        l1 = num * (2.0 - den);       // den = 1 + O(1e-7)
+    }
+    const float g2 = (A[0][0] - A[2][2]) * big, g3 = (A[0][0] - A[3][3]) * big;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = (double)V[k][0];
+    for (int it = 0; it < 10; ++it) {
+        // |v| = 1 to rounding (one Newton step of the reciprocal square root)
+        const double n2 = fma(v[0], v[0], fma(v[1], v[1], fma(v[2], v[2], v[3] * v[3])));
+        const double f = fma(-0.5, n2, 1.5);
+        double w[4], l = 0.0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] *= f;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            w[r] = fma(N[r][0], v[0], fma(N[r][1], v[1], fma(N[r][2], v[2], N[r][3] * v[3])));
+            l = fma(v[r], w[r], l);
+        }
+        float r4[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) r4[k] = (float)fma(-l, v[k], w[k]);
+        const float g1 = (float)(l - l1);
+        if (!(g1 > 0.f)) return false;
+        const float b1 = (V[0][1] * r4[0] + V[1][1] * r4[1] + V[2][1] * r4[2] + V[3][1] * r4[3]) / g1;
+        const float b2 = (V[0][2] * r4[0] + V[1][2] * r4[1] + V[2][2] * r4[2] + V[3][2] * r4[3]) / g2;
+        const float b3 = (V[0][3] * r4[0] + V[1][3] * r4[1] + V[2][3] * r4[2] + V[3][3] * r4[3]) / g3;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] += (double)(b1 * V[k][1] + b2 * V[k][2] + b3 * V[k][3]);
+        const float step = fmaxf(fabsf(b1), fmaxf(fabsf(b2), fabsf(b3)));
+        if (step < 1e-11f) return true;
+        if (!(step < 0.5f)) return false;
+    }
+    return false;
+}
+
 // Rigid least-squares fit q ~ R p + t from centroids and the cross-covariance
 // S_ab = sum (p - p_c)_a (q - q_c)_b (quaternion form).
 __device__ void fit_from_moments(const double (&S)[3][3], const double (&pc)[3], const double (&qc)[3], double* out)
@@ -118,7 +251,7 @@ __device__ void fit_from_moments(const double (&S)[3][3], const double (&pc)[3],
                       {Szx - Sxz, Sxy + Syx, -Sxx + Syy - Szz, Syz + Szy},
                       {Sxy - Syx, Szx + Sxz, Syz + Szy, -Sxx - Syy + Szz}};
     double v[4];
-    top_eigenvector4(N, v);
+    if (!top_eigenvector4_refined(N, v)) top_eigenvector4(N, v);
     const double nrm = sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2] + v[3] * v[3]);
     const double w = v[0] / nrm, x = v[1] / nrm, y = v[2] / nrm, z = v[3] / nrm;
     const double R[9] = {1.0 - 2.0 * (y * y + z * z), 2.0 * (x * y - w * z), 2.0 * (x * z + w * y),
@@ -130,7 +263,17 @@ __device__ void fit_from_moments(const double (&S)[3][3], const double (&pc)[3],
     for (int r = 0; r < 3; ++r) out[9 + r] = qc[r] - (R[3 * r] * pc[0] + R[3 * r + 1] * pc[1] + R[3 * r + 2] * pc[2]);
 }
 
-__global__ void hypothesis_kernel(const RSet* __restrict__ sets, int H, uint64_t seed, double* __restrict__ hyp,
+// x / 3: the product with the rounded reciprocal, corrected by its exact
+// remainder (a full FP64 division is ~10 times as many instructions).
+__device__ __forceinline__ double third(double x)
+{
+    const double q = x * (1.0 / 3.0);
+    return fma(fma(-3.0, q, x), 1.0 / 3.0, q);
+}
+
+constexpr int kHypThreads = 32;      // one warp a CTA: the FP64 units of all SMs share the samples
+
+__global__ void __launch_bounds__(kHypThreads) hypothesis_kernel(const RSet* __restrict__ sets, int H, uint64_t seed, double* __restrict__ hyp,
                                   int* __restrict__ valid)
 {
     const int s = blockIdx.y, h = blockIdx.x * blockDim.x + threadIdx.x;
@@ -160,14 +303,15 @@ __global__ void hypothesis_kernel(const RSet* __restrict__ sets, int H, uint64_t
     const double ax = p[1][0] - p[0][0], ay = p[1][1] - p[0][1], az = p[1][2] - p[0][2];
     const double bx = p[2][0] - p[0][0], by = p[2][1] - p[0][1], bz = p[2][2] - p[0][2];
     const double cx = ay * bz - az * by, cy = az * bx - ax * bz, cz = ax * by - ay * bx;
-    const double cr = sqrt(cx * cx + cy * cy + cz * cz);
+    const double cr2 = cx * cx + cy * cy + cz * cz;
     const double sc = ax * ax + ay * ay + az * az + bx * bx + by * by + bz * bz;
-    if (!(cr > 1e-12 * (sc > 1e-30 ? sc : 1e-30))) return;
+    const double lim = 1e-12 * (sc > 1e-30 ? sc : 1e-30);
+    if (!(cr2 > lim * lim)) return;
     double pc[3], qc[3], M[3][3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        pc[a] = (p[0][a] + p[1][a] + p[2][a]) / 3.0;
-        qc[a] = (q[0][a] + q[1][a] + q[2][a]) / 3.0;
+        pc[a] = third(p[0][a] + p[1][a] + p[2][a]);
+        qc[a] = third(q[0][a] + q[1][a] + q[2][a]);
     }
 #pragma unroll
     for (int a = 0; a < 3; ++a)
@@ -216,13 +360,23 @@ __global__ void score_kernel(const RSet* __restrict__ sets, int H, const double*
     for (int k = 0; k < 9; ++k) R[k] = (float)hyp[o * kHyp + k];
 #pragma unroll
     for (int k = 0; k < 3; ++k) t[k] = (float)hyp[o * kHyp + 9 + k];
+    // four points a lane at a time, their loads in flight together
     int c = 0;
-    for (int k0 = 0; k0 < S.n; k0 += 32) {
-        const int k = k0 + lane;
-        bool in = false;
-        if (k < S.n) in = inlier(R, t, S.p + 3 * k, S.q + 3 * k, thr2);
-        c += __popc(__ballot_sync(0xffffffffu, in));
+    for (int k0 = lane; k0 < S.n; k0 += 128) {
+        float p[4][3], q[4][3];
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            const int k = min(k0 + 32 * x, S.n - 1);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                p[x][a] = __ldg(S.p + 3 * k + a);
+                q[x][a] = __ldg(S.q + 3 * k + a);
+            }
+        }
+#pragma unroll
+        for (int x = 0; x < 4; ++x) c += k0 + 32 * x < S.n && inlier(R, t, p[x], q[x], thr2);
     }
+    c = __reduce_add_sync(0xffffffffu, c);
     if (lane == 0) count[o] = c;
 }
 
@@ -330,40 +484,53 @@ __global__ void select_kernel(const RSet* __restrict__ sets, int H, const double
     }
 }
 
-struct Scratch {
-    DevBuf sets, hyp, valid, count, out;
-};
-
 int run_ransac(const std::vector<RSet>& sets, int H, uint64_t seed, double delta, int refine, cudaStream_t st,
                std::vector<double>& out)
 {
     const int S = (int)sets.size();
     out.assign(16 * (size_t)S, 0.0);
     if (S == 0) return BT_OK;
-    Scratch sc;
-    auto cleanup = [&]() {
-        for (DevBuf* b : {&sc.sets, &sc.hyp, &sc.valid, &sc.count, &sc.out}) b->release();
+    // one block of the process-wide cache of idle device blocks, given back
+    // when the stream is done with it: a power of two from 64 KiB to 64 MiB,
+    // so that calls of all sizes leave a bounded number of blocks behind.  A
+    // larger one is allocated and freed here.
+    size_t off = 0;
+    auto take = [&off](size_t bytes) {
+        const size_t o = off;
+        off = align_up(o + bytes, 256);
+        return o;
     };
-    cudaError_t e = sc.sets.ensure(sizeof(RSet) * S);
-    if (e == cudaSuccess) e = sc.hyp.ensure(sizeof(double) * kHyp * (size_t)S * H);
-    if (e == cudaSuccess) e = sc.valid.ensure(sizeof(int) * (size_t)S * H);
-    if (e == cudaSuccess) e = sc.count.ensure(sizeof(int) * (size_t)S * H);
-    if (e == cudaSuccess) e = sc.out.ensure(sizeof(double) * 16 * (size_t)S);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(sc.sets.p, sets.data(), sizeof(RSet) * S, cudaMemcpyHostToDevice, st);
+    const size_t o_sets = take(sizeof(RSet) * S), o_hyp = take(sizeof(double) * kHyp * (size_t)S * H),
+                 o_valid = take(sizeof(int) * (size_t)S * H), o_count = take(sizeof(int) * (size_t)S * H),
+                 o_out = take(sizeof(double) * 16 * (size_t)S);
+    size_t cls = 65536;
+    while (cls < off && cls < ((size_t)64 << 20)) cls *= 2;
+    const bool cached = cls >= off;
+    int dev = 0;
+    void* blk = nullptr;
+    BT_CUDA(cudaGetDevice(&dev), "cudaGetDevice");
+    BT_CUDA(cached ? cache_take(cls, &blk) : alloc_should_fail() ? cudaErrorMemoryAllocation : cudaMalloc(&blk, off),
+            "alloc ransac scratch");
+    char* base = static_cast<char*>(blk);
+    RSet* sets_d = reinterpret_cast<RSet*>(base + o_sets);
+    double* hyp = reinterpret_cast<double*>(base + o_hyp);
+    int* valid = reinterpret_cast<int*>(base + o_valid);
+    int* count = reinterpret_cast<int*>(base + o_count);
+    double* out_d = reinterpret_cast<double*>(base + o_out);
+    cudaError_t e = cudaMemcpyAsync(sets_d, sets.data(), sizeof(RSet) * S, cudaMemcpyHostToDevice, st);
     const float thr2 = (float)(delta * delta);
     if (e == cudaSuccess) {
-        hypothesis_kernel<<<dim3((H + 127) / 128, S), 128, 0, st>>>(sc.sets.as<RSet>(), H, seed, sc.hyp.as<double>(),
-                                                                   sc.valid.as<int>());
-        score_kernel<<<dim3((H + 7) / 8, S), 256, 0, st>>>(sc.sets.as<RSet>(), H, sc.hyp.as<double>(),
-                                                          sc.valid.as<int>(), thr2, sc.count.as<int>());
-        select_kernel<<<S, 256, 0, st>>>(sc.sets.as<RSet>(), H, sc.hyp.as<double>(), sc.count.as<int>(), thr2,
-                                         refine, sc.out.as<double>());
+        hypothesis_kernel<<<dim3((H + kHypThreads - 1) / kHypThreads, S), kHypThreads, 0, st>>>(sets_d, H, seed, hyp, valid);
+        score_kernel<<<dim3((H + 7) / 8, S), 256, 0, st>>>(sets_d, H, hyp, valid, thr2, count);
+        select_kernel<<<S, 256, 0, st>>>(sets_d, H, hyp, count, thr2, refine, out_d);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(out.data(), sc.out.p, sizeof(double) * 16 * S, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cleanup();
+        e = cudaMemcpyAsync(out.data(), out_d, sizeof(double) * 16 * S, cudaMemcpyDeviceToHost, st);
+    const cudaError_t done = cudaStreamSynchronize(st);      // also after a failure: the block goes back idle
+    if (e == cudaSuccess) e = done;
+    if (cached) cache_give(dev, cls, blk);
+    else cudaFree(blk);
     if (e != cudaSuccess) return cuda_fail(e, "ransac");
     return BT_OK;
 }
