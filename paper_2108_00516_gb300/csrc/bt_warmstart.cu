@@ -558,124 +558,179 @@ int num_sms()
 }
 
 // ---------------------------------------------------------------------------
-// Backward pass: one CTA per set of the minibatch
+// Backward pass: one CTA per set of the minibatch leaves what the set
+// contributes to the gradient in factored form (a BwdRec of 11.5 KiB), and
+// one launch over the parameters sums the contributions of all sets.  The
+// gradients of layers 2, 3 and 4 are sums of outer products over the sets, so
+// writing them out per set first (264 KiB a set, read back by the sum) cost
+// 71 + 37 us for a minibatch of 256 sets.
 // ---------------------------------------------------------------------------
 
 constexpr int kBwdThreads = 256;
 
 __global__ void __launch_bounds__(kBwdThreads)
     backward_kernel(Net net, const Sample* __restrict__ smp, const int* __restrict__ ids, int n_sets,
-                    const Cache* __restrict__ cache, float inv_n, float* __restrict__ G,
-                    float* __restrict__ loss_per)
+                    Cache* __restrict__ cache, float inv_n, BwdRec* __restrict__ rec)
 {
-    __shared__ float sW1[kH1 * kIn], sB1[kH1];
-    __shared__ float sg[kH2], sdz2[kH2], sdz3[kH3], sh3[kH3], sz3[kH3], sdy[8], sMC[16];
-    __shared__ int sr[kH2];
-    __shared__ float sxr[kH2 * kIn];
-    __shared__ float spart[2][kH1][7];
+    __shared__ float sdz2[kH2], sdz3[kH3], sdy[8], sMC[16];
+    __shared__ float sxr[kH2 * 8];           // features of channel c's row at 8 c
+    __shared__ float spart[kH1][7];
     const int s = blockIdx.x, tid = threadIdx.x;
     const int sid = ids ? ids[s] : s;
     const Sample* S = smp + sid;
     const Cache* C = cache + s;
-    float* Gs = G + (size_t)s * kNumParams;
+    BwdRec& R = rec[s];
     const int n = S->n;
-    if (n <= 0) {
-        for (int k = tid; k < kNumParams; k += kBwdThreads) Gs[k] = 0.f;
-        if (tid == 0) loss_per[s] = 0.f;
+    if (n <= 0) {      // no forward pass: contributes nothing
+        cache[s].g[tid] = 0.f;
+        float* f = reinterpret_cast<float*>(&R);
+        for (int k = tid; k < (int)(sizeof(BwdRec) / sizeof(float)); k += kBwdThreads) f[k] = 0.f;
         return;
     }
-    for (int k = tid; k < kH1 * kIn; k += kBwdThreads) sW1[k] = bf2f(net.wb[bW1 + k]);
-    if (tid < kH1) sB1[tid] = net.master[ob1 + tid];
-    sg[tid] = C->g[tid];
-    sr[tid] = C->r[tid];
-    if (tid < kH3) {
-        sz3[tid] = C->z3[tid];
-        sh3[tid] = fmaxf(C->z3[tid], 0.f);
-    }
+    const float g = C->g[tid];
+    const int row = min(max(C->r[tid], 0), n - 1);
+    const float z3 = tid < kH3 ? C->z3[tid] : 0.f;
     if (tid < 12) sMC[tid] = S->m[tid];
     else if (tid < 15) sMC[tid] = S->c[tid - 12];
-    if (tid < kOut) sdy[tid] = (C->y[tid] - S->ystar[tid]);
+    if (tid < kOut) sdy[tid] = C->y[tid] - S->ystar[tid];
     __syncthreads();
     if (tid == 0) {
         float l = 0.f;
         for (int m = 0; m < kOut; ++m) l = __fmaf_rn(sdy[m], sdy[m], l);
-        loss_per[s] = 0.5f * l * inv_n;
+        R.loss = 0.5f * l * inv_n;
     }
-    __syncthreads();
-    if (tid < kOut) sdy[tid] *= inv_n;
-    __syncthreads();
     // layer 4
-    for (int k = tid; k < kOut * kH3; k += kBwdThreads) Gs[oW4 + k] = sdy[k / kH3] * sh3[k % kH3];
-    if (tid < kOut) Gs[ob4 + tid] = sdy[tid];
+    if (tid < kOut) R.dy[tid] = sdy[tid] * inv_n;
     if (tid < kH3) {
         float a = 0.f;
-        for (int m = 0; m < kOut; ++m) a = __fmaf_rn(bf2f(net.wb[bW4 + m * kH3 + tid]), sdy[m], a);
-        const float d = sz3[tid] > 0.f ? a : 0.f;
+#pragma unroll
+        for (int m = 0; m < kOut; ++m) a = __fmaf_rn(bf2f(net.wb[bW4 + m * kH3 + tid]), sdy[m] * inv_n, a);
+        const float d = z3 > 0.f ? a : 0.f;
         sdz3[tid] = d;
-        Gs[ob3 + tid] = d;
+        R.dz3[tid] = d;
+        R.h3[tid] = fmaxf(z3, 0.f);
+    }
+    float x[6];
+    point_features(S->p, S->q, sMC, sMC + 12, row, x);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        sxr[tid * 8 + k] = x[k];
+        R.x[tid][k] = x[k];
     }
     __syncthreads();
-    // layer 3: dW3 = dz3 g^T, dg = W3^T dz3
-    for (int k = tid; k < kH3 * kH2; k += kBwdThreads) Gs[oW3 + k] = sdz3[k >> 8] * sg[k & 255];
+    // layer 3: dg = W3^T dz3, and ReLU' at the row holding the maximum
     {
         float a = 0.f;
+#pragma unroll 32
         for (int o = 0; o < kH3; ++o) a = __fmaf_rn(bf2f(net.wb[bW3 + o * kH2 + tid]), sdz3[o], a);
-        const float d = sg[tid] > 0.f ? a : 0.f;     // ReLU' at the row holding the maximum
+        const float d = g > 0.f ? a : 0.f;
         sdz2[tid] = d;
-        Gs[ob2 + tid] = d;
-        float x[6];
-        point_features(S->p, S->q, sMC, sMC + 12, sr[tid], x);
-#pragma unroll
-        for (int k = 0; k < 6; ++k) sxr[tid * kIn + k] = x[k];
+        R.x[tid][6] = d;
     }
     __syncthreads();
-    // layer 2: dW2[c][j] = dz2[c] * bf16(relu(z1(row r_c, unit j)))
-    for (int k = tid; k < kH2 * kH1; k += kBwdThreads) {
-        const int c = k >> 7, j = k & 127;
-        const float z = z1_unit(sW1 + j * kIn, sB1[j], sxr + c * kIn);
-        const float h = __bfloat162float(__float2bfloat16_rn(fmaxf(z, 0.f)));
-        Gs[oW2 + k] = sdz2[c] * h;
-    }
     // layer 1: dW1[j][k] = sum_c dz2[c] W2[c][j] [z1(r_c, j) > 0] x(r_c)[k]
-    {
-        const int j = tid & 127, half = tid >> 7;
-        float a[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int c = half * 128; c < half * 128 + 128; ++c) {
-            const float d = sdz2[c];
-            if (d == 0.f) continue;
-            const float z = z1_unit(sW1 + j * kIn, sB1[j], sxr + c * kIn);
-            if (z > 0.f) {
-                const float w = d * bf2f(net.wb[bW2 + c * kH1 + j]);
+    const int j = tid & 127, half = tid >> 7;
+    float w1[6];
 #pragma unroll
-                for (int k = 0; k < 6; ++k) a[k] = __fmaf_rn(w, sxr[c * kIn + k], a[k]);
-                a[6] += w;
-            }
-        }
+    for (int k = 0; k < 6; ++k) w1[k] = bf2f(net.wb[bW1 + j * kIn + k]);
+    const float b1 = net.master[ob1 + j];
+    float a[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 16
+    for (int c = half * 128; c < half * 128 + 128; ++c) {
+        const float4 xa = *reinterpret_cast<const float4*>(sxr + c * 8);
+        const float2 xb = *reinterpret_cast<const float2*>(sxr + c * 8 + 4);
+        const float xc[6] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y};
+        const float w = z1_unit(w1, b1, xc) > 0.f ? sdz2[c] * bf2f(net.wb[bW2 + c * kH1 + j]) : 0.f;
 #pragma unroll
-        for (int k = 0; k < 7; ++k) spart[half][j][k] = a[k];
+        for (int k = 0; k < 6; ++k) a[k] = __fmaf_rn(w, xc[k], a[k]);
+        a[6] += w;
+    }
+    if (half == 1) {
+#pragma unroll
+        for (int k = 0; k < 7; ++k) spart[j][k] = a[k];
     }
     __syncthreads();
-    if (tid < kH1) {
+    if (half == 0) {
 #pragma unroll
-        for (int k = 0; k < 6; ++k) Gs[oW1 + tid * kIn + k] = spart[0][tid][k] + spart[1][tid][k];
-        Gs[ob1 + tid] = spart[0][tid][6] + spart[1][tid][6];
+        for (int k = 0; k < 6; ++k) R.dw1[j * kIn + k] = a[k] + spart[j][k];
+        R.dw1[kH1 * kIn + j] = a[6] + spart[j][6];
     }
 }
 
-__global__ void reduce_kernel(const float* __restrict__ G, const float* __restrict__ loss_per, int n,
-                              float* __restrict__ grad, double* __restrict__ loss)
+// grad = the sum over sets of each parameter's contributions, in a fixed
+// order: four groups of sets side by side in a CTA, then the groups.  CTAs
+// [0, 128): two rows of dW2 each, dW2[c][j] = sum_s dz2[c] bf16(relu(z1(row
+// r_c, unit j))) with the layer-1 output formed again from the row's features;
+// [128, 256): one row of dW3 = sum_s dz3 g^T each; the others 256 of the
+// remaining parameters each.
+constexpr int kSumThreads = 1024, kSumGroups = 4, kSumSets = 128;
+constexpr int kSumW2 = kH2 / 2, kSumW3 = kH3;
+constexpr int kSumRest = kH1 * kIn + kH1 + kH2 + kH3 + kOut * kH3 + kOut;
+constexpr int kSumBlocks = kSumW2 + kSumW3 + (kSumRest + 255) / 256;
+
+__global__ void __launch_bounds__(kSumThreads)
+    gradient_kernel(Net net, const BwdRec* __restrict__ rec, const Cache* __restrict__ cache, int n,
+                    float* __restrict__ grad, double* __restrict__ loss)
 {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < kNumParams) {
-        float a = 0.f;
-        for (int s = 0; s < n; ++s) a += G[(size_t)s * kNumParams + p];
-        grad[p] = a;
+    __shared__ float4 sx[kSumSets][2][2];        // features and dz2 of two channels' rows
+    __shared__ float part[kSumGroups][256];
+    const int tid = threadIdx.x, col = tid & 255, grp = tid >> 8, b = blockIdx.x;
+    float a = 0.f;
+    int p = -1;                                  // the parameter this thread's column sums
+    if (b < kSumW2) {
+        const int j = col & 127, cl = col >> 7;
+        p = oW2 + (2 * b + cl) * kH1 + j;
+        float w1[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) w1[k] = bf2f(net.wb[bW1 + j * kIn + k]);
+        const float b1 = net.master[ob1 + j];
+        for (int s0 = 0; s0 < n; s0 += kSumSets) {
+            const int m = min(kSumSets, n - s0);
+            __syncthreads();
+            if (tid < 4 * m)
+                sx[tid >> 2][(tid >> 1) & 1][tid & 1] =
+                    __ldg(reinterpret_cast<const float4*>(rec[s0 + (tid >> 2)].x[2 * b + ((tid >> 1) & 1)]) + (tid & 1));
+            __syncthreads();
+#pragma unroll 4
+            for (int s = grp; s < m; s += kSumGroups) {
+                const float4 xa = sx[s][cl][0], xb = sx[s][cl][1];
+                const float x[6] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y};
+                const float h = __bfloat162float(__float2bfloat16_rn(fmaxf(z1_unit(w1, b1, x), 0.f)));
+                a = __fmaf_rn(xb.z, h, a);
+            }
+        }
+    } else if (b < kSumW2 + kSumW3) {
+        const int o = b - kSumW2;
+        p = oW3 + o * kH2 + col;
+#pragma unroll 8
+        for (int s = grp; s < n; s += kSumGroups) a = __fmaf_rn(__ldg(&rec[s].dz3[o]), __ldg(&cache[s].g[col]), a);
+    } else {
+        const int q = (b - kSumW2 - kSumW3) * 256 + col;
+        constexpr int e1 = kH1 * kIn, e2 = e1 + kH1, e3 = e2 + kH2, e4 = e3 + kH3, e5 = e4 + kOut * kH3;
+        if (q < kSumRest) {
+            p = q < e1 ? oW1 + q : q < e2 ? ob1 + q - e1 : q < e3 ? ob2 + q - e2 : q < e4 ? ob3 + q - e3
+                : q < e5 ? oW4 + q - e4 : ob4 + q - e5;
+#pragma unroll 8
+            for (int s = grp; s < n; s += kSumGroups) {
+                const BwdRec& R = rec[s];
+                if (q < e2) a += __ldg(R.dw1 + q);                 // dW1, then db1
+                else if (q < e3) a += __ldg(&R.x[q - e2][6]);
+                else if (q < e4) a += __ldg(R.dz3 + q - e3);
+                else if (q < e5) a = __fmaf_rn(__ldg(R.dy + (q - e4) / kH3), __ldg(R.h3 + (q - e4) % kH3), a);
+                else a += __ldg(R.dy + q - e5);
+            }
+        }
+        if (b == kSumBlocks - 1 && tid >= kSumThreads - 32) {
+            double l = 0.0;
+            for (int s = tid & 31; s < n; s += 32) l += (double)__ldg(&rec[s].loss);
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+            if ((tid & 31) == 0) *loss = l;
+        }
     }
-    if (p == 0) {
-        double l = 0.0;
-        for (int s = 0; s < n; ++s) l += (double)loss_per[s];
-        *loss = l;
-    }
+    part[grp][col] = a;
+    __syncthreads();
+    if (grp == 0 && p >= 0) grad[p] = (part[0][col] + part[1][col]) + (part[2][col] + part[3][col]);
 }
 
 __device__ __forceinline__ int bf16_index(int p)
@@ -1132,18 +1187,12 @@ cudaError_t launch_forward(Net net, const Sample* smp, const int* ids, int n, fl
     return cudaGetLastError();
 }
 
-cudaError_t launch_backward(Net net, const Sample* smp, const int* ids, int n, const Cache* cache, float* G,
-                            float* loss_per, cudaStream_t s)
+cudaError_t launch_backward(Net net, const Sample* smp, const int* ids, int n, Cache* cache, BwdRec* rec,
+                            float* grad, double* loss, cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
-    backward_kernel<<<n, kBwdThreads, 0, s>>>(net, smp, ids, n, cache, 1.0f / (float)n, G, loss_per);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_reduce(const float* G, const float* loss_per, int n, float* grad, double* loss,
-                          cudaStream_t s)
-{
-    reduce_kernel<<<(kNumParams + 255) / 256, 256, 0, s>>>(G, loss_per, n, grad, loss);
+    backward_kernel<<<n, kBwdThreads, 0, s>>>(net, smp, ids, n, cache, 1.0f / (float)n, rec);
+    gradient_kernel<<<kSumBlocks, kSumThreads, 0, s>>>(net, rec, cache, n, grad, loss);
     return cudaGetLastError();
 }
 

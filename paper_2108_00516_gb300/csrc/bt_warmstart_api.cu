@@ -32,7 +32,7 @@ struct bt_warmstart {
     int64_t n_points = 0, cap_points = 0;
     int n_samples = 0, cap_samples = 0;
     // launch scratch
-    DevBuf ids, y, cache, G, loss_per, grad, loss;
+    DevBuf ids, y, cache, rec, grad, loss;
     DevBuf app_samples, app_y, app_graphs, app_scratch, app_status, app_items;
     PinBuf pin_app, pin_status;   // staging of the apply tables and the per-graph status
     // fault word of the forward pass (mapped pinned host memory: the kernel
@@ -53,8 +53,8 @@ struct bt_warmstart {
     ~bt_warmstart()
     {
         if (stream) cudaStreamSynchronize(stream);
-        for (DevBuf* b : {&master, &wb, &m, &v, &pool_p, &pool_q, &samples, &stage, &items, &ids, &y, &cache, &G,
-                          &loss_per, &grad, &loss, &app_samples, &app_y, &app_graphs, &app_scratch, &app_status,
+        for (DevBuf* b : {&master, &wb, &m, &v, &pool_p, &pool_q, &samples, &stage, &items, &ids, &y, &cache, &rec,
+                          &grad, &loss, &app_samples, &app_y, &app_graphs, &app_scratch, &app_status,
                           &app_items})
             b->release();
         pin_app.release();
@@ -140,7 +140,7 @@ int upload_ids(bt_warmstart* ws, const int32_t* ids, int n)
     return BT_OK;
 }
 
-// Forward (with cache), backward and reduction over the given samples:
+// Forward (with cache) and backward over the given samples:
 // leaves the mean gradient in ws->grad and the mean loss in ws->loss.
 int gradient_pass(bt_warmstart* ws, const int32_t* ids, int n)
 {
@@ -149,20 +149,16 @@ int gradient_pass(bt_warmstart* ws, const int32_t* ids, int n)
     cudaStream_t s = ws->stream;
     BT_CUDA(ws->y.ensure(sizeof(float) * W::kOut * (size_t)n), "alloc y");
     BT_CUDA(ws->cache.ensure(sizeof(W::Cache) * (size_t)n), "alloc cache");
-    BT_CUDA(ws->G.ensure(sizeof(float) * W::kNumParams * (size_t)n), "alloc per-set gradients");
-    BT_CUDA(ws->loss_per.ensure(sizeof(float) * (size_t)n), "alloc losses");
+    BT_CUDA(ws->rec.ensure(sizeof(W::BwdRec) * (size_t)n), "alloc gradient contributions");
     BT_CUDA(ws->grad.ensure(sizeof(float) * W::kNumParams), "alloc gradient");
     BT_CUDA(ws->loss.ensure(sizeof(double)), "alloc loss");
     const W::Net net = ws->net();
     const W::Sample* smp = ws->samples.as<W::Sample>();
     const int* d_ids = ws->ids.as<int>();
     BT_CUDA(W::launch_forward(net, smp, d_ids, n, ws->y.as<float>(), ws->cache.as<W::Cache>(), s), "launch forward");
-    BT_CUDA(W::launch_backward(net, smp, d_ids, n, ws->cache.as<W::Cache>(), ws->G.as<float>(),
-                               ws->loss_per.as<float>(), s),
+    BT_CUDA(W::launch_backward(net, smp, d_ids, n, ws->cache.as<W::Cache>(), ws->rec.as<W::BwdRec>(),
+                               ws->grad.as<float>(), ws->loss.as<double>(), s),
             "launch backward");
-    BT_CUDA(W::launch_reduce(ws->G.as<float>(), ws->loss_per.as<float>(), n, ws->grad.as<float>(),
-                             ws->loss.as<double>(), s),
-            "launch reduce");
     return BT_OK;
 }
 

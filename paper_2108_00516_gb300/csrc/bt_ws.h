@@ -77,6 +77,15 @@ struct Cache {
     float pad[2];
 };
 
+// What one set contributes to the gradient, in factored form.
+struct __align__(16) BwdRec {
+    float x[kH2][8];            // per channel of layer 2: features of the row holding its maximum, dz2, unused
+    float dz3[kH3], h3[kH3];    // layer 3: gradient of the pre-activations, outputs
+    float dw1[kH1 * kIn + kH1]; // layer 1: gradient of the weights, then of the biases
+    float dy[kOut];
+    float loss, pad;
+};
+
 // One graph of an averaging launch.
 struct AvgGraph {
     int N, n_edges, n_free, pad;
@@ -96,13 +105,10 @@ cudaError_t launch_to_bf16(Net net, cudaStream_t s);
 cudaError_t launch_forward(Net net, const Sample* smp, const int* ids, int n, float* y_out, Cache* cache,
                            cudaStream_t s);
 size_t forward_smem_bytes();
-// Per-set gradients of the mean loss 1/2 |y - y*|^2 into G [n][kNumParams],
-// per-set losses into loss_per [n].
-cudaError_t launch_backward(Net net, const Sample* smp, const int* ids, int n, const Cache* cache, float* G,
-                            float* loss_per, cudaStream_t s);
-// grad = sum over sets of G (fixed order), loss = sum of loss_per (FP64).
-cudaError_t launch_reduce(const float* G, const float* loss_per, int n, float* grad, double* loss,
-                          cudaStream_t s);
+// Gradient of the mean loss 1/2 |y - y*|^2 over n sets (sum over the sets in a
+// fixed order) and the loss (FP64); rec [n] is scratch.
+cudaError_t launch_backward(Net net, const Sample* smp, const int* ids, int n, Cache* cache, BwdRec* rec,
+                            float* grad, double* loss, cudaStream_t s);
 // Adam step: c1 = 1 / (1 - beta1^t), c2 = 1 / (1 - beta2^t).
 cudaError_t launch_adam(Net net, const float* grad, float lr, float beta1, float beta2, float eps, float c1,
                         float c2, cudaStream_t s);

@@ -361,3 +361,21 @@ def test_training_resumes_from_checkpoint(bt):
         c.set_adam(m, -np.abs(v) - 1.0, 5)
     for w in (a, b, c):
         w.close()
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 64, 128, 130, 256, 300])
+def test_gradient_is_the_mean_of_the_sets(bt, n):
+    """The sum over a minibatch, taken in groups of sets, against the mean of
+    the single sets' gradients.  For a power of two the factor 1 / n is exact
+    throughout, so each parameter is off by at most n / 4 + 8 roundings of the
+    sum of magnitudes; else 1 / n rounds ahead of sums that cancel, and the
+    whole gradient is compared, to 168 roundings."""
+    ws = _loaded(bt, _sets(12, [40 + k % 50 for k in range(n)]), _params(12))
+    loss, g = ws.gradient(range(n))
+    one = [ws.gradient([k]) for k in range(n)]
+    G = np.array([x for _, x in one], np.float64)
+    assert abs(loss - np.mean([x for x, _ in one])) <= 1e-6 * loss
+    if n & (n - 1) == 0:
+        assert np.all(np.abs(g - G.mean(0)) <= (n / 4 + 8) * 2.0**-24 * np.abs(G).mean(0) + 1e-30)
+    else:
+        assert np.linalg.norm(g - G.mean(0)) <= 168 * 2.0**-24 * np.linalg.norm(np.abs(G).mean(0))
