@@ -3,21 +3,21 @@
 // reduction, Adam, and the FP64 relative-pose averaging solve that turns the
 // predicted edge increments into node poses for Gauss-Newton (Sec. IV-D).
 //
-// Forward pass: a persistent CTA per SM keeps the BF16 W2 (in the tensor
-// cores' core-matrix layout) and W3 in shared memory and walks its sets in
-// chunks of 128 points.  Layer 1 (K = 6) runs on the FP32 pipes and is
-// rounded to BF16 into one of two shared-memory tiles; the 128 x 256 x 128
+// Forward pass: two persistent CTAs per SM keep the BF16 W2 (in the tensor
+// cores' core-matrix layout) in shared memory and walk equal shares of the
+// chunks of 128 points of all sets.  Layer 1 (K = 6) runs on the FP32 pipes
+// and is rounded to BF16 into a shared-memory tile; the 128 x 256 x 128
 // contraction of layer 2 runs on the fifth-generation tensor cores
 // (tcgen05.mma, BF16 in, FP32 accumulators in tensor memory, issued by one
-// thread, completion signalled on an mbarrier).  While the tensor cores work
-// on chunk c, the CUDA cores compute layer 1 of chunk c+1 into the other
-// tile, and then read chunk c's accumulators (tcgen05.ld) for bias, ReLU and
-// a running per-channel maximum (with the row that holds it, first row on
-// ties); two accumulators in tensor memory let chunk c+1's contraction run
-// during that read-out.  Then the 256 -> 128 -> 6 head.  Every wait on the
-// tensor cores is bounded (globaltimer); a wait that runs out sets the
-// network's fault word, drains the contraction in flight, frees the tensor
-// memory and ends the kernel, and the host reports BT_ERR_TIMEOUT.
+// thread, completion signalled on an mbarrier), while the CUDA cores form the
+// features of the next chunk and the SM's other CTA runs its layer 1 or
+// read-out; then the accumulators are read back (tcgen05.ld) into running
+// per-channel maxima, which are combined over the CTAs of a set with 64-bit
+// atomic maxima (value, then first row).  The 256 -> 128 -> 6 head of all sets
+// is a launch of its own.  Every wait on the tensor cores is bounded
+// (globaltimer); a wait that runs out sets the network's fault word, drains
+// the contraction in flight, frees the tensor memory and ends the kernel, and
+// the host reports BT_ERR_TIMEOUT.
 // Backward pass: only the rows that hold a channel's maximum receive
 // gradient, so layer 1 and layer 2 gradients are outer products over at most
 // 256 rows, recomputed from the inputs with the forward pass's arithmetic.
@@ -27,6 +27,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
+#include <stddef.h>
 #include <stdint.h>
 
 namespace bt {
@@ -58,52 +59,12 @@ __device__ __forceinline__ void features_from(const float v[6], const float* m, 
     x[5] = __fmul_rn(__fsub_rn(qz, uz), kInvSR);
 }
 
-// Point pair k of a set (zeros when k >= n).
-__device__ __forceinline__ void load_pair(const float* __restrict__ p, const float* __restrict__ q, int k, int n,
-                                          float v[6])
-{
-    if (k < n) {
-        v[0] = p[3 * k];
-        v[1] = p[3 * k + 1];
-        v[2] = p[3 * k + 2];
-        v[3] = q[3 * k];
-        v[4] = q[3 * k + 1];
-        v[5] = q[3 * k + 2];
-    } else {
-#pragma unroll
-        for (int e = 0; e < 6; ++e) v[e] = 0.f;
-    }
-}
-
 // Features of point k of a set.
 __device__ __forceinline__ void point_features(const float* __restrict__ p, const float* __restrict__ q,
                                                const float* m, const float* c, int k, float x[6])
 {
-    float v[6];
-    load_pair(p, q, k, k + 1, v);
+    const float v[6] = {p[3 * k], p[3 * k + 1], p[3 * k + 2], q[3 * k], q[3 * k + 1], q[3 * k + 2]};
     features_from(v, m, c, x);
-}
-
-// Offset (floats) of layer-1 unit u's packed weights in the forward kernel's
-// shared memory: 8 floats a unit, each block of 32 units skewed by 16 bytes,
-// so that the four threads of a row, which take the blocks u / 32 = 0..3,
-// read four different bank groups.
-__device__ __forceinline__ int w1_at(int u) { return u * 8 + (u >> 5) * 4; }
-
-// z1_unit with the unit's weights and bias packed as w[0..5], w[6] = bias
-// (two 16-byte shared-memory loads); the same operations in the same order.
-__device__ __forceinline__ float z1_unit8(const float* w8, const float x[6])
-{
-    const float4 a = *reinterpret_cast<const float4*>(w8);
-    const float4 b = *reinterpret_cast<const float4*>(w8 + 4);
-    float z = b.z;
-    z = __fmaf_rn(a.x, x[0], z);
-    z = __fmaf_rn(a.y, x[1], z);
-    z = __fmaf_rn(a.z, x[2], z);
-    z = __fmaf_rn(a.w, x[3], z);
-    z = __fmaf_rn(b.x, x[4], z);
-    z = __fmaf_rn(b.y, x[5], z);
-    return z;
 }
 
 // Layer-1 pre-activation of one unit (weights w[6], bias b), fixed order.
@@ -151,7 +112,7 @@ constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kH2
                             ((uint32_t)(kChunk >> 4) << 24);
 static_assert(kChunk == 128 && kH2 % 16 == 0 && kH2 <= 256, "shape of one kind::f16 contraction (M = 128)");
 
-constexpr int kTmemCols = 2 * kH2;                 // two FP32 [128][256] accumulators
+constexpr int kTmemCols = kH2;                     // one FP32 [128][256] accumulator: two CTAs share an SM's 512 columns
 constexpr long long kTensorWaitNs = 1000000000LL;  // default bound of a wait on the tensor cores (1 s)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p)
@@ -185,11 +146,13 @@ __device__ __forceinline__ void issue_layer2(uint32_t d_tmem, uint32_t a_saddr, 
 }
 
 // Waits until phase `parity` of the mbarrier at `bar` has completed, for at
-// most limit_ns of the global timer; limit_ns <= 0 gives up without polling.
+// most limit_ns of the global timer (read only once the first try, which
+// suspends the thread for a while, has come back without it); limit_ns <= 0
+// gives up without polling.
 __device__ __forceinline__ bool wait_tensor(uint32_t bar, uint32_t parity, long long limit_ns)
 {
     if (limit_ns <= 0) return false;
-    const unsigned long long t0 = global_ns();
+    unsigned long long t0 = 0;
     for (;;) {
         uint32_t done;
         asm volatile(
@@ -199,7 +162,9 @@ __device__ __forceinline__ bool wait_tensor(uint32_t bar, uint32_t parity, long 
             : "r"(bar), "r"(parity)
             : "memory");
         if (done) return true;
-        if ((long long)(global_ns() - t0) > limit_ns) return false;
+        const unsigned long long t = global_ns();
+        if (t0 == 0) t0 = t;
+        if ((long long)(t - t0) > limit_ns) return false;
     }
 }
 
@@ -224,99 +189,146 @@ __device__ __forceinline__ void tmem_load_16x256b_x8(uint32_t taddr, uint32_t (&
         : "memory");
 }
 
-// Layer 1 of one row of a chunk, 64 of the 128 units (half 0 or 1): ReLU,
-// rounded to BF16, written as eight 16-byte core-matrix rows of the tile.
-__device__ __forceinline__ void layer1_half_row(unsigned char* tile, const float* sW1, const float x[6], int row,
-                                                int half)
+// Row stride (floats) of the features of a chunk in shared memory: the 16-byte
+// loads of eight neighbouring rows fall into different banks.
+constexpr int kLdX = 12;
+
+// Layer 1 of a chunk, this thread's share: rows lane + 32 r (r = 0..3), units
+// 16 w .. 16 w + 15 of warp w; ReLU, rounded to BF16, into the core-matrix
+// layout of the tile.  Two units a packed FP32x2 instruction (each half rounds
+// as the scalar one: the backward pass forms the same bits with z1_unit); a
+// pair's weights are one warp-uniform read for four rows.  sW: per unit pair
+// (w0 w0' w1 w1' .. w5 w5' b b'), 16 floats.
+__device__ __forceinline__ void layer1_rows(unsigned char* tile, const float* sW, const float* sX, int warp, int lane)
 {
-    unsigned char* dst = tile + core_off(row, half * 64);
+    float2 x[4][6];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        uint32_t w[4];
+    for (int r = 0; r < 4; ++r) {
+        const float* xr = sX + (lane + 32 * r) * kLdX;
+        const float4 a = *reinterpret_cast<const float4*>(xr);
+        const float2 b = *reinterpret_cast<const float2*>(xr + 4);
+        x[r][0] = make_float2(a.x, a.x);
+        x[r][1] = make_float2(a.y, a.y);
+        x[r][2] = make_float2(a.z, a.z);
+        x[r][3] = make_float2(a.w, a.w);
+        x[r][4] = make_float2(b.x, b.x);
+        x[r][5] = make_float2(b.y, b.y);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {      // eight units: one 16-byte core-matrix row of each of the four rows
+        uint32_t o[4][4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const int u = half * 64 + 8 * j + 2 * e;
-            const float h0 = fmaxf(z1_unit8(sW1 + w1_at(u), x), 0.f);
-            const float h1 = fmaxf(z1_unit8(sW1 + w1_at(u + 1), x), 0.f);
-            __nv_bfloat162 b = __floats2bfloat162_rn(h0, h1);
-            w[e] = *reinterpret_cast<uint32_t*>(&b);
+            const float4* w4 = reinterpret_cast<const float4*>(sW + (8 * warp + 4 * h + e) * 16);
+            const float4 w01 = w4[0], w23 = w4[1], w45 = w4[2], bb = w4[3];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                float2 z = __ffma2_rn(make_float2(w01.x, w01.y), x[r][0], make_float2(bb.x, bb.y));
+                z = __ffma2_rn(make_float2(w01.z, w01.w), x[r][1], z);
+                z = __ffma2_rn(make_float2(w23.x, w23.y), x[r][2], z);
+                z = __ffma2_rn(make_float2(w23.z, w23.w), x[r][3], z);
+                z = __ffma2_rn(make_float2(w45.x, w45.y), x[r][4], z);
+                z = __ffma2_rn(make_float2(w45.z, w45.w), x[r][5], z);
+                __nv_bfloat162 b = __floats2bfloat162_rn(fmaxf(z.x, 0.f), fmaxf(z.y, 0.f));
+                o[r][e] = *reinterpret_cast<uint32_t*>(&b);
+            }
         }
-        *reinterpret_cast<uint4*>(dst + j * kCoreK) = make_uint4(w[0], w[1], w[2], w[3]);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            *reinterpret_cast<uint4*>(tile + core_off(lane + 32 * r, 16 * warp + 8 * h)) =
+                make_uint4(o[r][0], o[r][1], o[r][2], o[r][3]);
     }
 }
+
+__device__ __forceinline__ int set_chunks(int n) { return n > kChunk ? (n + kChunk - 1) / kChunk : 1; }
 
 // Shared-memory layout of the forward kernel (byte offsets).
 struct Fwd {
     static constexpr size_t W2 = 0;                                          // bf16 [256][128], core_off layout
-    static constexpr size_t H1 = W2 + 2 * (size_t)kH2 * kH1;                 // 2 x bf16 [128][128], core_off layout
-    static constexpr size_t W3 = H1 + 2 * (size_t)kH1TileBytes;              // bf16 [128][kLd3]
-    static constexpr size_t W1 = W3 + ((2 * (size_t)kH3 * kLd3 + 15) / 16) * 16;   // float [128][8] + skew (w1_at)
-    static constexpr size_t B2 = W1 + 4 * ((size_t)kH1 * 8 + 16);            // float [256]
-    static constexpr size_t B3 = B2 + 4 * (size_t)kH2;                       // float [128]
-    static constexpr size_t W4 = B3 + 4 * (size_t)kH3;                       // float [6][128]
-    static constexpr size_t B4 = W4 + 4 * (size_t)kOut * kH3;                // float [8]
-    static constexpr size_t G = B4 + 32;                                     // float [256]
-    static constexpr size_t R = G + 4 * (size_t)kH2;                         // int [256]
-    static constexpr size_t RV = R + 4 * (size_t)kH2;                        // float [4][256]
-    static constexpr size_t RI = RV + 16 * (size_t)kH2;                      // int [4][256]
-    static constexpr size_t H3 = RI + 16 * (size_t)kH2;                      // float [128]
-    static constexpr size_t Z3 = H3 + 4 * (size_t)kH3;                       // float [128]
-    static constexpr size_t MC = Z3 + 4 * (size_t)kH3;                       // float [16]: m[12], c[3]
-    static constexpr size_t BAR = MC + 64;                                   // two mbarriers (u64)
+    static constexpr size_t H1 = W2 + 2 * (size_t)kH2 * kH1;                 // bf16 [128][128], core_off layout
+    static constexpr size_t W1 = H1 + (size_t)kH1TileBytes;                  // float [64][16]: unit pairs (layer1_rows)
+    static constexpr size_t B2 = W1 + 4 * (size_t)kH1 * 8;                   // float [256]
+    static constexpr size_t X = B2 + 4 * (size_t)kH2;                        // float [128][kLdX]
+    static constexpr size_t SMP = X + 4 * (size_t)kChunk * kLdX;             // four Samples
+    static constexpr size_t SCAN = SMP + 4 * 128;                            // int [8 + 2]
+    static constexpr size_t BAR = SCAN + 48;                                 // mbarrier (u64)
     static constexpr size_t TM = BAR + 16;                                   // tensor-memory base address
     static constexpr size_t Total = TM + 16;
 };
-static_assert(Fwd::H1 % 16 == 0 && Fwd::W3 % 16 == 0 && Fwd::W1 % 16 == 0 && Fwd::BAR % 8 == 0, "alignment");
-static_assert(Fwd::Total <= 227 * 1024, "shared memory of one CTA");
-static_assert(Fwd::Total > 114 * 1024, "one CTA per SM: the two accumulators take all of its tensor memory");
-static_assert(kFwdThreads == 2 * kH3 && kFwdThreads == kH2, "head mapping: two threads per layer-3 unit");
-static_assert(kFwdThreads == 2 * kChunk, "layer 1: two threads per row of a chunk");
+static_assert(sizeof(Sample) <= 128 && offsetof(Sample, c) + 12 <= 128, "a set's description is one 128-byte read of a warp");
+static_assert(Fwd::H1 % 16 == 0 && Fwd::W1 % 16 == 0 && Fwd::X % 16 == 0 && Fwd::SMP % 16 == 0 && Fwd::BAR % 8 == 0,
+              "alignment");
+static_assert(2 * (Fwd::Total + 1024) <= 228 * 1024, "two CTAs per SM");
+static_assert(2 * kTmemCols <= 512, "two CTAs per SM");
+static_assert(kFwdThreads == kH2 && kFwdThreads == 2 * kChunk, "thread mappings");
 
+// The forward pass up to the max-pool.  pool[s][256]: running maximum of each
+// channel, (float bits of relu(max z + b2)) << 32 | ~row (row 0xffffffff where
+// it is not kept), zero on entry.  The chunks of all sets, in order, are
+// divided evenly over the CTAs, wherever the sets begin and end.
 template <bool kTrain>
-__global__ void __launch_bounds__(kFwdThreads, 1)
+__global__ void __launch_bounds__(kFwdThreads, kTrain ? 1 : 2)
     forward_kernel(Net net, const Sample* __restrict__ smp, const int* __restrict__ ids, int n_sets,
-                   float* __restrict__ y_out, Cache* __restrict__ cache)
+                   unsigned long long* __restrict__ pool)
 {
     extern __shared__ __align__(1024) unsigned char sm[];
-    __nv_bfloat16* sW3 = reinterpret_cast<__nv_bfloat16*>(sm + Fwd::W3);    // layer 3: [unit][kLd3]
-    float* sW1 = reinterpret_cast<float*>(sm + Fwd::W1);     // unit u at w1_at(u): weights [0..5], bias [6]
+    float* sW1 = reinterpret_cast<float*>(sm + Fwd::W1);
     float* sB2 = reinterpret_cast<float*>(sm + Fwd::B2);
-    float* sB3 = reinterpret_cast<float*>(sm + Fwd::B3);
-    float* sW4 = reinterpret_cast<float*>(sm + Fwd::W4);
-    float* sB4 = reinterpret_cast<float*>(sm + Fwd::B4);
-    float* sG = reinterpret_cast<float*>(sm + Fwd::G);
-    int* sR = reinterpret_cast<int*>(sm + Fwd::R);
-    float* sRV = reinterpret_cast<float*>(sm + Fwd::RV);
-    int* sRI = reinterpret_cast<int*>(sm + Fwd::RI);
-    float* sH3 = reinterpret_cast<float*>(sm + Fwd::H3);
-    float* sZ3 = reinterpret_cast<float*>(sm + Fwd::Z3);
-    float* sMC = reinterpret_cast<float*>(sm + Fwd::MC);
-
+    float* sX = reinterpret_cast<float*>(sm + Fwd::X);
+    int* sScan = reinterpret_cast<int*>(sm + Fwd::SCAN);
+    auto sample = [&](int set) { return reinterpret_cast<const Sample*>(sm + Fwd::SMP + 128 * (set & 3)); };
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+
+    // this CTA's share of the chunks: each thread adds up a run of sets, the
+    // thread whose run holds the first chunk finds its set
+    auto id_of = [&](int s) { return ids ? __ldg(ids + s) : s; };
+    const int r0 = (int)((long long)tid * n_sets / kFwdThreads), r1 = (int)((long long)(tid + 1) * n_sets / kFwdThreads);
+    int mine = 0;
+    for (int s = r0; s < r1; ++s) mine += set_chunks(__ldg(&smp[id_of(s)].n));
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) sScan[warp] = incl;
+    __syncthreads();
+    int total = 0, before = 0;
+#pragma unroll
+    for (int w = 0; w < kFwdThreads / 32; ++w) {
+        before += w < warp ? sScan[w] : 0;
+        total += sScan[w];
+    }
+    before += incl - mine;
+    const int x0 = (int)((long long)blockIdx.x * total / gridDim.x);
+    const int x1 = (int)((long long)(blockIdx.x + 1) * total / gridDim.x);
+    if (x0 >= x1) return;
+    if (before <= x0 && x0 < before + mine) {
+        int s = r0, at = before;
+        for (;; ++s) {
+            const int k = set_chunks(__ldg(&smp[id_of(s)].n));
+            if (x0 < at + k) break;
+            at += k;
+        }
+        sScan[8] = s;
+        sScan[9] = x0 - at;
+    }
+
     // stage the weights once per CTA; W2 as 16-byte core-matrix rows
     for (int k = tid; k < kH2 * kH1 / 8; k += kFwdThreads) {
         const int row = k >> 4, k8 = (k & 15) * 8;
         *reinterpret_cast<uint4*>(sm + Fwd::W2 + core_off(row, k8)) =
             *reinterpret_cast<const uint4*>(net.wb + bW2 + row * kH1 + k8);
     }
-    for (int k = tid; k < kH3 * kH2 / 2; k += kFwdThreads) {   // bf16 pairs, rows padded to kLd3
-        const int o = k / (kH2 / 2), c2 = (k % (kH2 / 2)) * 2;
-        *reinterpret_cast<uint32_t*>(sW3 + o * kLd3 + c2) =
-            *reinterpret_cast<const uint32_t*>(net.wb + bW3 + o * kH2 + c2);
-    }
     for (int k = tid; k < kH1 * 8; k += kFwdThreads) {
-        const int u = k >> 3, e = k & 7;
-        sW1[w1_at(u) + e] = e < kIn ? bf2f(net.wb[bW1 + u * kIn + e]) : (e == kIn ? net.master[ob1 + u] : 0.f);
+        const int u = 2 * (k >> 4) + (k & 1), e = (k & 15) >> 1;
+        sW1[k] = e < kIn ? bf2f(net.wb[bW1 + u * kIn + e]) : (e == kIn ? net.master[ob1 + u] : 0.f);
     }
-    for (int k = tid; k < kOut * kH3; k += kFwdThreads) sW4[k] = bf2f(net.wb[bW4 + k]);
-    for (int k = tid; k < kH2; k += kFwdThreads) sB2[k] = net.master[ob2 + k];
-    for (int k = tid; k < kH3; k += kFwdThreads) sB3[k] = net.master[ob3 + k];
-    if (tid < kOut) sB4[tid] = net.master[ob4 + tid];
+    sB2[tid] = net.master[ob2 + tid];
 
-    const uint32_t bar0 = smem_u32(sm + Fwd::BAR);    // mbarrier of accumulator b at bar0 + 8 b
+    const uint32_t bar = smem_u32(sm + Fwd::BAR);
     if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0) : "memory");
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0 + 8) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
@@ -325,7 +337,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    // the tensor cores read W2 and the layer-1 tiles through the async proxy
+    // the tensor cores read W2 and the layer-1 tile through the async proxy
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     tc_fence_before();
     __syncthreads();
@@ -333,191 +345,194 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(sm + Fwd::TM);
     const uint32_t w2_s = smem_u32(sm + Fwd::W2), h1_s = smem_u32(sm + Fwd::H1);
     unsigned char* const h1_tile = sm + Fwd::H1;
+    int s = sScan[8], c = sScan[9];          // the set and the chunk of it at hand
+
+    // a set's description (its Sample) goes to one of four slots, by warp 4:
+    // the first three here, each other one two sets ahead of its turn
+    auto desc_word = [&](int set) {
+        return lane < (int)(sizeof(Sample) / 4) ? __ldg(reinterpret_cast<const unsigned*>(smp + id_of(set)) + lane) : 0u;
+    };
+    auto desc_put = [&](int set, unsigned w) { reinterpret_cast<unsigned*>(sm + Fwd::SMP + 128 * (set & 3))[lane] = w; };
+    if (warp == 4)
+        for (int q = s; q < min(s + 3, n_sets); ++q) desc_put(q, desc_word(q));
+    __syncthreads();
+    // the point pair of this thread's row of chunk ch of set st (warps 0-3; zeros past the last point)
+    auto load_points = [&](int st, int ch, float (&v)[6]) {
+        const Sample* S = sample(st);
+        const int k = ch * kChunk + tid;
+        const bool in = k < S->n;
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+            v[e] = in ? __ldg(S->p + 3 * (size_t)k + e) : 0.f;
+            v[3 + e] = in ? __ldg(S->q + 3 * (size_t)k + e) : 0.f;
+        }
+    };
+    // its features, zeros past the last point
+    auto features = [&](int st, int ch, const float (&v)[6]) {
+        const Sample* S = sample(st);
+        float x[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if (ch * kChunk + tid < S->n) features_from(v, S->m, S->c, x);
+        float* xr = sX + tid * kLdX;
+        *reinterpret_cast<float4*>(xr) = make_float4(x[0], x[1], x[2], x[3]);
+        *reinterpret_cast<float2*>(xr + 4) = make_float2(x[4], x[5]);
+    };
+    // points are loaded a chunk before their features are formed, so that
+    // their latency passes behind a whole chunk's work: (fs, fc) is the chunk
+    // whose points are in pq
+    float pq[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    int fs = s, fc = c;
+    auto advance = [&]() {
+        if (fc + 1 < set_chunks(sample(fs)->n)) {
+            ++fc;
+        } else {
+            ++fs;
+            fc = 0;
+        }
+    };
+    if (tid < kChunk) {
+        load_points(fs, fc, pq);
+        features(fs, fc, pq);
+        advance();
+        if (x0 + 1 < x1) load_points(fs, fc, pq);
+    }
+    __syncthreads();
 
     // read-out: warp w takes the tensor-memory lanes (rows of a chunk)
     // 32 (w % 4) .. + 31 and the columns 128 (w / 4) .. + 127; a lane holds
     // 32 of those columns (idx: column 128 cw + 8 (idx / 2) + 2 (lane % 4) + idx % 2)
     const int qr = warp & 3, cw = warp >> 2;
-    float b2[32];
-#pragma unroll
-    for (int k = 0; k < 32; ++k) b2[k] = sB2[128 * cw + 8 * (k >> 1) + 2 * (lane & 3) + (k & 1)];
-    const int lrow = tid >> 1, lhalf = tid & 1;   // layer 1: thread = (row of the chunk, half of the 128 units)
-    uint32_t cc = 0;                              // chunks this CTA has contracted so far
-    bool fault = false;
-    for (int s = blockIdx.x; s < n_sets; s += gridDim.x) {
-        const int sid = ids ? ids[s] : s;
-        const Sample* S = smp + sid;
-        const int n = S->n;
-        if (tid < 12) sMC[tid] = S->m[tid];
-        else if (tid < 15) sMC[tid] = S->c[tid - 12];
-        __syncthreads();      // weights staged (first set), sMC ready, previous set's head done
-        if (n <= 0) {         // empty set: no prediction
-            if (tid < kOut) y_out[(size_t)s * kOut + tid] = 0.f;
-            continue;
-        }
-        const float* P = S->p;
-        const float* Q = S->q;
-        // running maxima of the thread's 32 columns (ReLU outputs are >= 0);
-        // training also keeps the row that holds each (first row on ties)
-        float best[32];
-        int bestr[32];
+    // running maxima of the thread's 32 columns; training keeps relu(z + b)
+    // and the row that holds it (first row on ties), inference the largest z:
+    // adding the bias and the ReLU are monotonic, so they follow the maximum
+    float best[32];
+    int bestr[kTrain ? 32 : 1];
+    auto reset = [&]() {
 #pragma unroll
         for (int k = 0; k < 32; ++k) {
-            best[k] = kTrain ? -1.f : 0.f;
-            bestr[k] = 0;
+            best[k] = kTrain ? -1.f : -INFINITY;
+            if constexpr (kTrain) bestr[k] = 0;
         }
-        const int nch = (n + kChunk - 1) / kChunk;
-        float pq[6];                             // the point pair of this thread's row of a chunk
-        load_pair(P, Q, lrow, n, pq);
-        {
-            float x[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            if (lrow < n) features_from(pq, sMC, sMC + 12, x);
-            layer1_half_row(h1_tile + (cc & 1) * kH1TileBytes, sW1, x, lrow, lhalf);
-        }
-        load_pair(P, Q, kChunk + lrow, n, pq);   // in flight during the first contraction
+    };
+    reset();
+    bool fault = false;
+    bool fresh = true;                       // the first chunk of this CTA of its set
+    for (int x = x0; x < x1; ++x) {
+        const int n = sample(s)->n, nch = set_chunks(n);
+        const bool last = c + 1 == nch;      // the last chunk of its set
+        const bool more = x + 1 < x1;
+        unsigned w = 0;
+        const bool fetch = fresh && warp == 4 && s + 2 < n_sets;
+        if (fetch) w = desc_word(s + 2);
+        fresh = false;
+        layer1_rows(h1_tile, sW1, sX, warp, lane);
+        if (fetch) desc_put(s + 2, w);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         tc_fence_before();
         __syncthreads();
         tc_fence_after();
-        if (tid == 0) issue_layer2(tmem + (cc & 1) * kH2, h1_s + (cc & 1) * kH1TileBytes, w2_s, bar0 + 8 * (cc & 1));
-        for (int c = 0; c < nch; ++c, ++cc) {
-            const uint32_t b = cc & 1;
-            if (c + 1 < nch) {   // layer 1 of the next chunk while the tensor cores work on this one
-                const int gr = (c + 1) * kChunk + lrow;
-                float x[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                if (gr < n) features_from(pq, sMC, sMC + 12, x);
-                layer1_half_row(h1_tile + (b ^ 1) * kH1TileBytes, sW1, x, lrow, lhalf);
-                load_pair(P, Q, (c + 2) * kChunk + lrow, n, pq);
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            }
-            const bool done = wait_tensor(bar0 + 8 * b, (cc >> 1) & 1, net.wait_ns);
-            tc_fence_before();
-            if (__syncthreads_or(!done)) {
-                // give the contraction in flight time to finish before the
-                // tensor memory is freed, then end the kernel
-                wait_tensor(bar0 + 8 * b, (cc >> 1) & 1, kTensorWaitNs);
-                fault = true;
-                break;
-            }
-            tc_fence_after();
-            if (c + 1 < nch && tid == 0)
-                issue_layer2(tmem + (b ^ 1) * kH2, h1_s + (b ^ 1) * kH1TileBytes, w2_s, bar0 + 8 * (b ^ 1));
-            // bias, ReLU and the running maximum of chunk c; rows in increasing order
-            const uint32_t tacc = tmem + b * kH2 + 128 * cw;
+        if (tid == 0) issue_layer2(tmem, h1_s, w2_s, bar);
+        // the next chunk's features while the tensor cores work on this one,
+        // and the loads of the one after it
+        if (more && tid < kChunk) {
+            features(fs, fc, pq);
+            advance();
+            if (x + 2 < x1) load_points(fs, fc, pq);
+        }
+        const uint32_t parity = (uint32_t)(x - x0) & 1u;
+        const bool done = wait_tensor(bar, parity, net.wait_ns);
+        tc_fence_before();
+        if (__syncthreads_or(!done)) {
+            // give the contraction in flight time to finish before the
+            // tensor memory is freed, then end the kernel
+            wait_tensor(bar, parity, kTensorWaitNs);
+            fault = true;
+            break;
+        }
+        tc_fence_after();
+        // the running maximum over the rows of the chunk, in increasing order
+        const uint32_t tacc = tmem + 128 * cw;
 #pragma unroll
-            for (int lh = 0; lh < 2; ++lh) {
-                const int rb = c * kChunk + 32 * qr + 16 * lh;
-                if (rb >= n) break;   // the same for the whole warp
-                const int ra = rb + (lane >> 2), rc = ra + 8;
-                const bool va = ra < n, vc = rc < n;
+        for (int lh = 0; lh < 2; ++lh) {
+            const int rb = c * kChunk + 32 * qr + 16 * lh;
+            if (rb >= n) break;   // the same for the whole warp
+            const int ra = rb + (lane >> 2), rc = ra + 8;
+            const bool va = ra < n, vc = rc < n;
 #pragma unroll
-                for (int cq = 0; cq < 2; ++cq) {
-                    uint32_t v[32];
-                    tmem_load_16x256b_x8(tacc + ((uint32_t)(32 * qr + 16 * lh) << 16) + 64 * cq, v);
+            for (int cq = 0; cq < 2; ++cq) {
+                uint32_t v[32];
+                tmem_load_16x256b_x8(tacc + ((uint32_t)(32 * qr + 16 * lh) << 16) + 64 * cq, v);
 #pragma unroll
-                    for (int g = 0; g < 8; ++g)
+                for (int g = 0; g < 8; ++g)
 #pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const int k = 2 * (8 * cq + g) + e;
-                            if constexpr (kTrain) {
-                                const float za = fmaxf(__uint_as_float(v[4 * g + e]) + b2[k], 0.f);
-                                if (va && za > best[k]) {
-                                    best[k] = za;
-                                    bestr[k] = ra;
-                                }
-                                const float zc = fmaxf(__uint_as_float(v[4 * g + 2 + e]) + b2[k], 0.f);
-                                if (vc && zc > best[k]) {
-                                    best[k] = zc;
-                                    bestr[k] = rc;
-                                }
-                            } else {   // max(0, max_rows z) = max_rows relu(z): one maximum an element
-                                if (va) best[k] = fmaxf(best[k], __uint_as_float(v[4 * g + e]) + b2[k]);
-                                if (vc) best[k] = fmaxf(best[k], __uint_as_float(v[4 * g + 2 + e]) + b2[k]);
+                    for (int e = 0; e < 2; ++e) {
+                        const int k = 2 * (8 * cq + g) + e;
+                        if constexpr (kTrain) {
+                            const float b2 = sB2[128 * cw + 8 * (k >> 1) + 2 * (lane & 3) + (k & 1)];
+                            const float za = fmaxf(__uint_as_float(v[4 * g + e]) + b2, 0.f);
+                            if (va && za > best[k]) {
+                                best[k] = za;
+                                bestr[k] = ra;
                             }
+                            const float zc = fmaxf(__uint_as_float(v[4 * g + 2 + e]) + b2, 0.f);
+                            if (vc && zc > best[k]) {
+                                best[k] = zc;
+                                bestr[k] = rc;
+                            }
+                        } else {
+                            if (va) best[k] = fmaxf(best[k], __uint_as_float(v[4 * g + e]));
+                            if (vc) best[k] = fmaxf(best[k], __uint_as_float(v[4 * g + 2 + e]));
                         }
-                }
-            }
-            tc_fence_before();
-        }
-        if (fault) break;
-        // combine the 8 lanes of each column, then the four row quarters
-#pragma unroll
-        for (int k = 0; k < 32; ++k) {
-            float v = best[k];
-            int r = bestr[k];
-#pragma unroll
-            for (int off = 4; off < 32; off <<= 1) {
-                const float ov = __shfl_xor_sync(0xffffffffu, v, off);
-                if constexpr (kTrain) {
-                    const int orr = __shfl_xor_sync(0xffffffffu, r, off);
-                    if (ov > v || (ov == v && orr < r)) {
-                        v = ov;
-                        r = orr;
                     }
-                } else {
-                    v = fmaxf(v, ov);
-                }
-            }
-            if (lane < 4) {
-                const int col = 128 * cw + 8 * (k >> 1) + 2 * lane + (k & 1);
-                sRV[qr * kH2 + col] = v;
-                if (kTrain) sRI[qr * kH2 + col] = r;
             }
         }
-        __syncthreads();
-        {
-            float v = sRV[tid];
-            int r = kTrain ? sRI[tid] : 0;
+        tc_fence_before();
+        if (last || !more) {
+            // combine the 8 lanes of each column by recursive halving: lane l
+            // ends with the columns idx0 .. idx0 + 3, idx0 = its bits 4, 3, 2
+            int idx0 = 0;
 #pragma unroll
-            for (int q = 1; q < 4; ++q) {
-                const float v1 = sRV[q * kH2 + tid];
-                if constexpr (kTrain) {
-                    const int r1 = sRI[q * kH2 + tid];
-                    if (v1 > v || (v1 == v && r1 < r)) {
-                        v = v1;
-                        r = r1;
+            for (int st = 0; st < 3; ++st) {
+                const int off = 16 >> st, half = 16 >> st;
+                const bool upper = (lane & off) != 0;
+#pragma unroll
+                for (int k = 0; k < half; ++k) {
+                    const float send = upper ? best[k] : best[k + half];
+                    float keep = upper ? best[k + half] : best[k];
+                    const float got = __shfl_xor_sync(0xffffffffu, send, off);
+                    if constexpr (kTrain) {
+                        const int rsend = upper ? bestr[k] : bestr[k + half];
+                        int rkeep = upper ? bestr[k + half] : bestr[k];
+                        const int rgot = __shfl_xor_sync(0xffffffffu, rsend, off);
+                        if (got > keep || (got == keep && rgot < rkeep)) {
+                            keep = got;
+                            rkeep = rgot;
+                        }
+                        bestr[k] = rkeep;
+                    } else {
+                        keep = fmaxf(keep, got);
                     }
-                } else {
-                    v = fmaxf(v, v1);
+                    best[k] = keep;
                 }
+                idx0 += upper ? half : 0;
             }
-            sG[tid] = v;
-            sR[tid] = r;
-        }
-        __syncthreads();
-        {   // head layer 3: unit tid % 128, input half tid / 128; the odd row
-            // stride kLd3 / 2 words puts the 32 units of a warp in 32 banks
-            const int o = tid & (kH3 - 1), half = tid >> 7;
-            const __nv_bfloat16* w = sW3 + o * kLd3 + half * 128;
-            const float* g = sG + half * 128;
-            float a = 0.f;
-#pragma unroll 8
-            for (int k = 0; k < 128; ++k) a = __fmaf_rn(bf2f(w[k]), g[k], a);
-            sRV[tid] = a;      // the max-pool scratch is free again
-        }
-        __syncthreads();
-        if (tid < kH3) {
-            const float z = sB3[tid] + (sRV[tid] + sRV[kH3 + tid]);
-            sZ3[tid] = z;
-            sH3[tid] = fmaxf(z, 0.f);
-        }
-        __syncthreads();
-        if (warp < kOut) {   // head layer 4: one warp per output
-            float a = 0.f;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a = __fmaf_rn(sW4[warp * kH3 + lane + 32 * i], sH3[lane + 32 * i], a);
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
-            const float y = sB4[warp] + a;
-            if (lane == 0) {
-                y_out[(size_t)s * kOut + warp] = y;
-                if (kTrain) cache[s].y[warp] = y;
+            for (int k = 0; k < 4; ++k) {
+                const int idx = idx0 + k;
+                const int col = 128 * cw + 8 * (idx >> 1) + 2 * (lane & 3) + (idx & 1);
+                const float g = kTrain ? best[k] : fmaxf(best[k] + sB2[col], 0.f);
+                const unsigned row = kTrain ? ~(unsigned)bestr[k] : 0u;
+                if (g > 0.f || (kTrain && g == 0.f))
+                    atomicMax(pool + (size_t)s * kH2 + col,
+                              ((unsigned long long)__float_as_uint(g) << 32) | row);
             }
+            reset();
         }
-        if (kTrain) {
-            cache[s].g[tid] = sG[tid];
-            cache[s].r[tid] = sR[tid];
-            if (tid < kH3) cache[s].z3[tid] = sZ3[tid];
+        if (last) {
+            ++s;
+            c = 0;
+            fresh = true;
+        } else {
+            ++c;
         }
     }
     if (fault && tid == 0) {
@@ -533,6 +548,101 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
     }
 }
 
+// The 256 -> 128 -> 6 head of kHeadSets sets a CTA: W3 is staged once (rows
+// padded to an odd word stride) and each of its values read once for all of
+// them.
+constexpr int kHeadSets = 8;
+struct Head {
+    static constexpr size_t W3 = 0;                                                   // bf16 [128][kLd3]
+    static constexpr size_t G = W3 + ((2 * (size_t)kH3 * kLd3 + 15) / 16) * 16;       // float [256][kHeadSets]
+    static constexpr size_t P = G + 4 * (size_t)kH2 * kHeadSets;                      // float [2][kHeadSets][128]
+    static constexpr size_t Total = P + 8 * (size_t)kHeadSets * kH3;
+};
+
+template <bool kTrain>
+__global__ void __launch_bounds__(kFwdThreads)
+    head_kernel(Net net, const Sample* __restrict__ smp, const int* __restrict__ ids, int n_sets,
+                const unsigned long long* __restrict__ pool, float* __restrict__ y_out, Cache* __restrict__ cache)
+{
+    extern __shared__ __align__(1024) unsigned char sm[];
+    __nv_bfloat16* sW3 = reinterpret_cast<__nv_bfloat16*>(sm + Head::W3);
+    float* sG = reinterpret_cast<float*>(sm + Head::G);
+    float* sP = reinterpret_cast<float*>(sm + Head::P);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int s0 = blockIdx.x * kHeadSets, m = min(kHeadSets, n_sets - s0);
+#pragma unroll 16
+    for (int k = tid; k < kH3 * kH2 / 2; k += kFwdThreads) {   // bf16 pairs, rows padded to kLd3
+        const int o = k / (kH2 / 2), c2 = (k % (kH2 / 2)) * 2;
+        *reinterpret_cast<uint32_t*>(sW3 + o * kLd3 + c2) =
+            *reinterpret_cast<const uint32_t*>(net.wb + bW3 + o * kH2 + c2);
+    }
+#pragma unroll
+    for (int q = 0; q < kHeadSets; ++q) {
+        const unsigned long long v = q < m ? __ldcg(pool + (size_t)(s0 + q) * kH2 + tid) : 0ull;
+        const float g = __uint_as_float((unsigned)(v >> 32));
+        sG[tid * kHeadSets + q] = g;
+        if (kTrain && q < m) {
+            cache[s0 + q].g[tid] = g;
+            cache[s0 + q].r[tid] = (int)~(unsigned)v;
+        }
+    }
+    __syncthreads();
+    {   // layer 3: unit tid % 128, input half tid / 128; the odd row stride
+        // kLd3 / 2 words puts the 32 units of a warp in 32 banks
+        const int o = tid & (kH3 - 1), half = tid >> 7;
+        const __nv_bfloat16* w = sW3 + o * kLd3 + half * 128;
+        float a[kHeadSets];
+#pragma unroll
+        for (int q = 0; q < kHeadSets; ++q) a[q] = 0.f;
+#pragma unroll 4
+        for (int k = 0; k < 128; ++k) {
+            const float wk = bf2f(w[k]);
+            const float4* g = reinterpret_cast<const float4*>(sG + (half * 128 + k) * kHeadSets);
+#pragma unroll
+            for (int q = 0; q < kHeadSets / 4; ++q) {
+                const float4 g4 = g[q];
+                a[4 * q] = __fmaf_rn(wk, g4.x, a[4 * q]);
+                a[4 * q + 1] = __fmaf_rn(wk, g4.y, a[4 * q + 1]);
+                a[4 * q + 2] = __fmaf_rn(wk, g4.z, a[4 * q + 2]);
+                a[4 * q + 3] = __fmaf_rn(wk, g4.w, a[4 * q + 3]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < kHeadSets; ++q) sP[(half * kHeadSets + q) * kH3 + o] = a[q];
+    }
+    __syncthreads();
+    if (tid < kH3) {
+        const float b3 = net.master[ob3 + tid];
+#pragma unroll
+        for (int q = 0; q < kHeadSets; ++q) {
+            const float z = b3 + (sP[q * kH3 + tid] + sP[(kHeadSets + q) * kH3 + tid]);
+            if (kTrain && q < m) cache[s0 + q].z3[tid] = z;
+            sP[q * kH3 + tid] = fmaxf(z, 0.f);
+        }
+    }
+    __syncthreads();
+    // layer 4: one warp per set, then its outputs in turn
+    static_assert(kFwdThreads / 32 == kHeadSets, "one warp per set");
+    if (warp < m) {
+        const int s = s0 + warp;
+        const bool empty = __ldg(&smp[ids ? __ldg(ids + s) : s].n) <= 0;       // no prediction
+#pragma unroll
+        for (int k = 0; k < kOut; ++k) {
+            float a = 0.f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                a = __fmaf_rn(bf2f(net.wb[bW4 + k * kH3 + lane + 32 * i]), sP[warp * kH3 + lane + 32 * i], a);
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+            const float y = empty ? 0.f : net.master[ob4 + k] + a;
+            if (lane == 0) {
+                y_out[(size_t)s * kOut + k] = y;
+                if (kTrain) cache[s].y[k] = y;
+            }
+        }
+    }
+}
+
 template <bool kTrain>
 struct ForwardAttr {
     static void set()
@@ -540,6 +650,7 @@ struct ForwardAttr {
         static const bool done = [] {      // once per process, thread-safe
             cudaFuncSetAttribute(forward_kernel<kTrain>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)Fwd::Total);
+            cudaFuncSetAttribute(head_kernel<kTrain>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Head::Total);
             return true;
         }();
         (void)done;
@@ -1172,19 +1283,25 @@ cudaError_t launch_to_bf16(Net net, cudaStream_t s)
 
 size_t forward_smem_bytes() { return Fwd::Total; }
 
-cudaError_t launch_forward(Net net, const Sample* smp, const int* ids, int n, float* y_out, Cache* cache,
-                           cudaStream_t s)
+template <bool kTrain>
+static cudaError_t launch_forward_t(Net net, const Sample* smp, const int* ids, int n, unsigned long long* pool,
+                                    float* y_out, Cache* cache, cudaStream_t s)
+{
+    ForwardAttr<kTrain>::set();
+    const cudaError_t e = cudaMemsetAsync(pool, 0, pool_bytes(n), s);
+    if (e != cudaSuccess) return e;
+    forward_kernel<kTrain><<<(kTrain ? 1 : 2) * num_sms(), kFwdThreads, Fwd::Total, s>>>(net, smp, ids, n, pool);
+    head_kernel<kTrain><<<(n + kHeadSets - 1) / kHeadSets, kFwdThreads, Head::Total, s>>>(net, smp, ids, n, pool, y_out,
+                                                                                         cache);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_forward(Net net, const Sample* smp, const int* ids, int n, unsigned long long* pool, float* y_out,
+                           Cache* cache, cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
-    const int grid = n < num_sms() ? n : num_sms();
-    if (cache) {
-        ForwardAttr<true>::set();
-        forward_kernel<true><<<grid, kFwdThreads, Fwd::Total, s>>>(net, smp, ids, n, y_out, cache);
-    } else {
-        ForwardAttr<false>::set();
-        forward_kernel<false><<<grid, kFwdThreads, Fwd::Total, s>>>(net, smp, ids, n, y_out, nullptr);
-    }
-    return cudaGetLastError();
+    return cache ? launch_forward_t<true>(net, smp, ids, n, pool, y_out, cache, s)
+                 : launch_forward_t<false>(net, smp, ids, n, pool, y_out, nullptr, s);
 }
 
 cudaError_t launch_backward(Net net, const Sample* smp, const int* ids, int n, Cache* cache, BwdRec* rec,

@@ -32,8 +32,8 @@ struct bt_warmstart {
     int64_t n_points = 0, cap_points = 0;
     int n_samples = 0, cap_samples = 0;
     // launch scratch
-    DevBuf ids, y, cache, rec, grad, loss;
-    DevBuf app_samples, app_y, app_graphs, app_scratch, app_status, app_items;
+    DevBuf ids, y, maxima, cache, rec, grad, loss;
+    DevBuf app_samples, app_y, app_maxima, app_graphs, app_scratch, app_status, app_items;
     PinBuf pin_app, pin_status;   // staging of the apply tables and the per-graph status
     // fault word of the forward pass (mapped pinned host memory: the kernel
     // writes it, the host reads it after the call's synchronisation)
@@ -53,8 +53,8 @@ struct bt_warmstart {
     ~bt_warmstart()
     {
         if (stream) cudaStreamSynchronize(stream);
-        for (DevBuf* b : {&master, &wb, &m, &v, &pool_p, &pool_q, &samples, &stage, &items, &ids, &y, &cache, &rec,
-                          &grad, &loss, &app_samples, &app_y, &app_graphs, &app_scratch, &app_status,
+        for (DevBuf* b : {&master, &wb, &m, &v, &pool_p, &pool_q, &samples, &stage, &items, &ids, &y, &maxima, &cache, &rec,
+                          &grad, &loss, &app_samples, &app_y, &app_maxima, &app_graphs, &app_scratch, &app_status,
                           &app_items})
             b->release();
         pin_app.release();
@@ -148,6 +148,7 @@ int gradient_pass(bt_warmstart* ws, const int32_t* ids, int n)
     if (st != BT_OK) return st;
     cudaStream_t s = ws->stream;
     BT_CUDA(ws->y.ensure(sizeof(float) * W::kOut * (size_t)n), "alloc y");
+    BT_CUDA(ws->maxima.ensure(W::pool_bytes(n)), "alloc pooled features");
     BT_CUDA(ws->cache.ensure(sizeof(W::Cache) * (size_t)n), "alloc cache");
     BT_CUDA(ws->rec.ensure(sizeof(W::BwdRec) * (size_t)n), "alloc gradient contributions");
     BT_CUDA(ws->grad.ensure(sizeof(float) * W::kNumParams), "alloc gradient");
@@ -155,7 +156,9 @@ int gradient_pass(bt_warmstart* ws, const int32_t* ids, int n)
     const W::Net net = ws->net();
     const W::Sample* smp = ws->samples.as<W::Sample>();
     const int* d_ids = ws->ids.as<int>();
-    BT_CUDA(W::launch_forward(net, smp, d_ids, n, ws->y.as<float>(), ws->cache.as<W::Cache>(), s), "launch forward");
+    BT_CUDA(W::launch_forward(net, smp, d_ids, n, ws->maxima.as<unsigned long long>(), ws->y.as<float>(),
+                              ws->cache.as<W::Cache>(), s),
+            "launch forward");
     BT_CUDA(W::launch_backward(net, smp, d_ids, n, ws->cache.as<W::Cache>(), ws->rec.as<W::BwdRec>(),
                                ws->grad.as<float>(), ws->loss.as<double>(), s),
             "launch backward");
@@ -224,6 +227,7 @@ int enqueue_apply(bt_warmstart* ws, bt_graph* const* gs, int n_graphs, double* c
     BT_CUDA(ws->app_samples.ensure(sizeof(W::Sample) * (size_t)std::max(S, 1)), "alloc samples");
     BT_CUDA(ws->app_items.ensure(sizeof(W::PrepItem) * (size_t)std::max(S, 1)), "alloc items");
     BT_CUDA(ws->app_y.ensure(sizeof(float) * W::kOut * (size_t)std::max(S, 1)), "alloc outputs");
+    BT_CUDA(ws->app_maxima.ensure(W::pool_bytes(std::max(S, 1))), "alloc pooled features");
     BT_CUDA(ws->app_scratch.ensure(sizeof(double) * W::kAvgScratch * (size_t)std::max(S, 1)), "alloc scratch");
     BT_CUDA(ws->app_graphs.ensure(sizeof(W::AvgGraph) * (size_t)n_graphs), "alloc graphs");
     BT_CUDA(ws->app_status.ensure(sizeof(int) * (size_t)n_graphs), "alloc status");
@@ -273,7 +277,9 @@ int launch_apply(bt_warmstart* ws, int S, int n_graphs, int max_free, cudaStream
 {
     W::Sample* d_smp = ws->app_samples.as<W::Sample>();
     BT_CUDA(W::launch_prep(d_smp, ws->app_items.as<W::PrepItem>(), S, s), "launch prep");
-    BT_CUDA(W::launch_forward(ws->net(), d_smp, nullptr, S, ws->app_y.as<float>(), nullptr, s), "launch forward");
+    BT_CUDA(W::launch_forward(ws->net(), d_smp, nullptr, S, ws->app_maxima.as<unsigned long long>(), ws->app_y.as<float>(),
+                              nullptr, s),
+            "launch forward");
     BT_CUDA(W::launch_average(ws->app_graphs.as<W::AvgGraph>(), n_graphs, max_free, s), "launch average");
     return BT_OK;
 }
@@ -590,8 +596,9 @@ int bt_warmstart_predict(bt_warmstart* ws, const int32_t* ids, int32_t n, float*
     st = upload_ids(ws, ids, n);
     if (st != BT_OK) return st;
     BT_CUDA(ws->y.ensure(sizeof(float) * W::kOut * (size_t)n), "alloc y");
-    BT_CUDA(W::launch_forward(ws->net(), ws->samples.as<W::Sample>(), ws->ids.as<int>(), n, ws->y.as<float>(),
-                              nullptr, ws->stream),
+    BT_CUDA(ws->maxima.ensure(W::pool_bytes(n)), "alloc pooled features");
+    BT_CUDA(W::launch_forward(ws->net(), ws->samples.as<W::Sample>(), ws->ids.as<int>(), n,
+                              ws->maxima.as<unsigned long long>(), ws->y.as<float>(), nullptr, ws->stream),
             "launch forward");
     BT_CUDA(cudaMemcpyAsync(y_out, ws->y.p, sizeof(float) * W::kOut * (size_t)n, cudaMemcpyDeviceToHost, ws->stream),
             "read outputs");

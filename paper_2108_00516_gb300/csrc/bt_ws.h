@@ -101,9 +101,10 @@ struct AvgGraph {
 cudaError_t launch_prep(Sample* smp, const PrepItem* items, int n, cudaStream_t s);
 cudaError_t launch_to_bf16(Net net, cudaStream_t s);
 // Forward over sets ids[0..n) (ids may be null: sets 0..n); y_out [n][6];
-// cache (training) [n] or null.
-cudaError_t launch_forward(Net net, const Sample* smp, const int* ids, int n, float* y_out, Cache* cache,
-                           cudaStream_t s);
+// cache (training) [n] or null; pool: scratch of pool_bytes(n).
+inline size_t pool_bytes(int n) { return sizeof(unsigned long long) * kH2 * (size_t)n; }
+cudaError_t launch_forward(Net net, const Sample* smp, const int* ids, int n, unsigned long long* pool, float* y_out,
+                           Cache* cache, cudaStream_t s);
 size_t forward_smem_bytes();
 // Gradient of the mean loss 1/2 |y - y*|^2 over n sets (sum over the sets in a
 // fixed order) and the loss (FP64); rec [n] is scratch.

@@ -363,6 +363,20 @@ def test_training_resumes_from_checkpoint(bt):
         w.close()
 
 
+@pytest.mark.parametrize("sizes", [[1], [20000], [128, 129, 5000, 1, 255, 3], [5] * 700])
+def test_forward_does_not_depend_on_the_split(bt, sizes):
+    """The chunks of all sets are divided over the CTAs wherever the sets
+    begin: a set's output has the same bits alone, among the others, and in a
+    launch that repeats it."""
+    ws = _loaded(bt, _sets(11, sizes), _params(11))
+    ids = list(range(len(sizes)))
+    y = ws.predict(ids)
+    assert np.isfinite(y).all()
+    for k in {0, len(ids) // 2, len(ids) - 1}:
+        assert np.array_equal(ws.predict([k]), y[k:k + 1])
+    assert np.array_equal(ws.predict(ids[::-1] + ids), np.concatenate([y[::-1], y]))
+
+
 @pytest.mark.parametrize("n", [1, 2, 3, 64, 128, 130, 256, 300])
 def test_gradient_is_the_mean_of_the_sets(bt, n):
     """The sum over a minibatch, taken in groups of sets, against the mean of
