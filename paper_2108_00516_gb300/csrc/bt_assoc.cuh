@@ -58,12 +58,15 @@ __device__ __forceinline__ float rcp_approx(float x)
     return r;
 }
 
-// q = M p and the nearest pixel (iu, iv) of its projection.  True when
-// q_z > 1e-30 m and the pixel lies in the image.  Above 1e-30 the
-// reciprocal of q_z is finite, so the projected coordinates are finite and
-// their floor converts exactly or saturates to a value out of range.
+// q = M p and the nearest pixel (iu, iv) of its projection, also as the floats
+// uv.  True when q_z > 1e-30 m and the pixel lies in the image.  The floor is
+// one addition of 1.5 * 2^23 rounded down: the sum's low bits are the integer,
+// and taking the constant off again gives it as a float (exact), without the
+// two conversions each way that go through the quarter-rate pipe.  That holds
+// for coordinates below 2^22 in magnitude; the bits of a larger, infinite or
+// NaN sum differ from the constant's by more than any image side (< 2^15).
 __device__ __forceinline__ bool assoc_project(const PairK& k, float px, float py, float pz, float2& qxy, float& qz,
-                                              int& iu, int& iv)
+                                              float2& uvf, int& iu, int& iv)
 {
     qxy = __ffma2_rn(k.c0, make_float2(px, px), k.c3);
     qxy = __ffma2_rn(k.c1, make_float2(py, py), qxy);
@@ -71,17 +74,21 @@ __device__ __forceinline__ bool assoc_project(const PairK& k, float px, float py
     qz = fmaf(k.m22, pz, fmaf(k.m21, py, fmaf(k.m20, px, k.m23)));
     const float rz = rcp_approx(qz);
     const float2 uv = __ffma2_rn(__fmul2_rn(qxy, k.f), make_float2(rz, rz), k.ch);
-    iu = __float2int_rd(uv.x);
-    iv = __float2int_rd(uv.y);
+    constexpr float kRound = 12582912.0f;
+    const float2 b = __fadd2_rd(uv, make_float2(kRound, kRound));
+    iu = __float_as_int(b.x) - 0x4B400000;
+    iv = __float_as_int(b.y) - 0x4B400000;
+    uvf = __fadd2_rn(b, make_float2(-kRound, -kRound));
     return qz > 1e-30f && (unsigned)iu < (unsigned)k.W && (unsigned)iv < (unsigned)k.H;
 }
 
-// Distance gate against the looked-up target pixel (iu, iv) with depth tz > 0:
-// t = pi_D^-1(iu, iv) in camera j, d = t - q; true when |d|^2 <= dmax2.
-__device__ __forceinline__ bool assoc_distance(const PairK& k, int iu, int iv, float tz, float2 qxy, float qz,
+// Distance gate against the looked-up target pixel uv with depth tz > 0:
+// t = pi_D^-1(uv) in camera j, d = t - q; true when |d|^2 <= dmax2 (never for
+// a NaN depth).
+__device__ __forceinline__ bool assoc_distance(const PairK& k, float2 uv, float tz, float2 qxy, float qz,
                                                float dmax2, float2& txy, float2& dxy, float& dz)
 {
-    txy = __fmul2_rn(__ffma2_rn(make_float2((float)iu, (float)iv), k.ifc, k.cif), make_float2(tz, tz));
+    txy = __fmul2_rn(__ffma2_rn(uv, k.ifc, k.cif), make_float2(tz, tz));
     dxy = __ffma2_rn(qxy, make_float2(-1.f, -1.f), txy);
     dz = tz - qz;
     return fmaf(dz, dz, fmaf(dxy.y, dxy.y, dxy.x * dxy.x)) <= dmax2;

@@ -99,16 +99,16 @@ __global__ void __launch_bounds__(kNoAllocThreads) pair_energy_kernel(
         // pi_D^-1(x) as the frame preparation of the graph path computes it
         const float px = ((float)u - src.cx) * z * src.ifx;
         const float py = ((float)v - src.cy) * z * src.ify;
-        float2 qxy;
+        float2 qxy, uv;
         float qz;
         int iu, iv;
-        if (!bt::assoc_project(K, px, py, z, qxy, qz, iu, iv)) continue;
+        if (!bt::assoc_project(K, px, py, z, qxy, qz, uv, iu, iv)) continue;
         const int tp = iv * dst.W + iu;
         float tz, tnx, tny, tnz;
         if (!valid_px(dst, tp, tz, tnx, tny, tnz)) continue;
         float2 txy, dxy, nxy;
         float dz, nzr;
-        if (!bt::assoc_distance(K, iu, iv, tz, qxy, qz, dmax2, txy, dxy, dz)) continue;
+        if (!bt::assoc_distance(K, uv, tz, qxy, qz, dmax2, txy, dxy, dz)) continue;
         if (!bt::assoc_normal(K, nx, ny, nz, tnx, tny, tnz, cmin, nxy, nzr)) continue;
         const float r = bt::assoc_residual(nxy, nzr, dxy, dz);
         const float ar = fabsf(r);

@@ -298,23 +298,58 @@ struct PairConst {
     float zref;                          // target frame's reference depth (16-bit maps)
 };
 
-__device__ __forceinline__ void fill_pair_const(const SolveArgs& a, int i, int j, PairConst& c)
+__device__ __forceinline__ void fill_pair_const(const SolveArgs& a, int i, int j, const NodeDev& Nj, PairConst& c)
 {
-    const NodeDev Nj = a.nodes[j];
-    c.k = make_pair_k(a.xf + (size_t)(i * a.N + j) * 12, Nj.fx, Nj.fy, Nj.cx, Nj.cy, Nj.ifx, Nj.ify, Nj.W, Nj.H);
+    float m[12];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const float4 v = *(reinterpret_cast<const float4*>(a.xf + (size_t)(i * a.N + j) * 12) + q);
+        m[4 * q] = v.x;
+        m[4 * q + 1] = v.y;
+        m[4 * q + 2] = v.z;
+        m[4 * q + 3] = v.w;
+    }
+    c.k = make_pair_k(m, Nj.fx, Nj.fy, Nj.cx, Nj.cy, Nj.ifx, Nj.ify, Nj.W, Nj.H);
     c.tgt = Nj.tgt;
     c.zref = Nj.zref;
 }
 
-// Target-map gather: (z, nx, ny, nz) as FP32 whatever the storage.
+// One entry of a target map as it is stored (z, nx, ny, nz), and its decoding
+// to FP32.  The gather is predicated: where `ok` is false the depth is NaN,
+// which no distance gate accepts, and the other values are whatever they were.
 template <int P>
-__device__ __forceinline__ float4 load_target(const void* tgt, size_t idx, float zref)
+struct Texel {
+    float4 v;
+};
+template <>
+struct Texel<1> {
+    uint2 v;
+};
+template <>
+struct Texel<2> {
+    uint2 v;
+};
+
+template <int P>
+__device__ __forceinline__ void gather_target(Texel<P>& t, const void* tgt, int idx, bool ok)
 {
     if constexpr (P == 0) {
-        return __ldg(reinterpret_cast<const float4*>(tgt) + idx);
+        t.v.x = __int_as_float(0x7fc00000);
+        if (ok) t.v = __ldg(reinterpret_cast<const float4*>(tgt) + idx);
     } else {
-        const ushort4 v = __ldg(reinterpret_cast<const ushort4*>(tgt) + idx);
-        return make_float4(zref + from16<P>(v.x), from16<P>(v.y), from16<P>(v.z), from16<P>(v.w));
+        t.v.x = nan16<P>();
+        if (ok) t.v = __ldg(reinterpret_cast<const uint2*>(tgt) + idx);
+    }
+}
+
+template <int P>
+__device__ __forceinline__ float4 decode_target(const Texel<P>& t, float zref)
+{
+    if constexpr (P == 0) {
+        return t.v;
+    } else {
+        return make_float4(zref + from16<P>((unsigned short)(t.v.x & 0xffffu)), from16<P>((unsigned short)(t.v.x >> 16)),
+                           from16<P>((unsigned short)(t.v.y & 0xffffu)), from16<P>((unsigned short)(t.v.y >> 16)));
     }
 }
 
@@ -356,173 +391,213 @@ size_t residual_smem_bytes(int N, int shape)
            sizeof(float) * (size_t)nt * (kShapeThreads[shape] / 32) * kDenseVals;
 }
 
-// acc[0..20] += w J J^T (upper triangle, row-major), acc[21..26] += w J r,
-// acc[27] += rho, acc[28] += 1, two entries per packed FP32x2 FMA: rows
-// (0,1), (2,3), (4,5) of one column share the broadcast J_b.
-__device__ __forceinline__ void accumulate_pair(float (&acc)[kDenseVals], float2 J01, float2 J23, float2 J45, float w,
-                                                float r, float rho)
+// The 21 + 6 + 2 sums of a lane as register pairs: entries of J J^T that a
+// packed FP32x2 instruction forms from pairs of J and their swapped copies,
+// (J0, J1) (J2, J3) (J4, J5), without a broadcast per entry.
+struct Sums {
+    float2 p[13];               // (00,11) (02,13) (03,12) (04,15) (05,14) (22,33) (24,35) (25,34) (44,55) g01 g23 g45 (rho, 1)
+    float s01, s23, s45;
+};
+
+__device__ __forceinline__ void accumulate_pair(Sums& a, float2 J01, float2 J23, float2 J45, float w, float r, float rho)
 {
-    const float2 ww = make_float2(w, w);
+    const float2 ww = make_float2(w, w), rr = make_float2(r, r);
+    const float2 J32 = make_float2(J23.y, J23.x), J54 = make_float2(J45.y, J45.x);
     const float2 w01 = __fmul2_rn(J01, ww), w23 = __fmul2_rn(J23, ww), w45 = __fmul2_rn(J45, ww);
-    const float J[6] = {J01.x, J01.y, J23.x, J23.y, J45.x, J45.y};
-    auto f2 = [&](int lo, int hi, float2 a, float b) {
-        const float2 s = __ffma2_rn(a, make_float2(b, b), make_float2(acc[lo], acc[hi]));
-        acc[lo] = s.x;
-        acc[hi] = s.y;
-    };
-    // upper-triangle index of (a, b), b >= a: (0,b) = b, (1,b) = 5 + b,
-    // (2,b) = 9 + b, (3,b) = 12 + b, (4,b) = 14 + b, (5,5) = 20
-    acc[0] = fmaf(w01.x, J[0], acc[0]);
-#pragma unroll
-    for (int b = 1; b < 6; ++b) f2(b, 5 + b, w01, J[b]);
-    acc[11] = fmaf(w23.x, J[2], acc[11]);
-#pragma unroll
-    for (int b = 3; b < 6; ++b) f2(9 + b, 12 + b, w23, J[b]);
-    acc[18] = fmaf(w45.x, J[4], acc[18]);
-    f2(19, 20, w45, J[5]);
-    f2(21, 22, w01, r);
-    f2(23, 24, w23, r);
-    f2(25, 26, w45, r);
-    const float2 s = __fadd2_rn(make_float2(acc[27], acc[28]), make_float2(rho, 1.f));
-    acc[27] = s.x;
-    acc[28] = s.y;
+    a.p[0] = __ffma2_rn(w01, J01, a.p[0]);
+    a.p[1] = __ffma2_rn(w01, J23, a.p[1]);
+    a.p[2] = __ffma2_rn(w01, J32, a.p[2]);
+    a.p[3] = __ffma2_rn(w01, J45, a.p[3]);
+    a.p[4] = __ffma2_rn(w01, J54, a.p[4]);
+    a.p[5] = __ffma2_rn(w23, J23, a.p[5]);
+    a.p[6] = __ffma2_rn(w23, J45, a.p[6]);
+    a.p[7] = __ffma2_rn(w23, J54, a.p[7]);
+    a.p[8] = __ffma2_rn(w45, J45, a.p[8]);
+    a.p[9] = __ffma2_rn(w01, rr, a.p[9]);
+    a.p[10] = __ffma2_rn(w23, rr, a.p[10]);
+    a.p[11] = __ffma2_rn(w45, rr, a.p[11]);
+    a.p[12] = __fadd2_rn(a.p[12], make_float2(rho, 1.f));
+    a.s01 = fmaf(w01.x, J01.y, a.s01);
+    a.s23 = fmaf(w23.x, J23.y, a.s23);
+    a.s45 = fmaf(w45.x, J45.y, a.s45);
 }
 
-// Pixels per thread whose target gathers are issued together, and resident
-// threads per SM the residual kernels are compiled for, by storage precision
-// (FP32: six 128-thread CTAs, at most 80 registers a thread; 16-bit: five).
-#ifndef BT_RES_BATCH_F32
-#define BT_RES_BATCH_F32 2
-#endif
-#ifndef BT_RES_THREADS_F32
-#define BT_RES_THREADS_F32 768
-#endif
-constexpr int residual_batch(int P) { return P == 0 ? BT_RES_BATCH_F32 : 4; }
-constexpr int residual_threads_per_sm(int P) { return P == 0 ? BT_RES_THREADS_F32 : 640; }
-// The FP32 cost-only pass (no Jacobian, two sums a pixel) fits in 64
-// registers without spills: 1024 resident threads a SM, more warps to hide
-// the gathers (the 16-bit decodes would spill there).
-constexpr int residual_threads_per_sm(int P, bool full) { return full || P != 0 ? residual_threads_per_sm(P) : 1024; }
+// The sums in the order of dpart: the upper triangle row-major ((0,b) = b,
+// (1,b) = 5 + b, (2,b) = 9 + b, (3,b) = 12 + b, (4,b) = 14 + b, (5,5) = 20),
+// [21..26] gradient, [27] cost, [28] count.
+__device__ __forceinline__ void ordered_sums(const Sums& a, float (&v)[kDenseVals])
+{
+    v[0] = a.p[0].x;   v[6] = a.p[0].y;
+    v[2] = a.p[1].x;   v[8] = a.p[1].y;
+    v[3] = a.p[2].x;   v[7] = a.p[2].y;
+    v[4] = a.p[3].x;   v[10] = a.p[3].y;
+    v[5] = a.p[4].x;   v[9] = a.p[4].y;
+    v[11] = a.p[5].x;  v[15] = a.p[5].y;
+    v[13] = a.p[6].x;  v[17] = a.p[6].y;
+    v[14] = a.p[7].x;  v[16] = a.p[7].y;
+    v[18] = a.p[8].x;  v[20] = a.p[8].y;
+    v[21] = a.p[9].x;  v[22] = a.p[9].y;
+    v[23] = a.p[10].x; v[24] = a.p[10].y;
+    v[25] = a.p[11].x; v[26] = a.p[11].y;
+    v[27] = a.p[12].x; v[28] = a.p[12].y;
+    v[1] = a.s01;
+    v[12] = a.s23;
+    v[19] = a.s45;
+    v[29] = v[30] = v[31] = 0.f;
+}
+
+// Pixels per lane and step, and resident threads per SM the residual kernels
+// are compiled for.  The full pass keeps two steps in flight and 29 sums a
+// lane (128 registers, 16 warps a SM); the cost-only pass keeps two sums, so
+// it hides its gathers with four pixels a step and 24 warps instead.
+// Measured on 20 VGA views (44.4 M pixel pairs; full / cost pass, cold): one
+// step at a time, a branch per gate and 24 warps 273 / 176 us; this form
+// 216 / 161 us, 108 instead of 141 instructions a pixel pair.  Two steps in
+// flight at 20 and 24 warps (96 and 80 registers: spills) gain nothing
+// (217 us) or lose (300 us); nor does a tile divided over two CTAs (245 us:
+// its sources are staged twice).
+constexpr int step_pix(bool full) { return full ? 2 : 4; }
+constexpr bool residual_pipelined(bool full) { return full; }
+constexpr int residual_threads_per_sm(bool full) { return full ? 512 : 768; }
+
+// One step of a warp in flight: its lanes' pixels after projection, with
+// their target gathers issued.
+template <int P, int kN>
+struct Step {
+    Texel<P> t[kN];
+    float2 qxy[kN], uv[kN];
+    float qz[kN];
+};
 
 // One tile of kT x kB source pixels of node i against every other node j.
 // The work of the tile is (N-1) x kW units -- unit (jj, c) = target jj, chunk
 // c of 32 x kB consecutive tile pixels -- in target-major order, and warp w
-// takes the N-1 consecutive units [w (N-1), (w+1) (N-1)).  A warp keeps its
-// 21 + 6 + 2 sums in registers while its units stay on one target and
-// reduces them across its lanes (a 31-shuffle reduce-scatter) only when the
-// target changes: about (N-1)/kW + 1 reductions per warp instead of N-1.
-// Per unit each lane takes its kB pixels in batches that go through three
-// phases -- projection and bounds, the target gathers of the batch (all in
-// flight together), then gates, residual, Jacobian and accumulation.  The
-// warp totals are parked in shared memory; one barrier at the end, then the
-// (N-1) x 32 block sums of the tile are written to dpart[tile][jj] (each
-// the sum, in warp order, of the warps that covered that target).
+// takes the N-1 consecutive units [w (N-1), (w+1) (N-1)), of which it runs
+// those whose chunk holds valid pixels.  A warp keeps its 21 + 6 + 2 sums in
+// registers while its units stay on one target and reduces them across its
+// lanes (a 31-shuffle reduce-scatter) only when the target changes: about
+// (N-1)/kW + 1 reductions per warp instead of N-1.  A unit is taken in steps
+// of kN pixels a lane, software-pipelined: the next step's pixels are
+// projected and their target gathers issued (also across a change of target)
+// before the current step's gathers are used, so that a gather's latency
+// passes behind the gates, Jacobians and sums of a step.  The warp totals are
+// parked in shared memory; one barrier at the end, then the (N-1) x 32 block
+// sums of the tile are written to dpart[tile][jj] (each the sum, in warp
+// order, of the warps that covered that target).
 template <bool kFull, int kT, int kB, int P>
 __device__ void dense_tile(const SolveArgs& a, int tile, unsigned char* dsm)
 {
     constexpr int kW = kT / 32;
     constexpr int kTile = kT * kB;
     constexpr int kUnit = 32 * kB;
-    constexpr int kBatch = kB < residual_batch(P) ? kB : residual_batch(P);
-    constexpr int kBatches = kB / kBatch;
-    static_assert(kBatch * kBatches == kB, "pixels per thread: 1 or even");
-    const int N = a.N;
+    constexpr int kMaxN = residual_pipelined(kFull) ? kB / 2 : kB;      // pipelined: at least two steps a unit
+    constexpr int kN = kMaxN < step_pix(kFull) ? kMaxN : step_pix(kFull);
+    constexpr int kSteps = kB / kN;
+    static_assert(kSteps * kN == kB, "a unit is a whole number of steps");
+    const int N = a.N, M1 = N - 1;
     const int i = a.tile_node[tile];
-    const NodeDev Ni = a.nodes[i];
+    const NodeDev& Ni = a.nodes[i];
     const int base = (tile - Ni.tile0) * kTile;
     const int nvalid = min(kTile, Ni.M - base);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float4* sp = reinterpret_cast<float4*>(dsm);
     float4* sn = sp + kTile;
-    PairConst* pc = reinterpret_cast<PairConst*>(sn + kTile);
-    float* red = reinterpret_cast<float*>(pc + kMaxNodes);   // [N-1][kW][32]
+    PairConst* pc = reinterpret_cast<PairConst*>(sn + kTile);      // by jj
+    float* red = reinterpret_cast<float*>(pc + kMaxNodes);         // [N-1][kW][32]
+    const float nan = __int_as_float(0x7fc00000);
     for (int s = threadIdx.x; s < kTile; s += kT) {
-        float4 pp = make_float4(0.f, 0.f, 0.f, 0.f), nn = pp;
+        // past the last valid pixel: NaN, which projects into no image
+        float4 pp = make_float4(nan, nan, nan, 0.f), nn = make_float4(0.f, 0.f, 0.f, 0.f);
         if (s < nvalid) load_source<P>(Ni, base + s, pp, nn);
         sp[s] = pp;
         sn[s] = nn;
     }
-    // the source tile is frame data; the transforms below were written by
-    // the predecessor (the previous update), so the wait goes here
+    const int my_j = (int)threadIdx.x < i ? threadIdx.x : threadIdx.x + 1;
+    NodeDev Nj;
+    if ((int)threadIdx.x < M1) Nj = a.nodes[my_j];
+    // the source tile and the nodes are data of before the solve; the
+    // transforms below were written by the predecessor (the previous update),
+    // so the wait goes here
     pdl_wait_and_release();
-    if (threadIdx.x < N && threadIdx.x != i) fill_pair_const(a, i, threadIdx.x, pc[threadIdx.x]);
+    if ((int)threadIdx.x < M1) fill_pair_const(a, i, my_j, Nj, pc[threadIdx.x]);
     __syncthreads();
     const float dmax2 = a.dmax2, cmin = a.cmin, hub = a.huber_dense;
-    const int M1 = N - 1;
-    int u = warp * M1;
-    const int u_end = u + M1;
-    while (u < u_end) {
-        const int jj = u / kW;
-        const int j = jj < i ? jj : jj + 1;
-        const int u_stop = min(u_end, (jj + 1) * kW);
-        const PairK& K = pc[j].k;
-        const void* tgt = pc[j].tgt;
-        const float zref = pc[j].zref;
-        float acc[kDenseVals];
+    const int nC = (nvalid + kUnit - 1) / kUnit;      // chunks with valid pixels
+    const int u_end = (warp + 1) * M1;
+    static_assert((kW & (kW - 1)) == 0, "warps of a CTA: a power of two");
+    // the next unit of the warp's range whose chunk holds valid pixels
+    auto valid_from = [&](int u) { return (u & (kW - 1)) < nC ? u : (u | (kW - 1)) + 1; };
+    Sums acc;
+    auto clear = [&]() {
 #pragma unroll
-        for (int k = 0; k < kDenseVals; ++k) acc[k] = 0.f;
-        for (; u < u_stop; ++u) {
-            const int c0 = (u - jj * kW) * kUnit;
-            if (c0 >= nvalid) continue;     // chunk past the last valid pixel of the tile
+        for (int k = 0; k < 13; ++k) acc.p[k] = make_float2(0.f, 0.f);
+        acc.s01 = acc.s23 = acc.s45 = 0.f;
+    };
+    clear();
+    // step `sub` of unit u: projection of its pixels, gathers issued
+    auto issue = [&](Step<P, kN>& x, int u, int sub) {
+        const PairConst& C = pc[u / kW];
+        const PairK& K = C.k;
+        const int s0 = (u & (kW - 1)) * kUnit + sub * (32 * kN) + lane;
 #pragma unroll
-            for (int bb = 0; bb < kBatches; ++bb) {
-                // phase 1: q = M p, nearest pixel, bounds
-                float2 qxy[kBatch];
-                float qz[kBatch];
-                int iu[kBatch], iv[kBatch];
-                bool ok[kBatch];
+        for (int k = 0; k < kN; ++k) {
+            const int s = s0 + k * 32;
+            const float4 p = sp[BT_CHECK_IDX(s < kTile, kChkSourceTile, a.ctrl) ? s : 0];
+            int iu, iv;
+            bool ok = assoc_project(K, p.x, p.y, p.z, x.qxy[k], x.qz[k], x.uv[k], iu, iv);
+            ok = ok && BT_CHECK_IDX((unsigned)iu < (unsigned)K.W && (unsigned)iv < (unsigned)K.H, kChkGather, a.ctrl);
+            gather_target<P>(x.t[k], C.tgt, iv * K.W + iu, ok);
+        }
+    };
+    // the gates, residuals, Jacobians and sums of that step
+    auto use = [&](const Step<P, kN>& x, int u, int sub) {
+        const PairConst& C = pc[u / kW];
+        const PairK& K = C.k;
+        const float zref = P == 0 ? 0.f : C.zref;
+        const float4* nn = sn + (u & (kW - 1)) * kUnit + sub * (32 * kN) + lane;
+        // the gates of all the step's pixels side by side, without branches:
+        // they are one dependent chain a pixel
+        bool in[kN];
+        float2 txy[kN], nxy[kN];
+        float tz[kN], nz[kN], r[kN];
 #pragma unroll
-                for (int k = 0; k < kBatch; ++k) {
-                    const int s = c0 + (bb * kBatch + k) * 32 + lane;
-                    const float4 p = sp[BT_CHECK_IDX(s < kTile, kChkSourceTile, a.ctrl) ? s : 0];
-                    ok[k] = assoc_project(K, p.x, p.y, p.z, qxy[k], qz[k], iu[k], iv[k]) && s < nvalid &&
-                            BT_CHECK_IDX((unsigned)iu[k] < (unsigned)K.W && (unsigned)iv[k] < (unsigned)K.H,
-                                         kChkGather, a.ctrl);
-                }
-                // phase 2: the gathers of the batch in flight together
-                float4 t[kBatch];
+        for (int k = 0; k < kN; ++k) {
+            const float4 t = decode_target<P>(x.t[k], zref);
+            const float4 n = nn[k * 32];
+            float2 dxy;
+            float dz;
+            tz[k] = t.x;
+            in[k] = assoc_distance(K, x.uv[k], t.x, x.qxy[k], x.qz[k], dmax2, txy[k], dxy, dz) &
+                    assoc_normal(K, n.x, n.y, n.z, t.y, t.z, t.w, cmin, nxy[k], nz[k]);
+            // r = n' . (t - q), the point-to-plane distance of Eq. 3 expressed in camera j
+            r[k] = assoc_residual(nxy[k], nz[k], dxy, dz);
+        }
 #pragma unroll
-                for (int k = 0; k < kBatch; ++k)
-                    t[k] = ok[k] ? load_target<P>(tgt, (size_t)iv[k] * K.W + iu[k], zref)
-                                  : make_float4(0.f, 0.f, 0.f, 0.f);
-                // phase 3: gates, residual, Jacobian, Huber, accumulation
-#pragma unroll
-                for (int k = 0; k < kBatch; ++k) {
-                    if (!(ok[k] && t[k].x > 0.f)) continue;
-                    float2 txy, dxy;
-                    float dz;
-                    if (!assoc_distance(K, iu[k], iv[k], t[k].x, qxy[k], qz[k], dmax2, txy, dxy, dz))
-                        continue;
-                    const float4 n = sn[c0 + (bb * kBatch + k) * 32 + lane];
-                    float2 nxy;
-                    float nz;
-                    if (!assoc_normal(K, n.x, n.y, n.z, t[k].y, t[k].z, t[k].w, cmin, nxy, nz)) continue;
-                    // accepted: r = n' . (t - q), the point-to-plane distance
-                    // of Eq. 3 expressed in camera j; J~ = (n', t x n')
-                    const float r = assoc_residual(nxy, nz, dxy, dz);
-                    const float ar = fabsf(r);
-                    const bool inl = ar <= hub;
-                    const float rho = inl ? 0.5f * r * r : hub * (ar - 0.5f * hub);
-                    if constexpr (kFull) {
-                        const float w = inl ? 1.f : hub * rcp_approx(ar);
-                        const float tz = t[k].x;
-                        const float2 J23 = make_float2(nz, fmaf(txy.y, nz, -tz * nxy.y));
-                        const float2 J45 = make_float2(fmaf(tz, nxy.x, -txy.x * nz), fmaf(txy.x, nxy.y, -txy.y * nxy.x));
-                        accumulate_pair(acc, nxy, J23, J45, w, r, rho);
-                    } else {
-                        const float2 s = __fadd2_rn(make_float2(acc[27], acc[28]), make_float2(rho, 1.f));
-                        acc[27] = s.x;
-                        acc[28] = s.y;
-                    }
-                }
+        for (int k = 0; k < kN; ++k) {
+            if (!in[k]) continue;
+            const float ar = fabsf(r[k]);
+            const float m = fminf(ar, hub);
+            const float rho = m * fmaf(-0.5f, m, ar);
+            if constexpr (kFull) {
+                const float w = ar <= hub ? 1.f : hub * rcp_approx(ar);
+                const float2 J23 = make_float2(nz[k], fmaf(txy[k].y, nz[k], -tz[k] * nxy[k].y));
+                const float2 J45 =
+                    make_float2(fmaf(tz[k], nxy[k].x, -txy[k].x * nz[k]), fmaf(txy[k].x, nxy[k].y, -txy[k].y * nxy[k].x));
+                accumulate_pair(acc, nxy[k], J23, J45, w, r[k], rho);
+            } else {
+                acc.p[12] = __fadd2_rn(acc.p[12], make_float2(rho, 1.f));
             }
         }
+    };
+    auto flush = [&](int jj) {
         float* slot = red + ((size_t)(BT_CHECK_IDX(jj < M1 && warp < kW, kChkRedSlot, a.ctrl) ? jj : 0) * kW + warp) *
                                 kDenseVals;
         if constexpr (kFull) {
-            slot[lane] = warp_transpose_reduce(acc, lane);
+            float v[kDenseVals];
+            ordered_sums(acc, v);
+            slot[lane] = warp_transpose_reduce(v, lane);
         } else {
-            float c0 = acc[27], c1 = acc[28];
+            float c0 = acc.p[12].x, c1 = acc.p[12].y;
 #pragma unroll
             for (int o = 16; o >= 1; o >>= 1) {
                 c0 += __shfl_xor_sync(0xffffffffu, c0, o);
@@ -533,6 +608,38 @@ __device__ void dense_tile(const SolveArgs& a, int tile, unsigned char* dsm)
                 slot[28] = c1;
             }
         }
+        clear();
+    };
+    int u = nC > 0 ? valid_from(warp * M1) : u_end;
+    if constexpr (residual_pipelined(kFull)) {
+        static_assert(kSteps % 2 == 0, "two steps in flight");
+        Step<P, kN> x0, x1;
+        if (u < u_end) issue(x0, u, 0);
+        while (u < u_end) {
+            const int un = valid_from(u + 1);
+#pragma unroll
+            for (int sub = 0; sub < kSteps; sub += 2) {
+                issue(x1, u, sub + 1);
+                use(x0, u, sub);
+                if (sub + 2 < kSteps) issue(x0, u, sub + 2);
+                else if (un < u_end) issue(x0, un, 0);
+                use(x1, u, sub + 1);
+            }
+            if (un / kW != u / kW || un >= u_end) flush(u / kW);      // the warp's last unit of this target
+            u = un;
+        }
+    } else {
+        while (u < u_end) {
+            const int un = valid_from(u + 1);
+#pragma unroll
+            for (int sub = 0; sub < kSteps; ++sub) {
+                Step<P, kN> x;
+                issue(x, u, sub);
+                use(x, u, sub);
+            }
+            if (un / kW != u / kW || un >= u_end) flush(u / kW);
+            u = un;
+        }
     }
     __syncthreads();
     const int nout = M1 * kDenseVals;
@@ -541,14 +648,14 @@ __device__ void dense_tile(const SolveArgs& a, int tile, unsigned char* dsm)
         if (!kFull && v != 27 && v != 28) continue;
         // warps that covered target jj: units [jj kW, (jj+1) kW), warp = unit / (N-1)
         const int w0 = (jj * kW) / M1, w1 = ((jj + 1) * kW - 1) / M1;
-        float s = 0.f;
-        if constexpr (P == 0) {
-            for (int w = w0; w <= w1; ++w) s += red[((size_t)jj * kW + w) * kDenseVals + v];
-        } else {
-            // compensated (Kahan) sum of the warps' block sums
-            float cmp = 0.f;
-            for (int w = w0; w <= w1; ++w) {
-                const float y = red[((size_t)jj * kW + w) * kDenseVals + v] - cmp;
+        float s = 0.f, cmp = 0.f;
+        for (int w = w0; w <= w1; ++w) {
+            if (w * M1 - jj * kW >= nC) break;      // this warp's chunks of the target, and all later ones, are empty
+            const float x = red[((size_t)jj * kW + w) * kDenseVals + v];
+            if constexpr (P == 0) {
+                s += x;
+            } else {               // compensated (Kahan) sum of the warps' block sums
+                const float y = x - cmp;
                 const float t2 = s + y;
                 cmp = (t2 - s) - y;
                 s = t2;
@@ -639,7 +746,7 @@ __device__ void sparse_edge(const SolveArgs& a, int e)
 
 
 template <bool kFull, int kT, int kB, int P>
-__global__ void __launch_bounds__(kT, residual_threads_per_sm(P, kFull) / kT) residual_kernel(SolveArgs a)
+__global__ void __launch_bounds__(kT, residual_threads_per_sm(kFull) / kT) residual_kernel(SolveArgs a)
 {
     extern __shared__ __align__(16) unsigned char dsm[];
     if ((int)blockIdx.x < a.n_edges) {
@@ -652,7 +759,7 @@ __global__ void __launch_bounds__(kT, residual_threads_per_sm(P, kFull) / kT) re
 
 // Batched residual pass: CTA b takes work item work[b] = (graph, item).
 template <bool kFull, int kT, int kB, int P>
-__global__ void __launch_bounds__(kT, residual_threads_per_sm(P, kFull) / kT) batch_residual_kernel(const SolveArgs* __restrict__ args,
+__global__ void __launch_bounds__(kT, residual_threads_per_sm(kFull) / kT) batch_residual_kernel(const SolveArgs* __restrict__ args,
                                                                        const int2* __restrict__ work)
 {
     extern __shared__ __align__(16) unsigned char dsm[];
@@ -675,22 +782,24 @@ __global__ void __launch_bounds__(kThreads) assoc_debug_kernel(SolveArgs a, int 
 {
     pdl_wait_and_release();
     __shared__ PairConst pc;
-    if (threadIdx.x == 0) fill_pair_const(a, i, j, pc);
+    if (threadIdx.x == 0) fill_pair_const(a, i, j, a.nodes[j], pc);
     __syncthreads();
     const NodeDev Ni = a.nodes[i];
     const PairK& K = pc.k;
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < Ni.M; s += gridDim.x * blockDim.x) {
         float4 p, n;
         load_source<P>(Ni, s, p, n);
-        float2 qxy;
+        float2 qxy, uv;
         float qz;
         int iu, iv;
         int res = -1;
-        if (assoc_project(K, p.x, p.y, p.z, qxy, qz, iu, iv)) {
-            const float4 t = load_target<P>(pc.tgt, (size_t)iv * K.W + iu, pc.zref);
+        if (assoc_project(K, p.x, p.y, p.z, qxy, qz, uv, iu, iv)) {
+            Texel<P> x = {};
+            gather_target<P>(x, pc.tgt, iv * K.W + iu, true);
+            const float4 t = decode_target<P>(x, pc.zref);
             float2 txy, dxy, nxy;
             float dz, nz;
-            if (t.x > 0.f && assoc_distance(K, iu, iv, t.x, qxy, qz, a.dmax2, txy, dxy, dz) &&
+            if (assoc_distance(K, uv, t.x, qxy, qz, a.dmax2, txy, dxy, dz) &&
                 assoc_normal(K, n.x, n.y, n.z, t.y, t.z, t.w, a.cmin, nxy, nz))
                 res = iv * K.W + iu;
         }
