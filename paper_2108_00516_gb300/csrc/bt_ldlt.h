@@ -188,12 +188,212 @@ __host__ __device__ constexpr size_t ldlt_shift_doubles(size_t n) { return (n + 
 // idle(warp): called once by each of warps 1-7 while warp 0 alone runs the
 // first block of the back substitution (work the caller has for otherwise
 // idle warps; it must not touch H, y or the scratch, and is not called when
-// a pivot failed).  All threads of the CTA (blockDim.x == 256) must call it.
+// a pivot failed).  Returns whether idle was called for (false: the system
+// was solved by its FP32 inverse, without a time when warps are idle).  All
+// threads of the CTA (blockDim.x == 256) must call it.
 struct LdltNoIdle {
     __device__ void operator()(int) const {}
 };
 
+// Systems that are solved by their FP32 inverse: its entries stay in the
+// threads' registers, and its panels have to fit the factorisation's.
+constexpr int kInvMinN = 12, kInvMaxN = 120;
+
 #ifdef __CUDACC__
+// H x = b by the FP32 inverse W of the scaled system and corrections of x from
+// its double-float residual, x += W (b - H x).  The scaled normal equations of
+// a pose graph in the object's frame have condition numbers of 20 .. 60, so W
+// is good to about 1e-6 and two corrections reach the accuracy of the
+// double-float residual, without the n dependent double-float pivots of the
+// factorisation below.  W is formed by Gauss-Jordan elimination in steps of
+// six unknowns, one barrier a step: lane = column, warps = column blocks x kG
+// row groups, kR entries of a column in a thread's registers; the panel (six
+// columns, six rows) of the next step goes through shared memory, and every
+// thread factorises the 6 x 6 pivot block for itself.
+// Returns false, F and b untouched, when a pivot is below 2^-10 (the diagonal
+// is in [1, 4)), so that the system may not be positive definite, or when the
+// corrections do not shrink by at least four each; the caller then factorises.
+// F: lower triangle, leading dimension ld; buf: 12 (kR kG + n) floats (16-byte
+// aligned); part: kG n; x: n.
+template <int kR, int kG>
+__device__ __forceinline__ bool inverse_solve(const float2* __restrict__ F, int ld, int n, const float2* __restrict__ b,
+                                              float* __restrict__ buf, float2* __restrict__ part,
+                                              float2* __restrict__ x)
+{
+    constexpr int kRows = kR * kG, kCol = kPan * kRows;      // rows with padding, floats of a column panel
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nb = (n + 31) >> 5, cb = warp % nb, g = warp / nb;
+    const bool active = g < kG;
+    const int j = cb * 32 + lane, jc = min(j, n - 1), i0 = g * kR;
+    float* rows = buf + 2 * kCol;                            // [2][6][n]
+    float w[kR];
+    // publishes the panel of columns c0 .. c0 + 5: columns by column, with 1
+    // taken off the diagonal, and rows
+    auto publish = [&](int c0, int par) {
+        const int jp = j - c0;
+        if ((unsigned)jp < (unsigned)kPan) {
+            float4* c = reinterpret_cast<float4*>(buf + par * kCol + jp * kRows + i0);
+#pragma unroll
+            for (int r = 0; r < kR / 4; ++r) {
+                const int d = j - i0 - 4 * r;
+                c[r] = make_float4(w[4 * r] - (d == 0 ? 1.f : 0.f), w[4 * r + 1] - (d == 1 ? 1.f : 0.f),
+                                   w[4 * r + 2] - (d == 2 ? 1.f : 0.f), w[4 * r + 3] - (d == 3 ? 1.f : 0.f));
+            }
+        }
+        if (i0 < c0 + kPan && i0 + kR > c0) {
+            float* to = rows + par * kPan * n + jc;
+#pragma unroll
+            for (int r = 0; r < kR; ++r) {
+                const int q = i0 + r - c0;
+                if ((unsigned)q < (unsigned)kPan && j < n) to[q * n] = w[r];
+            }
+        }
+    };
+    if (active) {
+#pragma unroll
+        for (int r = 0; r < kR; ++r) {
+            const int i = i0 + r;
+            w[r] = i < n ? F[max(i, jc) * ld + min(i, jc)].x : 0.f;
+        }
+        publish(0, 0);
+    }
+    __syncthreads();
+    bool ok = true;
+    int par = 0;
+    for (int c0 = 0; c0 < n; c0 += kPan, par ^= 1) {
+        if (active) {
+            const float* C = buf + par * kCol;
+            const float* R = rows + par * kPan * n + jc;
+            float D[kPan][kPan], z[kPan], rinv[kPan];
+#pragma unroll
+            for (int q = 0; q < kPan; ++q)
+#pragma unroll
+                for (int p = q; p < kPan; ++p) D[p][q] = C[q * kRows + c0 + p] + (p == q ? 1.f : 0.f);
+            const int jp = j - c0;
+            const bool in_panel = (unsigned)jp < (unsigned)kPan;
+#pragma unroll
+            for (int q = 0; q < kPan; ++q) {
+                const float a = R[q * n];
+                z[q] = in_panel ? (q == jp ? 1.f : 0.f) : a;
+            }
+            // D = L D' L^T in place (L below the diagonal), then D^-1 z
+#pragma unroll
+            for (int p = 0; p < kPan; ++p) {
+                ok = ok && D[p][p] > 0.0009765625f;
+                asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rinv[p]) : "f"(D[p][p]));
+#pragma unroll
+                for (int r = p + 1; r < kPan; ++r) {
+                    const float l = D[r][p] * rinv[p];
+#pragma unroll
+                    for (int c = p + 1; c <= r; ++c) D[r][c] = fmaf(-l, D[c][p], D[r][c]);
+                    z[r] = fmaf(-l, z[p], z[r]);
+                }
+            }
+#pragma unroll
+            for (int p = kPan - 1; p >= 0; --p) {
+#pragma unroll
+                for (int r = kPan - 1; r > p; --r) z[p] = fmaf(-D[r][p], z[r], z[p]);
+                z[p] *= rinv[p];
+            }
+            // the panel's own columns become those of the inverse: they start
+            // from the identity (the rows' 1 is taken off in the panel)
+            if (in_panel) {
+#pragma unroll
+                for (int r = 0; r < kR; ++r) w[r] = i0 + r == j ? 1.f : 0.f;
+            }
+#pragma unroll
+            for (int q = 0; q < kPan; ++q) {
+                const float2 zq = make_float2(-z[q], -z[q]);
+                const float4* c = reinterpret_cast<const float4*>(C + q * kRows + i0);
+#pragma unroll
+                for (int r = 0; r < kR / 4; ++r) {
+                    const float4 c4 = c[r];
+                    const float2 lo = __ffma2_rn(make_float2(c4.x, c4.y), zq, make_float2(w[4 * r], w[4 * r + 1]));
+                    const float2 hi = __ffma2_rn(make_float2(c4.z, c4.w), zq, make_float2(w[4 * r + 2], w[4 * r + 3]));
+                    w[4 * r] = lo.x;
+                    w[4 * r + 1] = lo.y;
+                    w[4 * r + 2] = hi.x;
+                    w[4 * r + 3] = hi.y;
+                }
+            }
+            if (c0 + kPan < n) publish(c0 + kPan, par ^ 1);
+        }
+        __syncthreads();
+    }
+    if (__syncthreads_or(!ok)) return false;
+    float* v = buf;                      // FP32 right-hand side of a correction, zeros in the padding
+    float* top = buf + kRows;            // [8] per-warp maxima of |x|, then [8] of |dx|
+    float* pf = reinterpret_cast<float*>(part);
+    if (tid < kRows) v[tid] = tid < n ? b[tid].x : 0.f;
+    if (tid < n) x[tid] = make_float2(0.f, 0.f);
+    __syncthreads();
+    float before = INFINITY;
+    for (int it = 0; it < 8; ++it) {
+        if (active) {
+            float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+            for (int r = 0; r < kR / 4; ++r) {
+                const float4 v4 = *reinterpret_cast<const float4*>(v + i0 + 4 * r);
+                s0 = fmaf(w[4 * r], v4.x, s0);
+                s1 = fmaf(w[4 * r + 1], v4.y, s1);
+                s0 = fmaf(w[4 * r + 2], v4.z, s0);
+                s1 = fmaf(w[4 * r + 3], v4.w, s1);
+            }
+            if (j < n) pf[g * n + j] = s0 + s1;
+        }
+        __syncthreads();
+        float dx = 0.f, ax = 0.f;
+        if (tid < n) {
+#pragma unroll
+            for (int q = 0; q < kG; ++q) dx += pf[q * n + tid];
+            const float2 xn = ff_add(x[tid], make_float2(dx, 0.f));
+            x[tid] = xn;
+            ax = fabsf(xn.x);
+            dx = fabsf(dx);
+        }
+        // maxima of the bit patterns: a NaN counts as large
+        const unsigned mx = __reduce_max_sync(0xffffffffu, __float_as_uint(ax)),
+                       md = __reduce_max_sync(0xffffffffu, __float_as_uint(dx));
+        if (lane == 0) {
+            top[warp] = __uint_as_float(mx);
+            top[8 + warp] = __uint_as_float(md);
+        }
+        __syncthreads();
+        unsigned ux = 0, ud = 0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            ux = max(ux, __float_as_uint(top[q]));
+            ud = max(ud, __float_as_uint(top[8 + q]));
+        }
+        const float X = __uint_as_float(ux), step = __uint_as_float(ud);
+        if (!(X < INFINITY) || !(step <= 0.25f * before)) return false;
+        // the next correction would be about step^2 / before: below 2^-45 of x?
+        if (step == 0.f || (it > 0 && step * (step / before) <= 2.8e-14f * X)) return true;
+        before = step;
+        if (active) {
+            float2 s0 = g == 0 ? b[jc] : make_float2(0.f, 0.f), s1 = make_float2(0.f, 0.f);
+            const int k1 = min(i0 + kR, n);
+            // H_jk: row j of the triangle up to the diagonal, column j below it
+            int k = i0;
+            for (; k + 1 < k1; k += 2) {
+                s0 = ff_msub_acc(s0, F[max(k, jc) * ld + min(k, jc)], x[k]);
+                s1 = ff_msub_acc(s1, F[max(k + 1, jc) * ld + min(k + 1, jc)], x[k + 1]);
+            }
+            if (k < k1) s0 = ff_msub_acc(s0, F[max(k, jc) * ld + min(k, jc)], x[k]);
+            if (j < n) part[g * n + j] = ff_add(s0, s1);
+        }
+        __syncthreads();
+        if (tid < n) {
+            float2 s = part[tid];
+#pragma unroll
+            for (int q = 1; q < kG; ++q) s = ff_add(s, part[q * n + tid]);
+            v[tid] = s.x + s.y;
+        }
+        __syncthreads();
+    }
+    return false;
+}
+
 // The six values of row i of a panel buffer.
 __device__ __forceinline__ void pan_load(const float2* pan, int i, float2 (&v)[kPan])
 {
@@ -329,7 +529,7 @@ __device__ __forceinline__ void ldlt_trailing(float2* F, int ld, int n, int c1, 
 }
 
 template <typename Idle = LdltNoIdle>
-__device__ __forceinline__ void ldlt_solve(double* __restrict__ H, int ld, int n, double* __restrict__ y,
+__device__ __forceinline__ bool ldlt_solve(double* __restrict__ H, int ld, int n, double* __restrict__ y,
                                            const LdltScratch& sc, int* fail, unsigned long long& t_mid,
                                            const Idle& idle = Idle())
 {
@@ -363,6 +563,23 @@ __device__ __forceinline__ void ldlt_solve(double* __restrict__ H, int ld, int n
         for (int i = lane; i < n; i += 32) yf[i] = ff_from_f64(y[i], shift[i] + e);
     }
     __syncthreads();
+    if (n >= kInvMinN && n <= kInvMaxN && *fail == 0) {
+        float* buf = reinterpret_cast<float*>(pan);
+        float2* p = reinterpret_cast<float2*>(sc.part);
+        const int rows = n <= 32 ? 32 : n <= 64 ? 64 : n <= 96 ? 96 : 120;
+        float2* x = reinterpret_cast<float2*>(buf + 12 * (rows + n));
+        const bool done = n <= 32   ? inverse_solve<4, 8>(F, ld, n, yf, buf, p, x)
+                          : n <= 64 ? inverse_solve<16, 4>(F, ld, n, yf, buf, p, x)
+                          : n <= 96 ? inverse_solve<48, 2>(F, ld, n, yf, buf, p, x)
+                                    : inverse_solve<60, 2>(F, ld, n, yf, buf, p, x);
+        if (done) {
+            t_mid = clock64();
+            for (int i = tid; i < n; i += nt) y[i] = ff_to_f64(x[i], shift[i] - shift[n]);
+            __syncthreads();
+            return false;
+        }
+        __syncthreads();
+    }
     // LDL^T in panels of six columns (one node), the right-hand side carried
     // along as row n, one barrier a panel: the warps that hold the panel's
     // rows bring it up to date and factorise it -- the serial chain of the
@@ -450,6 +667,7 @@ __device__ __forceinline__ void ldlt_solve(double* __restrict__ H, int ld, int n
         y[i] = ff_to_f64(x, shift[i] - shift[n]);
     }
     __syncthreads();
+    return true;
 }
 #endif
 

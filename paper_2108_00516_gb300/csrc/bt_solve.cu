@@ -530,6 +530,7 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
     }
     unsigned long long t1 = clock64();
     unsigned long long t2, t3;
+    bool costs_due = true;      // the energies are still to be added up
     if (a.solver == 1) {
         // Conjugate gradients with the diagonal preconditioner (the paper's
         // inner solver, Sec. IV-D), FP64, from dx = 0.  The matrix-vector
@@ -615,15 +616,15 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
         __syncthreads();
         t2 = t3 = clock64();
     } else {
-    // LDL^T in panels of six columns, D w = z, blocked L^T dx = w
-    // (bt_ldlt.h); the forward substitution of -g is carried along
+    // by the FP32 inverse and corrections, or LDL^T in panels of six columns,
+    // D w = z, blocked L^T dx = w (bt_ldlt.h)
     LdltScratch sc;
     sc.pan = colb;
     sc.shift = reinterpret_cast<int*>(shift);
     sc.part = scratch;
-    // the energies are added up by the last warp while warp 0 runs the
-    // first block of the back substitution alone
-    ldlt_solve(H, ld, n, y, sc, &s_fail, t2, [&](int w) {
+    // the factorisation leaves the last warp time to add the energies up while
+    // warp 0 runs the first block of the back substitution alone
+    costs_due = !ldlt_solve(H, ld, n, y, sc, &s_fail, t2, [&](int w) {
         if (w == cost_warp) write_costs();
     });
     if (s_fail) {
@@ -650,7 +651,7 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
             cf[4 * lane + 1 + warp] = c;
             if (warp == 0) cf[4 * lane] = fma(xi[5], xi[5], fma(xi[4], xi[4], xi[3] * xi[3]));
         }
-        if (a.solver == 1 && warp == cost_warp) write_costs();
+        if (costs_due && warp == cost_warp) write_costs();
         __syncthreads();
         for (int q = tid; q < 12 * nf; q += nt) {
             // rotation entries (f, r, c < 3) first, then the translations
