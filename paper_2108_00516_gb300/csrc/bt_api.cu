@@ -969,7 +969,7 @@ int batch_enqueue(bt_batch* b, int iters, int shape)
     return BT_OK;
 }
 
-// Times one full residual pass per CTA shape and keeps the fastest.
+// Times one full residual pass per CTA shape and picks one.
 int batch_autotune(bt_batch* b)
 {
     cudaEvent_t e0, e1;
@@ -988,8 +988,12 @@ int batch_autotune(bt_batch* b)
         }
         const bt::SolveArgs* A = b->d_args.as<bt::SolveArgs>();
         BT_CUDA(bt::launch_batch_xforms(A, (int)b->graphs.size(), b->stream), "batch xforms");
-        float ms = 0.f, tot = 0.f;
-        for (int rep = 0; rep < 3; ++rep) {
+        // the better of two passes; one where the first is already far off
+        // (the tuning is part of a new batch's first solve: 47 -> 24 ms of
+        // residual passes for 64 graphs against three passes a shape)
+        double us = 1e300;
+        for (int rep = 0; rep < 2 && (rep == 0 || us < 1.3 * best_us); ++rep) {
+            float ms = 0.f;
             BT_CUDA(cudaEventRecord(e0, b->stream), "event");
             BT_CUDA(bt::launch_batch_residual(A, b->d_work_res.as<int2>(), b->n_work_res, b->max_N, true, sh,
                                               b->precision, b->stream),
@@ -997,15 +1001,18 @@ int batch_autotune(bt_batch* b)
             BT_CUDA(cudaEventRecord(e1, b->stream), "event");
             BT_CUDA(cudaEventSynchronize(e1), "event sync");
             BT_CUDA(cudaEventElapsedTime(&ms, e0, e1), "event time");
-            if (rep > 0) tot += ms;
+            us = std::min(us, 1e3 * (double)ms);
         }
-        const double us = 1e3 * tot / 2.0;
         b->tune_us[sh] = us;
         if (us < best_us) {
             best_us = us;
             best = sh;
         }
     }
+    // the single-graph solve's shape where it is within 2 %: the fastest three
+    // shapes are often that close, and with it a graph's result has the same
+    // bits in a batch as on its own
+    if (b->tune_us[bt::kSingleShape] <= 1.02 * best_us) best = bt::kSingleShape;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     b->tuned_shape = best;
