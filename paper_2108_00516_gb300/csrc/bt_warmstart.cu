@@ -3,21 +3,21 @@
 // reduction, Adam, and the FP64 relative-pose averaging solve that turns the
 // predicted edge increments into node poses for Gauss-Newton (Sec. IV-D).
 //
-// Forward pass: two persistent CTAs per SM keep the BF16 W2 (in the tensor
-// cores' core-matrix layout) in shared memory and walk equal shares of the
-// chunks of 128 points of all sets.  Layer 1 (K = 6) runs on the FP32 pipes
-// and is rounded to BF16 into a shared-memory tile; the 128 x 256 x 128
-// contraction of layer 2 runs on the fifth-generation tensor cores
-// (tcgen05.mma, BF16 in, FP32 accumulators in tensor memory, issued by one
-// thread, completion signalled on an mbarrier), while the CUDA cores form the
-// features of the next chunk and the SM's other CTA runs its layer 1 or
-// read-out; then the accumulators are read back (tcgen05.ld) into running
-// per-channel maxima, which are combined over the CTAs of a set with 64-bit
-// atomic maxima (value, then first row).  The 256 -> 128 -> 6 head of all sets
-// is a launch of its own.  Every wait on the tensor cores is bounded
-// (globaltimer); a wait that runs out sets the network's fault word, drains
-// the contraction in flight, frees the tensor memory and ends the kernel, and
-// the host reports BT_ERR_TIMEOUT.
+// Forward pass: a persistent CTA per SM keeps the BF16 W2 (in the tensor
+// cores' core-matrix layout) in shared memory and walks an equal share of the
+// chunks of 128 points of all sets.  Its warps form two groups that work on
+// different chunks at the same time: eight run layer 1 (K = 6) on the FP32
+// pipes, rounded to BF16 into one of two shared-memory tiles, from which one
+// thread issues the 128 x 256 x 128 contraction of layer 2 to the
+// fifth-generation tensor cores (tcgen05.mma, BF16 in, FP32 accumulators in
+// tensor memory, completion signalled on an mbarrier); the other eight read
+// the accumulators of earlier chunks back (tcgen05.ld) into running
+// per-channel maxima and form the features of later ones.  The maxima are
+// combined over the CTAs of a set with 64-bit atomic maxima (value, then
+// first row).  The 256 -> 128 -> 6 head of all sets is a launch of its own.
+// Every wait on the tensor cores is bounded (globaltimer); a wait that runs
+// out sets the network's fault word, drains the contractions in flight, frees
+// the tensor memory and ends the kernel, and the host reports BT_ERR_TIMEOUT.
 // Backward pass: only the rows that hold a channel's maximum receive
 // gradient, so layer 1 and layer 2 gradients are outer products over at most
 // 256 rows, recomputed from the inputs with the forward pass's arithmetic.
@@ -35,7 +35,8 @@ namespace ws {
 
 namespace {
 
-constexpr int kFwdThreads = 256;
+constexpr int kFwdThreads = 512;          // forward kernel: two groups of eight warps
+constexpr int kGroupThreads = 256;        // one of them; also the head kernel
 constexpr int kChunk = 128;     // points per layer-2 tile: the M of one tensor-core contraction
 constexpr int kLd3 = 258;       // padded row length (BF16) of the layer-3 weights (odd word stride)
 
@@ -112,7 +113,7 @@ constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kH2
                             ((uint32_t)(kChunk >> 4) << 24);
 static_assert(kChunk == 128 && kH2 % 16 == 0 && kH2 <= 256, "shape of one kind::f16 contraction (M = 128)");
 
-constexpr int kTmemCols = kH2;                     // one FP32 [128][256] accumulator: two CTAs share an SM's 512 columns
+constexpr int kTmemCols = 2 * kH2;                 // two FP32 [128][256] accumulators
 constexpr long long kTensorWaitNs = 1000000000LL;  // default bound of a wait on the tensor cores (1 s)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p)
@@ -170,6 +171,29 @@ __device__ __forceinline__ bool wait_tensor(uint32_t bar, uint32_t parity, long 
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+
+__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+// Barrier of the kGroupThreads threads of the layer-1 group; true in all of
+// them when any passes `fail`.
+__device__ __forceinline__ bool group_sync_or(bool fail)
+{
+    uint32_t any;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, 1, %2, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(any)
+        : "r"((uint32_t)fail), "n"(kGroupThreads)
+        : "memory");
+    return any != 0;
+}
 
 // Eight 16-lane x 256-bit blocks of tensor memory from taddr on (columns
 // taddr + 8j .. + 8j + 7 for block j), waited for: lane l of the warp gets
@@ -245,29 +269,26 @@ __device__ __forceinline__ int set_chunks(int n) { return n > kChunk ? (n + kChu
 // Shared-memory layout of the forward kernel (byte offsets).
 struct Fwd {
     static constexpr size_t W2 = 0;                                          // bf16 [256][128], core_off layout
-    static constexpr size_t H1 = W2 + 2 * (size_t)kH2 * kH1;                 // bf16 [128][128], core_off layout
-    static constexpr size_t W1 = H1 + (size_t)kH1TileBytes;                  // float [64][16]: unit pairs (layer1_rows)
+    static constexpr size_t H1 = W2 + 2 * (size_t)kH2 * kH1;                 // 2 x bf16 [128][128], core_off layout
+    static constexpr size_t W1 = H1 + 2 * (size_t)kH1TileBytes;              // float [64][16]: unit pairs (layer1_rows)
     static constexpr size_t B2 = W1 + 4 * (size_t)kH1 * 8;                   // float [256]
-    static constexpr size_t X = B2 + 4 * (size_t)kH2;                        // float [128][kLdX]
-    static constexpr size_t SMP = X + 4 * (size_t)kChunk * kLdX;             // four Samples
-    static constexpr size_t SCAN = SMP + 4 * 128;                            // int [8 + 2]
-    static constexpr size_t BAR = SCAN + 48;                                 // mbarrier (u64)
-    static constexpr size_t TM = BAR + 16;                                   // tensor-memory base address
+    static constexpr size_t X = B2 + 4 * (size_t)kH2;                        // 2 x float [128][kLdX]
+    static constexpr size_t SCAN = X + 8 * (size_t)kChunk * kLdX;            // int [16 + 2], fault word
+    static constexpr size_t BAR = SCAN + 80;                                 // six mbarriers (u64)
+    static constexpr size_t TM = BAR + 48;                                   // tensor-memory base address
     static constexpr size_t Total = TM + 16;
 };
-static_assert(sizeof(Sample) <= 128 && offsetof(Sample, c) + 12 <= 128, "a set's description is one 128-byte read of a warp");
-static_assert(Fwd::H1 % 16 == 0 && Fwd::W1 % 16 == 0 && Fwd::X % 16 == 0 && Fwd::SMP % 16 == 0 && Fwd::BAR % 8 == 0,
-              "alignment");
-static_assert(2 * (Fwd::Total + 1024) <= 228 * 1024, "two CTAs per SM");
-static_assert(2 * kTmemCols <= 512, "two CTAs per SM");
-static_assert(kFwdThreads == kH2 && kFwdThreads == 2 * kChunk, "thread mappings");
+static_assert(Fwd::H1 % 16 == 0 && Fwd::W1 % 16 == 0 && Fwd::X % 16 == 0 && Fwd::BAR % 8 == 0, "alignment");
+static_assert(Fwd::Total <= 227 * 1024, "shared memory of one CTA");
+static_assert(Fwd::Total > 114 * 1024, "one CTA per SM: the two accumulators take all of its tensor memory");
+static_assert(kFwdThreads == 2 * kGroupThreads && kGroupThreads == kH2 && kGroupThreads == 2 * kChunk, "thread mappings");
 
 // The forward pass up to the max-pool.  pool[s][256]: running maximum of each
 // channel, (float bits of relu(max z + b2)) << 32 | ~row (row 0xffffffff where
 // it is not kept), zero on entry.  The chunks of all sets, in order, are
 // divided evenly over the CTAs, wherever the sets begin and end.
 template <bool kTrain>
-__global__ void __launch_bounds__(kFwdThreads, kTrain ? 1 : 2)
+__global__ void __launch_bounds__(kFwdThreads, 1)
     forward_kernel(Net net, const Sample* __restrict__ smp, const int* __restrict__ ids, int n_sets,
                    unsigned long long* __restrict__ pool)
 {
@@ -276,15 +297,17 @@ __global__ void __launch_bounds__(kFwdThreads, kTrain ? 1 : 2)
     float* sB2 = reinterpret_cast<float*>(sm + Fwd::B2);
     float* sX = reinterpret_cast<float*>(sm + Fwd::X);
     int* sScan = reinterpret_cast<int*>(sm + Fwd::SCAN);
-    auto sample = [&](int set) { return reinterpret_cast<const Sample*>(sm + Fwd::SMP + 128 * (set & 3)); };
+    volatile int* sFault = sScan + 18;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
     // this CTA's share of the chunks: each thread adds up a run of sets, the
     // thread whose run holds the first chunk finds its set
     auto id_of = [&](int s) { return ids ? __ldg(ids + s) : s; };
+    auto points_of = [&](int s) { return __ldg(&smp[id_of(s)].n); };
     const int r0 = (int)((long long)tid * n_sets / kFwdThreads), r1 = (int)((long long)(tid + 1) * n_sets / kFwdThreads);
     int mine = 0;
-    for (int s = r0; s < r1; ++s) mine += set_chunks(__ldg(&smp[id_of(s)].n));
+#pragma unroll 4
+    for (int s = r0; s < r1; ++s) mine += set_chunks(points_of(s));
     int incl = mine;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -301,20 +324,21 @@ __global__ void __launch_bounds__(kFwdThreads, kTrain ? 1 : 2)
     }
     before += incl - mine;
     const int x0 = (int)((long long)blockIdx.x * total / gridDim.x);
-    const int x1 = (int)((long long)(blockIdx.x + 1) * total / gridDim.x);
-    if (x0 >= x1) return;
+    const int count = (int)((long long)(blockIdx.x + 1) * total / gridDim.x) - x0;
+    if (count <= 0) return;
     if (before <= x0 && x0 < before + mine) {
         int s = r0, at = before;
         for (;; ++s) {
-            const int k = set_chunks(__ldg(&smp[id_of(s)].n));
+            const int k = set_chunks(points_of(s));
             if (x0 < at + k) break;
             at += k;
         }
-        sScan[8] = s;
-        sScan[9] = x0 - at;
+        sScan[16] = s;
+        sScan[17] = x0 - at;
     }
 
     // stage the weights once per CTA; W2 as 16-byte core-matrix rows
+#pragma unroll 8
     for (int k = tid; k < kH2 * kH1 / 8; k += kFwdThreads) {
         const int row = k >> 4, k8 = (k & 15) * 8;
         *reinterpret_cast<uint4*>(sm + Fwd::W2 + core_off(row, k8)) =
@@ -324,12 +348,21 @@ __global__ void __launch_bounds__(kFwdThreads, kTrain ? 1 : 2)
         const int u = 2 * (k >> 4) + (k & 1), e = (k & 15) >> 1;
         sW1[k] = e < kIn ? bf2f(net.wb[bW1 + u * kIn + e]) : (e == kIn ? net.master[ob1 + u] : 0.f);
     }
-    sB2[tid] = net.master[ob2 + tid];
+    if (tid < kH2) sB2[tid] = net.master[ob2 + tid];
 
+    // mbarriers of the two buffers: contraction done (the accumulator is full,
+    // the tile free), accumulator free again (one arrival a read-out warp),
+    // features ready (one a feature warp)
     const uint32_t bar = smem_u32(sm + Fwd::BAR);
+    const uint32_t bar_done = bar, bar_free = bar + 16, bar_x = bar + 32;
     if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(bar_done + 8 * b, 1);
+            mbar_init(bar_free + 8 * b, kGroupThreads / 32);
+            mbar_init(bar_x + 8 * b, kChunk / 32);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        *sFault = 0;
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(sm + Fwd::TM)),
@@ -337,205 +370,229 @@ __global__ void __launch_bounds__(kFwdThreads, kTrain ? 1 : 2)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    // the tensor cores read W2 and the layer-1 tile through the async proxy
+    // the tensor cores read W2 and the layer-1 tiles through the async proxy
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(sm + Fwd::TM);
     const uint32_t w2_s = smem_u32(sm + Fwd::W2), h1_s = smem_u32(sm + Fwd::H1);
-    unsigned char* const h1_tile = sm + Fwd::H1;
-    int s = sScan[8], c = sScan[9];          // the set and the chunk of it at hand
+    int issued = 0;                          // contractions issued (thread 0)
 
-    // a set's description (its Sample) goes to one of four slots, by warp 4:
-    // the first three here, each other one two sets ahead of its turn
-    auto desc_word = [&](int set) {
-        return lane < (int)(sizeof(Sample) / 4) ? __ldg(reinterpret_cast<const unsigned*>(smp + id_of(set)) + lane) : 0u;
-    };
-    auto desc_put = [&](int set, unsigned w) { reinterpret_cast<unsigned*>(sm + Fwd::SMP + 128 * (set & 3))[lane] = w; };
-    if (warp == 4)
-        for (int q = s; q < min(s + 3, n_sets); ++q) desc_put(q, desc_word(q));
-    __syncthreads();
-    // the point pair of this thread's row of chunk ch of set st (warps 0-3; zeros past the last point)
-    auto load_points = [&](int st, int ch, float (&v)[6]) {
-        const Sample* S = sample(st);
-        const int k = ch * kChunk + tid;
-        const bool in = k < S->n;
-#pragma unroll
-        for (int e = 0; e < 3; ++e) {
-            v[e] = in ? __ldg(S->p + 3 * (size_t)k + e) : 0.f;
-            v[3 + e] = in ? __ldg(S->q + 3 * (size_t)k + e) : 0.f;
-        }
-    };
-    // its features, zeros past the last point
-    auto features = [&](int st, int ch, const float (&v)[6]) {
-        const Sample* S = sample(st);
-        float x[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        if (ch * kChunk + tid < S->n) features_from(v, S->m, S->c, x);
-        float* xr = sX + tid * kLdX;
-        *reinterpret_cast<float4*>(xr) = make_float4(x[0], x[1], x[2], x[3]);
-        *reinterpret_cast<float2*>(xr + 4) = make_float2(x[4], x[5]);
-    };
-    // points are loaded a chunk before their features are formed, so that
-    // their latency passes behind a whole chunk's work: (fs, fc) is the chunk
-    // whose points are in pq
-    float pq[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    int fs = s, fc = c;
-    auto advance = [&]() {
-        if (fc + 1 < set_chunks(sample(fs)->n)) {
-            ++fc;
-        } else {
-            ++fs;
-            fc = 0;
-        }
-    };
-    if (tid < kChunk) {
-        load_points(fs, fc, pq);
-        features(fs, fc, pq);
-        advance();
-        if (x0 + 1 < x1) load_points(fs, fc, pq);
-    }
-    __syncthreads();
-
-    // read-out: warp w takes the tensor-memory lanes (rows of a chunk)
-    // 32 (w % 4) .. + 31 and the columns 128 (w / 4) .. + 127; a lane holds
-    // 32 of those columns (idx: column 128 cw + 8 (idx / 2) + 2 (lane % 4) + idx % 2)
-    const int qr = warp & 3, cw = warp >> 2;
-    // running maxima of the thread's 32 columns; training keeps relu(z + b)
-    // and the row that holds it (first row on ties), inference the largest z:
-    // adding the bias and the ReLU are monotonic, so they follow the maximum
-    float best[32];
-    int bestr[kTrain ? 32 : 1];
-    auto reset = [&]() {
-#pragma unroll
-        for (int k = 0; k < 32; ++k) {
-            best[k] = kTrain ? -1.f : -INFINITY;
-            if constexpr (kTrain) bestr[k] = 0;
-        }
-    };
-    reset();
-    bool fault = false;
-    bool fresh = true;                       // the first chunk of this CTA of its set
-    for (int x = x0; x < x1; ++x) {
-        const int n = sample(s)->n, nch = set_chunks(n);
-        const bool last = c + 1 == nch;      // the last chunk of its set
-        const bool more = x + 1 < x1;
-        unsigned w = 0;
-        const bool fetch = fresh && warp == 4 && s + 2 < n_sets;
-        if (fetch) w = desc_word(s + 2);
-        fresh = false;
-        layer1_rows(h1_tile, sW1, sX, warp, lane);
-        if (fetch) desc_put(s + 2, w);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        tc_fence_before();
-        __syncthreads();
-        tc_fence_after();
-        if (tid == 0) issue_layer2(tmem, h1_s, w2_s, bar);
-        // the next chunk's features while the tensor cores work on this one,
-        // and the loads of the one after it
-        if (more && tid < kChunk) {
-            features(fs, fc, pq);
-            advance();
-            if (x + 2 < x1) load_points(fs, fc, pq);
-        }
-        const uint32_t parity = (uint32_t)(x - x0) & 1u;
-        const bool done = wait_tensor(bar, parity, net.wait_ns);
-        tc_fence_before();
-        if (__syncthreads_or(!done)) {
-            // give the contraction in flight time to finish before the
-            // tensor memory is freed, then end the kernel
-            wait_tensor(bar, parity, kTensorWaitNs);
-            fault = true;
-            break;
-        }
-        tc_fence_after();
-        // the running maximum over the rows of the chunk, in increasing order
-        const uint32_t tacc = tmem + 128 * cw;
-#pragma unroll
-        for (int lh = 0; lh < 2; ++lh) {
-            const int rb = c * kChunk + 32 * qr + 16 * lh;
-            if (rb >= n) break;   // the same for the whole warp
-            const int ra = rb + (lane >> 2), rc = ra + 8;
-            const bool va = ra < n, vc = rc < n;
-#pragma unroll
-            for (int cq = 0; cq < 2; ++cq) {
-                uint32_t v[32];
-                tmem_load_16x256b_x8(tacc + ((uint32_t)(32 * qr + 16 * lh) << 16) + 64 * cq, v);
-#pragma unroll
-                for (int g = 0; g < 8; ++g)
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int k = 2 * (8 * cq + g) + e;
-                        if constexpr (kTrain) {
-                            const float b2 = sB2[128 * cw + 8 * (k >> 1) + 2 * (lane & 3) + (k & 1)];
-                            const float za = fmaxf(__uint_as_float(v[4 * g + e]) + b2, 0.f);
-                            if (va && za > best[k]) {
-                                best[k] = za;
-                                bestr[k] = ra;
-                            }
-                            const float zc = fmaxf(__uint_as_float(v[4 * g + 2 + e]) + b2, 0.f);
-                            if (vc && zc > best[k]) {
-                                best[k] = zc;
-                                bestr[k] = rc;
-                            }
-                        } else {
-                            if (va) best[k] = fmaxf(best[k], __uint_as_float(v[4 * g + e]));
-                            if (vc) best[k] = fmaxf(best[k], __uint_as_float(v[4 * g + 2 + e]));
-                        }
-                    }
+    if (warp < kGroupThreads / 32) {
+        // layer 1 of chunk i into tile i % 2, once its features are there and
+        // the contraction of chunk i - 2 has read the tile; then the
+        // contraction, once the accumulator of chunk i - 2 has been read
+        for (int i = 0; i < count; ++i) {
+            const uint32_t b = i & 1, ph = (i >> 1) & 1;
+            bool ok = wait_tensor(bar_x + 8 * b, ph, net.wait_ns);
+            if (i >= 2) ok = ok && wait_tensor(bar_done + 8 * b, ph ^ 1, net.wait_ns);
+            layer1_rows(sm + Fwd::H1 + b * kH1TileBytes, sW1, sX + b * kChunk * kLdX, warp, lane);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            tc_fence_before();
+            if (group_sync_or(!ok || *sFault != 0)) {
+                *sFault = 1;
+                break;
             }
-        }
-        tc_fence_before();
-        if (last || !more) {
-            // combine the 8 lanes of each column by recursive halving: lane l
-            // ends with the columns idx0 .. idx0 + 3, idx0 = its bits 4, 3, 2
-            int idx0 = 0;
-#pragma unroll
-            for (int st = 0; st < 3; ++st) {
-                const int off = 16 >> st, half = 16 >> st;
-                const bool upper = (lane & off) != 0;
-#pragma unroll
-                for (int k = 0; k < half; ++k) {
-                    const float send = upper ? best[k] : best[k + half];
-                    float keep = upper ? best[k + half] : best[k];
-                    const float got = __shfl_xor_sync(0xffffffffu, send, off);
-                    if constexpr (kTrain) {
-                        const int rsend = upper ? bestr[k] : bestr[k + half];
-                        int rkeep = upper ? bestr[k + half] : bestr[k];
-                        const int rgot = __shfl_xor_sync(0xffffffffu, rsend, off);
-                        if (got > keep || (got == keep && rgot < rkeep)) {
-                            keep = got;
-                            rkeep = rgot;
-                        }
-                        bestr[k] = rkeep;
-                    } else {
-                        keep = fmaxf(keep, got);
-                    }
-                    best[k] = keep;
+            tc_fence_after();
+            if (tid == 0) {
+                if (i < 2 || wait_tensor(bar_free + 8 * b, ph ^ 1, net.wait_ns)) {
+                    tc_fence_after();
+                    issue_layer2(tmem + b * kH2, h1_s + b * kH1TileBytes, w2_s, bar_done + 8 * b);
+                    issued = i + 1;
+                } else {
+                    *sFault = 1;             // seen by the group at its next barrier
                 }
-                idx0 += upper ? half : 0;
             }
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int idx = idx0 + k;
-                const int col = 128 * cw + 8 * (idx >> 1) + 2 * (lane & 3) + (idx & 1);
-                const float g = kTrain ? best[k] : fmaxf(best[k] + sB2[col], 0.f);
-                const unsigned row = kTrain ? ~(unsigned)bestr[k] : 0u;
-                if (g > 0.f || (kTrain && g == 0.f))
-                    atomicMax(pool + (size_t)s * kH2 + col,
-                              ((unsigned long long)__float_as_uint(g) << 32) | row);
-            }
-            reset();
         }
-        if (last) {
-            ++s;
-            c = 0;
-            fresh = true;
-        } else {
-            ++c;
+    } else {
+        const int gw = warp - kGroupThreads / 32, gt = tid - kGroupThreads;
+        int s = sScan[16], c = sScan[17];    // the set and the chunk of it to be read out
+        // features (the first kChunk threads of the group, one row each) are
+        // formed two chunks ahead of the read-out, and their points loaded one
+        // chunk before that; (fs, fc) is the chunk whose points are in pq, and
+        // the description of its set and of the next is kept in registers so
+        // that a change of set waits for no chain of loads
+        int fs = s, fc = c;
+        struct Set {
+            const Sample* S;
+            const float* p;
+            const float* q;
+            int n;
+        };
+        auto describe = [&](int set) {
+            Set d;
+            d.S = smp + id_of(min(set, n_sets - 1));
+            d.n = __ldg(&d.S->n);
+            d.p = reinterpret_cast<const float*>(__ldg(reinterpret_cast<const unsigned long long*>(&d.S->p)));
+            d.q = reinterpret_cast<const float*>(__ldg(reinterpret_cast<const unsigned long long*>(&d.S->q)));
+            return d;
+        };
+        Set cur, nxt;
+        float pq[6];
+        auto load_points = [&]() {
+            const int k = fc * kChunk + gt;
+            const bool in = k < cur.n;
+#pragma unroll
+            for (int e = 0; e < 3; ++e) {
+                pq[e] = in ? __ldg(cur.p + 3 * (size_t)k + e) : 0.f;
+                pq[3 + e] = in ? __ldg(cur.q + 3 * (size_t)k + e) : 0.f;
+            }
+        };
+        // features of (fs, fc) into buffer b, then the points of the chunk after it
+        auto features = [&](uint32_t b, bool more) {
+            float x[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            float m[12], cc[3];
+#pragma unroll
+            for (int e = 0; e < 12; ++e) m[e] = __ldg(cur.S->m + e);
+#pragma unroll
+            for (int e = 0; e < 3; ++e) cc[e] = __ldg(cur.S->c + e);
+            if (fc * kChunk + gt < cur.n) features_from(pq, m, cc, x);
+            float* xr = sX + b * kChunk * kLdX + gt * kLdX;
+            *reinterpret_cast<float4*>(xr) = make_float4(x[0], x[1], x[2], x[3]);
+            *reinterpret_cast<float2*>(xr + 4) = make_float2(x[4], x[5]);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_x + 8 * b);
+            if (!more) return;
+            if (fc + 1 < set_chunks(cur.n)) {
+                ++fc;
+            } else {
+                ++fs;
+                fc = 0;
+                cur = nxt;
+                nxt = describe(fs + 1);
+            }
+            load_points();
+        };
+        if (gt < kChunk) {
+            cur = describe(fs);
+            nxt = describe(fs + 1);
+            load_points();
+            features(0, count > 1);
+            if (count > 1) features(1, count > 2);
+        }
+        // read-out: warp gw takes the tensor-memory lanes (rows of a chunk)
+        // 32 (gw % 4) .. + 31 and the columns 128 (gw / 4) .. + 127; a lane holds
+        // 32 of those columns (idx: column 128 cw + 8 (idx / 2) + 2 (lane % 4) + idx % 2)
+        const int qr = gw & 3, cw = gw >> 2;
+        // running maxima of the thread's 32 columns; training keeps relu(z + b)
+        // and the row that holds it (first row on ties), inference the largest z:
+        // adding the bias and the ReLU are monotonic, so they follow the maximum
+        float best[32];
+        int bestr[kTrain ? 32 : 1];
+        auto reset = [&]() {
+#pragma unroll
+            for (int k = 0; k < 32; ++k) {
+                best[k] = kTrain ? -1.f : -INFINITY;
+                if constexpr (kTrain) bestr[k] = 0;
+            }
+        };
+        reset();
+        int n = points_of(s), n_next = points_of(min(s + 1, n_sets - 1));
+        for (int i = 0; i < count; ++i) {
+            const uint32_t b = i & 1, ph = (i >> 1) & 1;
+            if (__any_sync(0xffffffffu, !wait_tensor(bar_done + 8 * b, ph, net.wait_ns))) {
+                if (lane == 0) *sFault = 1;
+                break;
+            }
+            tc_fence_after();
+            // the contraction has read the tile, so layer 1 is done with the features of chunk i
+            if (gt < kChunk && i + 2 < count) features(b, i + 3 < count);
+            // the running maximum over the rows of the chunk, in increasing order
+            const uint32_t tacc = tmem + b * kH2 + 128 * cw;
+#pragma unroll
+            for (int lh = 0; lh < 2; ++lh) {
+                const int rb = c * kChunk + 32 * qr + 16 * lh;
+                if (rb >= n) break;   // the same for the whole warp
+                const int ra = rb + (lane >> 2), rc = ra + 8;
+                const bool va = ra < n, vc = rc < n;
+#pragma unroll
+                for (int cq = 0; cq < 2; ++cq) {
+                    uint32_t v[32];
+                    tmem_load_16x256b_x8(tacc + ((uint32_t)(32 * qr + 16 * lh) << 16) + 64 * cq, v);
+#pragma unroll
+                    for (int g = 0; g < 8; ++g)
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const int k = 2 * (8 * cq + g) + e;
+                            if constexpr (kTrain) {
+                                const float b2 = sB2[128 * cw + 8 * (k >> 1) + 2 * (lane & 3) + (k & 1)];
+                                const float za = fmaxf(__uint_as_float(v[4 * g + e]) + b2, 0.f);
+                                if (va && za > best[k]) {
+                                    best[k] = za;
+                                    bestr[k] = ra;
+                                }
+                                const float zc = fmaxf(__uint_as_float(v[4 * g + 2 + e]) + b2, 0.f);
+                                if (vc && zc > best[k]) {
+                                    best[k] = zc;
+                                    bestr[k] = rc;
+                                }
+                            } else {
+                                if (va) best[k] = fmaxf(best[k], __uint_as_float(v[4 * g + e]));
+                                if (vc) best[k] = fmaxf(best[k], __uint_as_float(v[4 * g + 2 + e]));
+                            }
+                        }
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_free + 8 * b);
+            const bool last = c + 1 == set_chunks(n);      // the last chunk of its set
+            if (last || i + 1 == count) {
+                // combine the 8 lanes of each column by recursive halving: lane l
+                // ends with the columns idx0 .. idx0 + 3, idx0 = its bits 4, 3, 2
+                int idx0 = 0;
+#pragma unroll
+                for (int st = 0; st < 3; ++st) {
+                    const int half = 16 >> st;
+                    const bool upper = (lane & half) != 0;
+#pragma unroll
+                    for (int k = 0; k < half; ++k) {
+                        const float send = upper ? best[k] : best[k + half];
+                        float keep = upper ? best[k + half] : best[k];
+                        const float got = __shfl_xor_sync(0xffffffffu, send, half);
+                        if constexpr (kTrain) {
+                            const int rsend = upper ? bestr[k] : bestr[k + half];
+                            int rkeep = upper ? bestr[k + half] : bestr[k];
+                            const int rgot = __shfl_xor_sync(0xffffffffu, rsend, half);
+                            if (got > keep || (got == keep && rgot < rkeep)) {
+                                keep = got;
+                                rkeep = rgot;
+                            }
+                            bestr[k] = rkeep;
+                        } else {
+                            keep = fmaxf(keep, got);
+                        }
+                        best[k] = keep;
+                    }
+                    idx0 += upper ? half : 0;
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int idx = idx0 + k;
+                    const int col = 128 * cw + 8 * (idx >> 1) + 2 * (lane & 3) + (idx & 1);
+                    const float g = kTrain ? best[k] : fmaxf(best[k] + sB2[col], 0.f);
+                    const unsigned row = kTrain ? ~(unsigned)bestr[k] : 0u;
+                    if (g > 0.f || (kTrain && g == 0.f))
+                        atomicMax(pool + (size_t)s * kH2 + col, ((unsigned long long)__float_as_uint(g) << 32) | row);
+                }
+                reset();
+            }
+            if (last) {
+                ++s;
+                c = 0;
+                n = n_next;
+                n_next = points_of(min(s + 1, n_sets - 1));
+            } else {
+                ++c;
+            }
         }
     }
-    if (fault && tid == 0) {
+    __syncthreads();
+    if (*sFault != 0 && tid == 0) {
+        // give the contractions in flight time to finish before the tensor
+        // memory is freed
+        for (int i = max(0, issued - 2); i < issued; ++i) wait_tensor(bar_done + 8 * (i & 1), (i >> 1) & 1, kTensorWaitNs);
         *reinterpret_cast<volatile int*>(net.fault) = 1;
         __threadfence_system();
     }
@@ -560,7 +617,7 @@ struct Head {
 };
 
 template <bool kTrain>
-__global__ void __launch_bounds__(kFwdThreads)
+__global__ void __launch_bounds__(kGroupThreads)
     head_kernel(Net net, const Sample* __restrict__ smp, const int* __restrict__ ids, int n_sets,
                 const unsigned long long* __restrict__ pool, float* __restrict__ y_out, Cache* __restrict__ cache)
 {
@@ -571,7 +628,7 @@ __global__ void __launch_bounds__(kFwdThreads)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int s0 = blockIdx.x * kHeadSets, m = min(kHeadSets, n_sets - s0);
 #pragma unroll 16
-    for (int k = tid; k < kH3 * kH2 / 2; k += kFwdThreads) {   // bf16 pairs, rows padded to kLd3
+    for (int k = tid; k < kH3 * kH2 / 2; k += kGroupThreads) {   // bf16 pairs, rows padded to kLd3
         const int o = k / (kH2 / 2), c2 = (k % (kH2 / 2)) * 2;
         *reinterpret_cast<uint32_t*>(sW3 + o * kLd3 + c2) =
             *reinterpret_cast<const uint32_t*>(net.wb + bW3 + o * kH2 + c2);
@@ -622,7 +679,7 @@ __global__ void __launch_bounds__(kFwdThreads)
     }
     __syncthreads();
     // layer 4: one warp per set, then its outputs in turn
-    static_assert(kFwdThreads / 32 == kHeadSets, "one warp per set");
+    static_assert(kGroupThreads / 32 == kHeadSets, "one warp per set");
     if (warp < m) {
         const int s = s0 + warp;
         const bool empty = __ldg(&smp[ids ? __ldg(ids + s) : s].n) <= 0;       // no prediction
@@ -1290,8 +1347,8 @@ static cudaError_t launch_forward_t(Net net, const Sample* smp, const int* ids, 
     ForwardAttr<kTrain>::set();
     const cudaError_t e = cudaMemsetAsync(pool, 0, pool_bytes(n), s);
     if (e != cudaSuccess) return e;
-    forward_kernel<kTrain><<<(kTrain ? 1 : 2) * num_sms(), kFwdThreads, Fwd::Total, s>>>(net, smp, ids, n, pool);
-    head_kernel<kTrain><<<(n + kHeadSets - 1) / kHeadSets, kFwdThreads, Head::Total, s>>>(net, smp, ids, n, pool, y_out,
+    forward_kernel<kTrain><<<num_sms(), kFwdThreads, Fwd::Total, s>>>(net, smp, ids, n, pool);
+    head_kernel<kTrain><<<(n + kHeadSets - 1) / kHeadSets, kGroupThreads, Head::Total, s>>>(net, smp, ids, n, pool, y_out,
                                                                                          cache);
     return cudaGetLastError();
 }
