@@ -627,11 +627,29 @@ __global__ void __launch_bounds__(kGroupThreads)
     float* sP = reinterpret_cast<float*>(sm + Head::P);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int s0 = blockIdx.x * kHeadSets, m = min(kHeadSets, n_sets - s0);
-#pragma unroll 16
-    for (int k = tid; k < kH3 * kH2 / 2; k += kGroupThreads) {   // bf16 pairs, rows padded to kLd3
-        const int o = k / (kH2 / 2), c2 = (k % (kH2 / 2)) * 2;
-        *reinterpret_cast<uint32_t*>(sW3 + o * kLd3 + c2) =
-            *reinterpret_cast<const uint32_t*>(net.wb + bW3 + o * kH2 + c2);
+    constexpr int kPer = kH3 * kH2 / 8 / kGroupThreads;
+    uint4 w16[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k)
+        w16[k] = __ldg(reinterpret_cast<const uint4*>(net.wb + bW3) + tid + k * kGroupThreads);
+    float w4[kOut][kH3 / 32], b4[kOut];
+#pragma unroll
+    for (int k = 0; k < kOut; ++k) {
+#pragma unroll
+        for (int i = 0; i < kH3 / 32; ++i) w4[k][i] = bf2f(net.wb[bW4 + k * kH3 + lane + 32 * i]);
+        b4[k] = net.master[ob4 + k];
+    }
+    const float b3 = net.master[ob3 + (tid & (kH3 - 1))];
+    // everything above is parameters; the maxima come from the predecessor
+    pdl_wait_and_release();
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {   // eight values, rows padded to kLd3
+        const int at = (tid + k * kGroupThreads) * 8;
+        uint32_t* to = reinterpret_cast<uint32_t*>(sW3 + (at / kH2) * kLd3 + at % kH2);
+        to[0] = w16[k].x;
+        to[1] = w16[k].y;
+        to[2] = w16[k].z;
+        to[3] = w16[k].w;
     }
 #pragma unroll
     for (int q = 0; q < kHeadSets; ++q) {
@@ -652,16 +670,20 @@ __global__ void __launch_bounds__(kGroupThreads)
 #pragma unroll
         for (int q = 0; q < kHeadSets; ++q) a[q] = 0.f;
 #pragma unroll 4
-        for (int k = 0; k < 128; ++k) {
-            const float wk = bf2f(w[k]);
-            const float4* g = reinterpret_cast<const float4*>(sG + (half * 128 + k) * kHeadSets);
+        for (int k = 0; k < 128; k += 2) {
+            const __nv_bfloat162 w2 = *reinterpret_cast<const __nv_bfloat162*>(w + k);
 #pragma unroll
-            for (int q = 0; q < kHeadSets / 4; ++q) {
-                const float4 g4 = g[q];
-                a[4 * q] = __fmaf_rn(wk, g4.x, a[4 * q]);
-                a[4 * q + 1] = __fmaf_rn(wk, g4.y, a[4 * q + 1]);
-                a[4 * q + 2] = __fmaf_rn(wk, g4.z, a[4 * q + 2]);
-                a[4 * q + 3] = __fmaf_rn(wk, g4.w, a[4 * q + 3]);
+            for (int e = 0; e < 2; ++e) {
+                const float wk = e == 0 ? __low2float(w2) : __high2float(w2);
+                const float4* g = reinterpret_cast<const float4*>(sG + (half * 128 + k + e) * kHeadSets);
+#pragma unroll
+                for (int q = 0; q < kHeadSets / 4; ++q) {
+                    const float4 g4 = g[q];
+                    a[4 * q] = __fmaf_rn(wk, g4.x, a[4 * q]);
+                    a[4 * q + 1] = __fmaf_rn(wk, g4.y, a[4 * q + 1]);
+                    a[4 * q + 2] = __fmaf_rn(wk, g4.z, a[4 * q + 2]);
+                    a[4 * q + 3] = __fmaf_rn(wk, g4.w, a[4 * q + 3]);
+                }
             }
         }
 #pragma unroll
@@ -669,7 +691,6 @@ __global__ void __launch_bounds__(kGroupThreads)
     }
     __syncthreads();
     if (tid < kH3) {
-        const float b3 = net.master[ob3 + tid];
 #pragma unroll
         for (int q = 0; q < kHeadSets; ++q) {
             const float z = b3 + (sP[q * kH3 + tid] + sP[(kHeadSets + q) * kH3 + tid]);
@@ -688,10 +709,10 @@ __global__ void __launch_bounds__(kGroupThreads)
             float a = 0.f;
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-                a = __fmaf_rn(bf2f(net.wb[bW4 + k * kH3 + lane + 32 * i]), sP[warp * kH3 + lane + 32 * i], a);
+                a = __fmaf_rn(w4[k][i], sP[warp * kH3 + lane + 32 * i], a);
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
-            const float y = empty ? 0.f : net.master[ob4 + k] + a;
+            const float y = empty ? 0.f : b4[k] + a;
             if (lane == 0) {
                 y_out[(size_t)s * kOut + k] = y;
                 if (kTrain) cache[s].y[k] = y;
@@ -734,94 +755,118 @@ int num_sms()
 // 71 + 37 us for a minibatch of 256 sets.
 // ---------------------------------------------------------------------------
 
-constexpr int kBwdThreads = 256;
+// 1024 threads: a set's chain of loads and sums is what takes the time, and
+// splitting its sums over 256 outputs eight and four ways shortens it (256
+// threads: 32 us for 256 sets).
+constexpr int kBwdThreads = 1024;
 
 __global__ void __launch_bounds__(kBwdThreads)
     backward_kernel(Net net, const Sample* __restrict__ smp, const int* __restrict__ ids, int n_sets,
                     Cache* __restrict__ cache, float inv_n, BwdRec* __restrict__ rec)
 {
-    __shared__ float sdz2[kH2], sdz3[kH3], sdy[8], sMC[16];
+    constexpr int kPartsO = kBwdThreads / kH2, kO = kH3 / kPartsO;      // layer 3: units of a part
+    constexpr int kPartsC = kBwdThreads / kH1, kC = kH2 / kPartsC;      // layer 1: channels of a part
+    __shared__ float sdz2[kH2], sdz3[kH3], sMC[16], sg[kPartsO][kH2];
     __shared__ float sxr[kH2 * 8];           // features of channel c's row at 8 c
-    __shared__ float spart[kH1][7];
+    __shared__ float spart[kPartsC][kH1][7];
     const int s = blockIdx.x, tid = threadIdx.x;
     const int sid = ids ? ids[s] : s;
     const Sample* S = smp + sid;
-    const Cache* C = cache + s;
     BwdRec& R = rec[s];
     const int n = S->n;
+    const int c = tid & (kH2 - 1), part = tid >> 8, j = tid & (kH1 - 1), seg = tid >> 7;
+    // parameters and the set's own data first: the cache comes from the predecessor
+    float w3[kO], w1[6], w2[kC];
+#pragma unroll
+    for (int o = 0; o < kO; ++o) w3[o] = bf2f(net.wb[bW3 + (part * kO + o) * kH2 + c]);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) w1[k] = bf2f(net.wb[bW1 + j * kIn + k]);
+    const float b1 = net.master[ob1 + j];
+    if (tid < 12) sMC[tid] = S->m[tid];
+    else if (tid < 15) sMC[tid] = S->c[tid - 12];
+    pdl_wait_and_release();
     if (n <= 0) {      // no forward pass: contributes nothing
-        cache[s].g[tid] = 0.f;
+        if (tid < kH2) cache[s].g[tid] = 0.f;
         float* f = reinterpret_cast<float*>(&R);
         for (int k = tid; k < (int)(sizeof(BwdRec) / sizeof(float)); k += kBwdThreads) f[k] = 0.f;
         return;
     }
-    const float g = C->g[tid];
-    const int row = min(max(C->r[tid], 0), n - 1);
-    const float z3 = tid < kH3 ? C->z3[tid] : 0.f;
-    if (tid < 12) sMC[tid] = S->m[tid];
-    else if (tid < 15) sMC[tid] = S->c[tid - 12];
-    if (tid < kOut) sdy[tid] = C->y[tid] - S->ystar[tid];
-    __syncthreads();
+    const Cache* C = cache + s;
+    float dy[kOut];
+#pragma unroll
+    for (int m = 0; m < kOut; ++m) dy[m] = __ldcg(&C->y[m]) - __ldg(&S->ystar[m]);
+    const float g = __ldcg(&C->g[c]);
+    const int row = min(max(__ldcg(&C->r[c]), 0), n - 1);
+    __syncthreads();      // sMC
     if (tid == 0) {
         float l = 0.f;
-        for (int m = 0; m < kOut; ++m) l = __fmaf_rn(sdy[m], sdy[m], l);
+#pragma unroll
+        for (int m = 0; m < kOut; ++m) l = __fmaf_rn(dy[m], dy[m], l);
         R.loss = 0.5f * l * inv_n;
+#pragma unroll
+        for (int m = 0; m < kOut; ++m) R.dy[m] = dy[m] * inv_n;
     }
     // layer 4
-    if (tid < kOut) R.dy[tid] = sdy[tid] * inv_n;
     if (tid < kH3) {
+        const float z3 = __ldcg(&C->z3[tid]);
         float a = 0.f;
 #pragma unroll
-        for (int m = 0; m < kOut; ++m) a = __fmaf_rn(bf2f(net.wb[bW4 + m * kH3 + tid]), sdy[m] * inv_n, a);
+        for (int m = 0; m < kOut; ++m) a = __fmaf_rn(bf2f(net.wb[bW4 + m * kH3 + tid]), dy[m] * inv_n, a);
         const float d = z3 > 0.f ? a : 0.f;
         sdz3[tid] = d;
         R.dz3[tid] = d;
         R.h3[tid] = fmaxf(z3, 0.f);
-    }
-    float x[6];
-    point_features(S->p, S->q, sMC, sMC + 12, row, x);
+    } else if (part == 1) {
+        float x[6];
+        point_features(S->p, S->q, sMC, sMC + 12, row, x);
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        sxr[tid * 8 + k] = x[k];
-        R.x[tid][k] = x[k];
+        for (int k = 0; k < 6; ++k) {
+            sxr[c * 8 + k] = x[k];
+            R.x[c][k] = x[k];
+        }
     }
     __syncthreads();
     // layer 3: dg = W3^T dz3, and ReLU' at the row holding the maximum
     {
         float a = 0.f;
-#pragma unroll 32
-        for (int o = 0; o < kH3; ++o) a = __fmaf_rn(bf2f(net.wb[bW3 + o * kH2 + tid]), sdz3[o], a);
+#pragma unroll
+        for (int o = 0; o < kO; ++o) a = __fmaf_rn(w3[o], sdz3[part * kO + o], a);
+        sg[part][c] = a;
+    }
+#pragma unroll
+    for (int q = 0; q < kC; ++q) w2[q] = bf2f(net.wb[bW2 + (seg * kC + q) * kH1 + j]);
+    __syncthreads();
+    if (part == 0) {
+        float a = sg[0][c];
+#pragma unroll
+        for (int q = 1; q < kPartsO; ++q) a += sg[q][c];
         const float d = g > 0.f ? a : 0.f;
-        sdz2[tid] = d;
-        R.x[tid][6] = d;
+        sdz2[c] = d;
+        R.x[c][6] = d;
     }
     __syncthreads();
     // layer 1: dW1[j][k] = sum_c dz2[c] W2[c][j] [z1(r_c, j) > 0] x(r_c)[k]
-    const int j = tid & 127, half = tid >> 7;
-    float w1[6];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) w1[k] = bf2f(net.wb[bW1 + j * kIn + k]);
-    const float b1 = net.master[ob1 + j];
     float a[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll 16
-    for (int c = half * 128; c < half * 128 + 128; ++c) {
-        const float4 xa = *reinterpret_cast<const float4*>(sxr + c * 8);
-        const float2 xb = *reinterpret_cast<const float2*>(sxr + c * 8 + 4);
+#pragma unroll
+    for (int q = 0; q < kC; ++q) {
+        const int ch = seg * kC + q;
+        const float4 xa = *reinterpret_cast<const float4*>(sxr + ch * 8);
+        const float2 xb = *reinterpret_cast<const float2*>(sxr + ch * 8 + 4);
         const float xc[6] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y};
-        const float w = z1_unit(w1, b1, xc) > 0.f ? sdz2[c] * bf2f(net.wb[bW2 + c * kH1 + j]) : 0.f;
+        const float w = z1_unit(w1, b1, xc) > 0.f ? sdz2[ch] * w2[q] : 0.f;
 #pragma unroll
         for (int k = 0; k < 6; ++k) a[k] = __fmaf_rn(w, xc[k], a[k]);
         a[6] += w;
     }
-    if (half == 1) {
 #pragma unroll
-        for (int k = 0; k < 7; ++k) spart[j][k] = a[k];
-    }
+    for (int k = 0; k < 7; ++k) spart[seg][j][k] = a[k];
     __syncthreads();
-    if (half == 0) {
+    if (tid < kH1 * 7) {
+        const int jj = tid / 7, k = tid % 7;
+        float v = spart[0][jj][k];
 #pragma unroll
-        for (int k = 0; k < 6; ++k) R.dw1[j * kIn + k] = a[k] + spart[j][k];
-        R.dw1[kH1 * kIn + j] = a[6] + spart[j][6];
+        for (int q = 1; q < kPartsC; ++q) v += spart[q][jj][k];
+        R.dw1[k < 6 ? jj * kIn + k : kH1 * kIn + jj] = v;
     }
 }
 
@@ -829,19 +874,21 @@ __global__ void __launch_bounds__(kBwdThreads)
 // order: four groups of sets side by side in a CTA, then the groups.  CTAs
 // [0, 128): two rows of dW2 each, dW2[c][j] = sum_s dz2[c] bf16(relu(z1(row
 // r_c, unit j))) with the layer-1 output formed again from the row's features;
-// [128, 256): one row of dW3 = sum_s dz3 g^T each; the others 256 of the
-// remaining parameters each.
+// [128, 160): four rows of dW3 = sum_s dz3 g^T each (one row a CTA would read
+// the pooled features 128 times); the others 256 of the remaining parameters
+// each.
 constexpr int kSumThreads = 1024, kSumGroups = 4, kSumSets = 128;
-constexpr int kSumW2 = kH2 / 2, kSumW3 = kH3;
+constexpr int kSumRows = 4, kSumW2 = kH2 / 2, kSumW3 = kH3 / kSumRows;
 constexpr int kSumRest = kH1 * kIn + kH1 + kH2 + kH3 + kOut * kH3 + kOut;
 constexpr int kSumBlocks = kSumW2 + kSumW3 + (kSumRest + 255) / 256;
 
-__global__ void __launch_bounds__(kSumThreads)
+__global__ void __launch_bounds__(kSumThreads, 1)
     gradient_kernel(Net net, const BwdRec* __restrict__ rec, const Cache* __restrict__ cache, int n,
                     float* __restrict__ grad, double* __restrict__ loss)
 {
     __shared__ float4 sx[kSumSets][2][2];        // features and dz2 of two channels' rows
     __shared__ float part[kSumGroups][256];
+    pdl_wait_and_release();
     const int tid = threadIdx.x, col = tid & 255, grp = tid >> 8, b = blockIdx.x;
     float a = 0.f;
     int p = -1;                                  // the parameter this thread's column sums
@@ -857,7 +904,7 @@ __global__ void __launch_bounds__(kSumThreads)
             __syncthreads();
             if (tid < 4 * m)
                 sx[tid >> 2][(tid >> 1) & 1][tid & 1] =
-                    __ldg(reinterpret_cast<const float4*>(rec[s0 + (tid >> 2)].x[2 * b + ((tid >> 1) & 1)]) + (tid & 1));
+                    __ldcg(reinterpret_cast<const float4*>(rec[s0 + (tid >> 2)].x[2 * b + ((tid >> 1) & 1)]) + (tid & 1));
             __syncthreads();
 #pragma unroll 4
             for (int s = grp; s < m; s += kSumGroups) {
@@ -868,29 +915,63 @@ __global__ void __launch_bounds__(kSumThreads)
             }
         }
     } else if (b < kSumW2 + kSumW3) {
-        const int o = b - kSumW2;
-        p = oW3 + o * kH2 + col;
-#pragma unroll 8
-        for (int s = grp; s < n; s += kSumGroups) a = __fmaf_rn(__ldg(&rec[s].dz3[o]), __ldg(&cache[s].g[col]), a);
+        const int o = (b - kSumW2) * kSumRows;
+        float r[kSumRows] = {0.f, 0.f, 0.f, 0.f};
+        // eight sets' loads in flight (left to the compiler they follow one another)
+        for (int s0 = grp; s0 < n; s0 += 8 * kSumGroups) {
+            float4 d[8];
+            float g[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int s = s0 + u * kSumGroups;
+                d[u] = s < n ? __ldcg(reinterpret_cast<const float4*>(&rec[s].dz3[o])) : make_float4(0.f, 0.f, 0.f, 0.f);
+                g[u] = s < n ? __ldcg(&cache[s].g[col]) : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                r[0] = __fmaf_rn(d[u].x, g[u], r[0]);
+                r[1] = __fmaf_rn(d[u].y, g[u], r[1]);
+                r[2] = __fmaf_rn(d[u].z, g[u], r[2]);
+                r[3] = __fmaf_rn(d[u].w, g[u], r[3]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < kSumRows; ++q) {
+            __syncthreads();
+            part[grp][col] = r[q];
+            __syncthreads();
+            if (grp == 0) grad[oW3 + (o + q) * kH2 + col] = (part[0][col] + part[1][col]) + (part[2][col] + part[3][col]);
+        }
+        return;
     } else {
         const int q = (b - kSumW2 - kSumW3) * 256 + col;
         constexpr int e1 = kH1 * kIn, e2 = e1 + kH1, e3 = e2 + kH2, e4 = e3 + kH3, e5 = e4 + kOut * kH3;
         if (q < kSumRest) {
             p = q < e1 ? oW1 + q : q < e2 ? ob1 + q - e1 : q < e3 ? ob2 + q - e2 : q < e4 ? ob3 + q - e3
                 : q < e5 ? oW4 + q - e4 : ob4 + q - e5;
-#pragma unroll 8
-            for (int s = grp; s < n; s += kSumGroups) {
-                const BwdRec& R = rec[s];
-                if (q < e2) a += __ldg(R.dw1 + q);                 // dW1, then db1
-                else if (q < e3) a += __ldg(&R.x[q - e2][6]);
-                else if (q < e4) a += __ldg(R.dz3 + q - e3);
-                else if (q < e5) a = __fmaf_rn(__ldg(R.dy + (q - e4) / kH3), __ldg(R.h3 + (q - e4) % kH3), a);
-                else a += __ldg(R.dy + q - e5);
+            // where in a set's record the parameter's terms are (a product of two for W4)
+            const int at = q < e2   ? (int)(offsetof(BwdRec, dw1) / 4) + q      // dW1, then db1
+                           : q < e3 ? 8 * (q - e2) + 6
+                           : q < e4 ? (int)(offsetof(BwdRec, dz3) / 4) + q - e3
+                           : q < e5 ? (int)(offsetof(BwdRec, h3) / 4) + (q - e4) % kH3
+                                    : (int)(offsetof(BwdRec, dy) / 4) + q - e5;
+            const int fac = q >= e4 && q < e5 ? (int)(offsetof(BwdRec, dy) / 4) + (q - e4) / kH3 : -1;
+            for (int s0 = grp; s0 < n; s0 += 8 * kSumGroups) {
+                float v[8], f[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int s = s0 + u * kSumGroups;
+                    const float* R = reinterpret_cast<const float*>(rec + min(s, n - 1));
+                    v[u] = s < n ? __ldcg(R + at) : 0.f;
+                    f[u] = fac >= 0 ? __ldcg(R + fac) : 1.f;
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u) a = __fmaf_rn(v[u], f[u], a);
             }
         }
         if (b == kSumBlocks - 1 && tid >= kSumThreads - 32) {
             double l = 0.0;
-            for (int s = tid & 31; s < n; s += 32) l += (double)__ldg(&rec[s].loss);
+            for (int s = tid & 31; s < n; s += 32) l += (double)__ldcg(&rec[s].loss);
 #pragma unroll
             for (int o = 16; o >= 1; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
             if ((tid & 31) == 0) *loss = l;
@@ -1348,9 +1429,10 @@ static cudaError_t launch_forward_t(Net net, const Sample* smp, const int* ids, 
     const cudaError_t e = cudaMemsetAsync(pool, 0, pool_bytes(n), s);
     if (e != cudaSuccess) return e;
     forward_kernel<kTrain><<<num_sms(), kFwdThreads, Fwd::Total, s>>>(net, smp, ids, n, pool);
-    head_kernel<kTrain><<<(n + kHeadSets - 1) / kHeadSets, kGroupThreads, Head::Total, s>>>(net, smp, ids, n, pool, y_out,
-                                                                                         cache);
-    return cudaGetLastError();
+    const cudaError_t f = cudaGetLastError();
+    if (f != cudaSuccess) return f;
+    return launch_chained(head_kernel<kTrain>, dim3((n + kHeadSets - 1) / kHeadSets), dim3(kGroupThreads), Head::Total, s,
+                          net, smp, ids, n, pool, y_out, cache);
 }
 
 cudaError_t launch_forward(Net net, const Sample* smp, const int* ids, int n, unsigned long long* pool, float* y_out,
@@ -1365,9 +1447,10 @@ cudaError_t launch_backward(Net net, const Sample* smp, const int* ids, int n, C
                             float* grad, double* loss, cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
-    backward_kernel<<<n, kBwdThreads, 0, s>>>(net, smp, ids, n, cache, 1.0f / (float)n, rec);
-    gradient_kernel<<<kSumBlocks, kSumThreads, 0, s>>>(net, rec, cache, n, grad, loss);
-    return cudaGetLastError();
+    const cudaError_t e = launch_chained(backward_kernel, dim3(n), dim3(kBwdThreads), 0, s, net, smp, ids, n, cache,
+                                         1.0f / (float)n, rec);
+    if (e != cudaSuccess) return e;
+    return launch_chained(gradient_kernel, dim3(kSumBlocks), dim3(kSumThreads), 0, s, net, rec, cache, n, grad, loss);
 }
 
 cudaError_t launch_adam(Net net, const float* grad, float lr, float beta1, float beta2, float eps, float c1,
