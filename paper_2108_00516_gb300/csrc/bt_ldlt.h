@@ -1,26 +1,29 @@
 // bt_ldlt.h -- solve of a symmetric positive-definite FP64 system H x = y by
-// one CTA of 256 threads: the square-root-free Cholesky factorisation
-// H = L D L^T with a one-column look-ahead (forward substitution L z = y
-// carried along), D w = z, and a blocked back substitution L^T x = w.  Used
-// by the Gauss-Newton step of Sec. IV-D (bt_solve.cu) and by the learned
+// one CTA of 256 threads: by an FP32 inverse and corrections from the
+// double-float residual (18 .. 120 unknowns), or, for other sizes and where
+// the corrections do not settle, by the square-root-free Cholesky
+// factorisation H = L D L^T with a one-panel look-ahead (forward substitution
+// L z = y carried along), D w = z, and a blocked back substitution L^T x = w.
+// Used by the Gauss-Newton step of Sec. IV-D (bt_solve.cu) and by the learned
 // warm start's relative-pose averaging (bt_warmstart.cu).
 //
-// Arithmetic: every value is a pair of FP32 numbers h + l (double-float, 48
-// bits), on the FP32 pipes.  On GB300 a dependent FP64 operation costs ~64
-// cycles or more and a warp-wide FP64 instruction holds its sub-partition's
-// DP unit for ~64 cycles whatever the number of active lanes; a double-float
-// multiply-subtract is 12 FP32 instructions with a dependent chain of ~30
-// cycles.  The solve is bound by the chain of n pivots, so that latency sets
-// its pace.  The system is first scaled by powers of two to a diagonal in
-// [1, 4) (exact, and it keeps every value inside the FP32 exponent range).
+// Arithmetic: the system, the right-hand side and the solution are pairs of
+// FP32 numbers h + l (double-float, 48 bits), on the FP32 pipes.  On GB300 a
+// dependent FP64 operation costs ~64 cycles or more and a warp-wide FP64
+// instruction holds its sub-partition's DP unit for ~64 cycles whatever the
+// number of active lanes; a double-float multiply-subtract is 12 FP32
+// instructions with a dependent chain of ~30 cycles.  The system is first
+// scaled by powers of two to a diagonal in [1, 4) (exact, and it keeps every
+// value inside the FP32 exponent range).
 // Error of the solution against an 80-bit one, relative to its largest entry
-// (72 Gauss-Newton systems of 6 .. 138 unknowns): median 1e-14 .. 3e-13, at
-// most 8e-13; the FP64 form this replaced, whose pivots' reciprocals were
-// good to 1e-12: median 2e-13 .. 1.4e-12, at most 2.1e-12.
-// Measured (one CTA, cycles, factorisation + back substitution): n = 18:
-// 10.8 k + 2.7 k -> 6.9 k + 2.1 k; n = 54: 45.5 k + 9.5 k -> 22.1 k + 6.2 k;
-// n = 114: 213.6 k + 22.4 k -> 90.2 k + 14.2 k.  What is left is mostly the
-// instructions of one warp's panel (~850 of them, ~2.4 k cycles a panel).
+// (60 Gauss-Newton systems, worst of each size): inverse and corrections
+// 4e-14 .. 1.5e-13 for 24 .. 120 unknowns, factorisation 8e-13; an FP64
+// factorisation with pivots' reciprocals good to 1e-12: 7e-13 .. 2.5e-12.
+// Measured (one CTA, cycles, whole solve, inverse against factorisation): n =
+// 18: 9.8 k against 9.0 k, n = 54: 23 k against 28 k, n = 114: 104 k against
+// 104 k of which 14 k are the back substitution's; FP64 factorisation: 13 k,
+// 55 k, 236 k.  One pivot a step instead of six, without the redundant 6 x 6
+// factorisations: 32 k at n = 54, 135 k at n = 114.
 #pragma once
 
 #include "bt_internal.h"
@@ -197,7 +200,7 @@ struct LdltNoIdle {
 
 // Systems that are solved by their FP32 inverse: its entries stay in the
 // threads' registers, and its panels have to fit the factorisation's.
-constexpr int kInvMinN = 12, kInvMaxN = 120;
+constexpr int kInvMinN = 18, kInvMaxN = 120;
 
 #ifdef __CUDACC__
 // H x = b by the FP32 inverse W of the scaled system and corrections of x from
@@ -207,53 +210,51 @@ constexpr int kInvMinN = 12, kInvMaxN = 120;
 // double-float residual, without the n dependent double-float pivots of the
 // factorisation below.  W is formed by Gauss-Jordan elimination in steps of
 // six unknowns, one barrier a step: lane = column, warps = column blocks x kG
-// row groups, kR entries of a column in a thread's registers; the panel (six
-// columns, six rows) of the next step goes through shared memory, and every
-// thread factorises the 6 x 6 pivot block for itself.
+// row groups, kR entries of a column in a thread's registers (kR a multiple of
+// six, so that a panel's rows lie in one group); the panel (six columns, six
+// rows) of the next step goes through shared memory, and every thread
+// factorises the 6 x 6 pivot block for itself.
 // Returns false, F and b untouched, when a pivot is below 2^-10 (the diagonal
 // is in [1, 4)), so that the system may not be positive definite, or when the
 // corrections do not shrink by at least four each; the caller then factorises.
-// F: lower triangle, leading dimension ld; buf: 12 (kR kG + n) floats (16-byte
-// aligned); part: kG n; x: n.
+// F: lower triangle, leading dimension ld; buf: 12 (inv_stride(kR) kG + n)
+// floats (16-byte aligned); part: kG n; x: n.
+__host__ __device__ constexpr int inv_stride(int kR) { return (kR + 3) & ~3; }                 // of a row group, in floats
 template <int kR, int kG>
 __device__ __forceinline__ bool inverse_solve(const float2* __restrict__ F, int ld, int n, const float2* __restrict__ b,
                                               float* __restrict__ buf, float2* __restrict__ part,
                                               float2* __restrict__ x)
 {
-    constexpr int kRows = kR * kG, kCol = kPan * kRows;      // rows with padding, floats of a column panel
+    static_assert(kR % kPan == 0, "a panel's rows in one group");
+    constexpr int kS = inv_stride(kR), kRows = kS * kG, kCol = kPan * kRows;      // floats of a column, of a column panel
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nb = (n + 31) >> 5, cb = warp % nb, g = warp / nb;
     const bool active = g < kG;
     const int j = cb * 32 + lane, jc = min(j, n - 1), i0 = g * kR;
     float* rows = buf + 2 * kCol;                            // [2][6][n]
-    float w[kR];
-    // publishes the panel of columns c0 .. c0 + 5: columns by column, with 1
-    // taken off the diagonal, and rows
+    float w[kS];
+    // publishes the panel of columns and rows c0 .. c0 + 5
     auto publish = [&](int c0, int par) {
         const int jp = j - c0;
         if ((unsigned)jp < (unsigned)kPan) {
-            float4* c = reinterpret_cast<float4*>(buf + par * kCol + jp * kRows + i0);
+            float4* c = reinterpret_cast<float4*>(buf + par * kCol + jp * kRows + g * kS);
 #pragma unroll
-            for (int r = 0; r < kR / 4; ++r) {
-                const int d = j - i0 - 4 * r;
-                c[r] = make_float4(w[4 * r] - (d == 0 ? 1.f : 0.f), w[4 * r + 1] - (d == 1 ? 1.f : 0.f),
-                                   w[4 * r + 2] - (d == 2 ? 1.f : 0.f), w[4 * r + 3] - (d == 3 ? 1.f : 0.f));
-            }
+            for (int r = 0; r < kS / 4; ++r) c[r] = make_float4(w[4 * r], w[4 * r + 1], w[4 * r + 2], w[4 * r + 3]);
         }
-        if (i0 < c0 + kPan && i0 + kR > c0) {
-            float* to = rows + par * kPan * n + jc;
+        float* to = rows + par * kPan * n + jc;
 #pragma unroll
-            for (int r = 0; r < kR; ++r) {
-                const int q = i0 + r - c0;
-                if ((unsigned)q < (unsigned)kPan && j < n) to[q * n] = w[r];
+        for (int q = 0; q < kR / kPan; ++q)
+            if (i0 + kPan * q == c0) {
+#pragma unroll
+                for (int e = 0; e < kPan; ++e)
+                    if (j < n) to[e * n] = w[kPan * q + e];
             }
-        }
     };
     if (active) {
 #pragma unroll
-        for (int r = 0; r < kR; ++r) {
+        for (int r = 0; r < kS; ++r) {
             const int i = i0 + r;
-            w[r] = i < n ? F[max(i, jc) * ld + min(i, jc)].x : 0.f;
+            w[r] = r < kR && i < n ? F[max(i, jc) * ld + min(i, jc)].x : 0.f;
         }
         publish(0, 0);
     }
@@ -264,11 +265,12 @@ __device__ __forceinline__ bool inverse_solve(const float2* __restrict__ F, int 
         if (active) {
             const float* C = buf + par * kCol;
             const float* R = rows + par * kPan * n + jc;
+            const float* Cd = C + c0 / kR * kS + c0 % kR;      // the panel's own rows
             float D[kPan][kPan], z[kPan], rinv[kPan];
 #pragma unroll
             for (int q = 0; q < kPan; ++q)
 #pragma unroll
-                for (int p = q; p < kPan; ++p) D[p][q] = C[q * kRows + c0 + p] + (p == q ? 1.f : 0.f);
+                for (int p = q; p < kPan; ++p) D[p][q] = Cd[q * kRows + p];
             const int jp = j - c0;
             const bool in_panel = (unsigned)jp < (unsigned)kPan;
 #pragma unroll
@@ -295,18 +297,17 @@ __device__ __forceinline__ bool inverse_solve(const float2* __restrict__ F, int 
                 for (int r = kPan - 1; r > p; --r) z[p] = fmaf(-D[r][p], z[r], z[p]);
                 z[p] *= rinv[p];
             }
-            // the panel's own columns become those of the inverse: they start
-            // from the identity (the rows' 1 is taken off in the panel)
+            // the panel's own columns become those of the inverse
             if (in_panel) {
 #pragma unroll
-                for (int r = 0; r < kR; ++r) w[r] = i0 + r == j ? 1.f : 0.f;
+                for (int r = 0; r < kS; ++r) w[r] = 0.f;
             }
 #pragma unroll
             for (int q = 0; q < kPan; ++q) {
                 const float2 zq = make_float2(-z[q], -z[q]);
-                const float4* c = reinterpret_cast<const float4*>(C + q * kRows + i0);
+                const float4* c = reinterpret_cast<const float4*>(C + q * kRows + g * kS);
 #pragma unroll
-                for (int r = 0; r < kR / 4; ++r) {
+                for (int r = 0; r < kS / 4; ++r) {
                     const float4 c4 = c[r];
                     const float2 lo = __ffma2_rn(make_float2(c4.x, c4.y), zq, make_float2(w[4 * r], w[4 * r + 1]));
                     const float2 hi = __ffma2_rn(make_float2(c4.z, c4.w), zq, make_float2(w[4 * r + 2], w[4 * r + 3]));
@@ -316,6 +317,13 @@ __device__ __forceinline__ bool inverse_solve(const float2* __restrict__ F, int 
                     w[4 * r + 3] = hi.y;
                 }
             }
+            // and its own rows D^-1 times what they were
+#pragma unroll
+            for (int q = 0; q < kR / kPan; ++q)
+                if (i0 + kPan * q == c0) {
+#pragma unroll
+                    for (int e = 0; e < kPan; ++e) w[kPan * q + e] = z[e];
+                }
             if (c0 + kPan < n) publish(c0 + kPan, par ^ 1);
         }
         __syncthreads();
@@ -324,16 +332,21 @@ __device__ __forceinline__ bool inverse_solve(const float2* __restrict__ F, int 
     float* v = buf;                      // FP32 right-hand side of a correction, zeros in the padding
     float* top = buf + kRows;            // [8] per-warp maxima of |x|, then [8] of |dx|
     float* pf = reinterpret_cast<float*>(part);
-    if (tid < kRows) v[tid] = tid < n ? b[tid].x : 0.f;
-    if (tid < n) x[tid] = make_float2(0.f, 0.f);
+    const int vi = tid / kR * kS + tid % kR;      // place of entry tid among the row groups
+    if (tid < kRows) v[tid] = 0.f;
+    __syncthreads();
+    if (tid < n) {
+        v[vi] = b[tid].x;
+        x[tid] = make_float2(0.f, 0.f);
+    }
     __syncthreads();
     float before = INFINITY;
     for (int it = 0; it < 8; ++it) {
         if (active) {
             float s0 = 0.f, s1 = 0.f;
 #pragma unroll
-            for (int r = 0; r < kR / 4; ++r) {
-                const float4 v4 = *reinterpret_cast<const float4*>(v + i0 + 4 * r);
+            for (int r = 0; r < kS / 4; ++r) {
+                const float4 v4 = *reinterpret_cast<const float4*>(v + g * kS + 4 * r);
                 s0 = fmaf(w[4 * r], v4.x, s0);
                 s1 = fmaf(w[4 * r + 1], v4.y, s1);
                 s0 = fmaf(w[4 * r + 2], v4.z, s0);
@@ -387,7 +400,7 @@ __device__ __forceinline__ bool inverse_solve(const float2* __restrict__ F, int 
             float2 s = part[tid];
 #pragma unroll
             for (int q = 1; q < kG; ++q) s = ff_add(s, part[q * n + tid]);
-            v[tid] = s.x + s.y;
+            v[vi] = s.x + s.y;
         }
         __syncthreads();
     }
@@ -548,8 +561,27 @@ __device__ __forceinline__ bool ldlt_solve(double* __restrict__ H, int ld, int n
         shift[i] = -((f - 1023) >> 1);
     }
     __syncthreads();
-    for (int i = warp; i < n; i += nt >> 5)
-        for (int j = lane; j <= i; j += 32) F[i * ld + j] = ff_from_f64(H[i * ld + j], shift[i] + shift[j]);
+    for (int i = warp; i < n; i += nt >> 5) {
+        // a row's parts together: the compiler keeps loads behind the stores
+        // to the same memory
+        constexpr int kParts = (kLdltMaxN + 31) / 32;
+        double h[kParts];
+        int e[kParts];
+#pragma unroll
+        for (int q = 0; q < kParts; ++q) {
+            const int j = min(lane + 32 * q, i);
+            h[q] = H[i * ld + j];
+            e[q] = shift[j];
+        }
+        const int si = shift[i];
+#pragma unroll
+        for (int q = 0; q < kParts; ++q) {
+            const int j = lane + 32 * q;
+            if (32 * q > i) break;
+            const float2 f = ff_from_f64(h[q], si + e[q]);
+            if (j <= i) F[i * ld + j] = f;
+        }
+    }
     if (warp == 7) {
         int e = -100000;
         for (int i = lane; i < n; i += 32) {
@@ -566,10 +598,11 @@ __device__ __forceinline__ bool ldlt_solve(double* __restrict__ H, int ld, int n
     if (n >= kInvMinN && n <= kInvMaxN && *fail == 0) {
         float* buf = reinterpret_cast<float*>(pan);
         float2* p = reinterpret_cast<float2*>(sc.part);
-        const int rows = n <= 32 ? 32 : n <= 64 ? 64 : n <= 96 ? 96 : 120;
-        float2* x = reinterpret_cast<float2*>(buf + 12 * (rows + n));
-        const bool done = n <= 32   ? inverse_solve<4, 8>(F, ld, n, yf, buf, p, x)
-                          : n <= 64 ? inverse_solve<16, 4>(F, ld, n, yf, buf, p, x)
+        // rows (with padding) of the row groups, by size
+        const int rows = n <= 30 ? inv_stride(6) * 5 : n <= 60 ? inv_stride(18) * 4 : n <= 96 ? 48 * 2 : 60 * 2;
+        float2* x = reinterpret_cast<float2*>(buf + 2 * kPan * (rows + n));
+        const bool done = n <= 30   ? inverse_solve<6, 5>(F, ld, n, yf, buf, p, x)
+                          : n <= 60 ? inverse_solve<18, 4>(F, ld, n, yf, buf, p, x)
                           : n <= 96 ? inverse_solve<48, 2>(F, ld, n, yf, buf, p, x)
                                     : inverse_solve<60, 2>(F, ld, n, yf, buf, p, x);
         if (done) {

@@ -60,15 +60,19 @@ struct View {
     int W, H;
 };
 
-__device__ __forceinline__ bool valid_px(const View& v, int pix, float& z, float& nx, float& ny, float& nz)
+// A pixel's mask, depth and normal, all loads issued together (gating one on
+// the other would make them a chain); z = 0 where it is not valid.
+__device__ __forceinline__ float4 load_px(const View& v, int pix, bool in)
 {
-    if (!v.mask[pix]) return false;
-    z = v.depth[pix];
-    if (!(z > 0.f) || !isfinite(z)) return false;
-    nx = v.normals[3 * pix];
-    ny = v.normals[3 * pix + 1];
-    nz = v.normals[3 * pix + 2];
-    return isfinite(nx) && isfinite(ny) && isfinite(nz);
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (in) {
+        const uint8_t m = __ldg(v.mask + pix);
+        const float* n = v.normals + 3 * (size_t)pix;
+        x = make_float4(__ldg(v.depth + pix), __ldg(n), __ldg(n + 1), __ldg(n + 2));
+        const bool ok = m != 0 && x.x > 0.f && isfinite(x.x) && isfinite(x.y) && isfinite(x.z) && isfinite(x.w);
+        if (!ok) x.x = 0.f;
+    }
+    return x;
 }
 
 // One direction per half of the grid: CTAs [0, nb_a) take source frame a and
@@ -87,43 +91,55 @@ __global__ void __launch_bounds__(kNoAllocThreads) pair_energy_kernel(
     const View& dst = rev ? va : vb;
     const bt::PairK& K = rev ? xf.kba : xf.kab;
     const int blk = rev ? blockIdx.x - nb_a : blockIdx.x;
-    float e = 0.f, cnt = 0.f;
+    float e = 0.f;
+    int cnt = 0;
     const int HW = src.W * src.H;
+    // the sources of the thread's pixels, their projections, then their
+    // targets, each with all loads in flight
+    float4 ps[kNoAllocPix], pt[kNoAllocPix];
+    float2 qxy[kNoAllocPix], uv[kNoAllocPix];
+    float qz[kNoAllocPix];
 #pragma unroll
     for (int k = 0; k < kNoAllocPix; ++k) {
         const int pix = blk * kNoAllocBlockPix + k * kNoAllocThreads + threadIdx.x;
-        if (pix >= HW) continue;
-        float z, nx, ny, nz;
-        if (!valid_px(src, pix, z, nx, ny, nz)) continue;
+        ps[k] = load_px(src, pix, pix < HW);
+    }
+#pragma unroll
+    for (int k = 0; k < kNoAllocPix; ++k) {
+        const int pix = blk * kNoAllocBlockPix + k * kNoAllocThreads + threadIdx.x;
         const int u = pix % src.W, v = pix / src.W;
+        const float z = ps[k].x;
         // pi_D^-1(x) as the frame preparation of the graph path computes it
         const float px = ((float)u - src.cx) * z * src.ifx;
         const float py = ((float)v - src.cy) * z * src.ify;
-        float2 qxy, uv;
-        float qz;
         int iu, iv;
-        if (!bt::assoc_project(K, px, py, z, qxy, qz, uv, iu, iv)) continue;
-        const int tp = iv * dst.W + iu;
-        float tz, tnx, tny, tnz;
-        if (!valid_px(dst, tp, tz, tnx, tny, tnz)) continue;
+        const bool ok = bt::assoc_project(K, px, py, z, qxy[k], qz[k], uv[k], iu, iv) && z > 0.f;
+        pt[k] = load_px(dst, iv * dst.W + iu, ok);
+    }
+#pragma unroll
+    for (int k = 0; k < kNoAllocPix; ++k) {
+        if (!(pt[k].x > 0.f)) continue;
         float2 txy, dxy, nxy;
         float dz, nzr;
-        if (!bt::assoc_distance(K, uv, tz, qxy, qz, dmax2, txy, dxy, dz)) continue;
-        if (!bt::assoc_normal(K, nx, ny, nz, tnx, tny, tnz, cmin, nxy, nzr)) continue;
+        if (!bt::assoc_distance(K, uv[k], pt[k].x, qxy[k], qz[k], dmax2, txy, dxy, dz)) continue;
+        if (!bt::assoc_normal(K, ps[k].y, ps[k].z, ps[k].w, pt[k].y, pt[k].z, pt[k].w, cmin, nxy, nzr)) continue;
         const float r = bt::assoc_residual(nxy, nzr, dxy, dz);
         const float ar = fabsf(r);
         e += ar <= hub ? 0.5f * r * r : hub * (ar - 0.5f * hub);
-        cnt += 1.f;
+        cnt += 1;
     }
-    double de = e, dc = cnt;
+    // a warp-wide FP64 instruction takes 64 cycles of its sub-partition: only
+    // warps with an association add their energies up
+    double de = 0.0;
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if (cnt > 0) {
+        de = e;
 #pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {
-        de += __shfl_xor_sync(0xffffffffu, de, o);
-        dc += __shfl_xor_sync(0xffffffffu, dc, o);
+        for (int o = 16; o >= 1; o >>= 1) de += __shfl_xor_sync(0xffffffffu, de, o);
     }
     if ((threadIdx.x & 31) == 0) {
         red[threadIdx.x >> 5][0] = de;
-        red[threadIdx.x >> 5][1] = dc;
+        red[threadIdx.x >> 5][1] = (double)cnt;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -140,24 +156,42 @@ __global__ void __launch_bounds__(kNoAllocThreads) pair_energy_kernel(
     }
     __syncthreads();
     if (!s_last) return;
-    // last CTA: fixed-order sum of every CTA's partial (deterministic)
+    // last CTA: fixed-order sum of every CTA's partial (deterministic), four
+    // partials a thread in flight
     __threadfence();
-    if (threadIdx.x < 32) {
-        double s0 = 0.0, s1 = 0.0;
-        for (int b = threadIdx.x; b < (int)gridDim.x; b += 32) {
-            s0 += __ldcg(&scr->partial[b][0]);
-            s1 += __ldcg(&scr->partial[b][1]);
+    double s0 = 0.0, s1 = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += 4 * kNoAllocThreads) {
+        double2 v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int at = b + q * kNoAllocThreads;
+            v[q] = at < (int)gridDim.x ? __ldcg(reinterpret_cast<const double2*>(scr->partial[at])) : make_double2(0.0, 0.0);
         }
 #pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) {
-            s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        for (int q = 0; q < 4; ++q) {
+            s0 += v[q].x;
+            s1 += v[q].y;
         }
-        if (threadIdx.x == 0) {
-            out[0] = lambda * s0;
-            out[1] = s1;
-            scr->counter = 0u;
+    }
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) {
+        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        red[threadIdx.x >> 5][0] = s0;
+        red[threadIdx.x >> 5][1] = s1;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s0 = s1 = 0.0;
+        for (int w = 0; w < kNoAllocThreads / 32; ++w) {
+            s0 += red[w][0];
+            s1 += red[w][1];
         }
+        out[0] = lambda * s0;
+        out[1] = s1;
+        scr->counter = 0u;
     }
 }
 
