@@ -406,14 +406,27 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
     // energies of the iteration, by one warp: at once when there is no
     // system to solve, else while warp 0 is busy alone
     const bool solves = kFull && n > 0 && status0 == 0;
-    auto write_costs = [&]() {
-        double ed = 0.0, es = 0.0, cnt = 0.0;
-        for (int u = lane; u < U; u += 32) {
-            const double* o = a.upairblk + (size_t)u * kUPairBlk;
-            ed += __ldcg(o + 90);
-            es += __ldcg(o + 91);
-            cnt += __ldcg(o + 92);
+    double ed = 0.0, es = 0.0, cnt = 0.0;
+    auto add_costs = [&]() {
+        // three pairs a lane at a time, their loads in flight together
+        for (int u0 = lane; u0 < U; u0 += 96) {
+            double x[3][3];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const double* o = a.upairblk + (size_t)min(u0 + 32 * q, U - 1) * kUPairBlk;
+#pragma unroll
+                for (int e = 0; e < 3; ++e) x[q][e] = __ldcg(o + 90 + e);
+            }
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                if (u0 + 32 * q >= U) break;
+                ed += x[q][0];
+                es += x[q][1];
+                cnt += x[q][2];
+            }
         }
+    };
+    auto store_costs = [&]() {
 #pragma unroll
         for (int off = 16; off >= 1; off >>= 1) {
             ed += __shfl_xor_sync(0xffffffffu, ed, off);
@@ -426,6 +439,10 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
             a.costs[iter * 4 + 2] = es;
             a.costs[iter * 4 + 3] = cnt;
         }
+    };
+    auto write_costs = [&]() {
+        add_costs();
+        store_costs();
     };
     if (!solves) {
         if (tid < 32) write_costs();
@@ -443,45 +460,58 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
     double* shift = colb + ldlt_pan_doubles(n);
     int* node_of = reinterpret_cast<int*>(shift + ldlt_shift_doubles(n));
     double* scratch = reinterpret_cast<double*>(node_of + kMaxNodes);      // 264 doubles
-    __shared__ int s_fail;
+    __shared__ int s_fail, free_of[kMaxNodes];
+    if (tid < N) free_of[tid] = pf.free_idx;
     if (tid < N && pf.free_idx >= 0) node_of[pf.free_idx] = tid;
     if (tid < 12 * N) ps[tid] = pf.pose0;
     if (tid + nt < 12 * N) ps[tid + nt] = pf.pose1;
     if (tid == 0) s_fail = 0;
     __syncthreads();
-    // Assembly straight from the pair blocks in L2.  What it costs is L2
-    // round trips and FP64 adds, so each thread has up to twelve loads in
-    // flight (cycles, against staging the blocks in shared memory first: ten
-    // nodes 7.4 k -> 7.5 k; twenty nodes, whose blocks do not fit there,
-    // 59.6 k -> 28.6 k, and no staging room is needed).
+    // Assembly straight from the pair blocks in L2: no room for staging them
+    // is needed, and what it costs is L2 round trips, FP64 adds and index
+    // arithmetic, so loads go out in batches and a warp takes a whole block at
+    // a time (one entry a thread, each with its own square root and divisions
+    // for the block's place: ten nodes 7.5 k cycles, twenty 29 k).
     const int cost_warp = (nt >> 5) - 1;
-    constexpr int kFly = 12;
+    constexpr int kFly = 12, kBlocks = 6;
     const double* blk = a.upairblk;
-    // off-diagonal blocks (fa > fb)
-    const int nob = nf * (nf - 1) / 2;
-    for (int q0 = tid; q0 < nob * 36; q0 += kFly * nt) {
-        double v[kFly];
-        int at[kFly];
+    // off-diagonal blocks: O_ab with a < b is the transpose of block (b, a) of
+    // the lower triangle (free nodes are numbered in the order of the nodes);
+    // lanes 0-17 hold two neighbouring entries of a row each
+    {
+        const int nw = nt >> 5;
+        const int rr = 2 * lane / 6, cc = 2 * lane % 6;
+        int A = 0, B = 1 + warp;      // pair of index `warp`, then every nw-th
+        auto settle = [&]() {
+            while (A < N - 1 && B >= N) {
+                ++A;
+                B += A + 1 - N;
+            }
+        };
+        settle();
+        for (int u0 = warp; u0 < U; u0 += kBlocks * nw) {
+            double2 v[kBlocks];
+            int fa[kBlocks], fb[kBlocks];
 #pragma unroll
-        for (int x = 0; x < kFly; ++x) {
-            const int q = q0 + x * nt;
-            at[x] = -1;
-            if (q >= nob * 36) continue;
-            const int b = q / 36, e = q % 36, rr = e / 6, cc = e % 6;
-            // b = fa (fa - 1) / 2 + fb with fb < fa: fa from the square root,
-            // corrected by one step either way (b < 253, exact in FP32)
-            int fa = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)b)) * 0.5f);
-            if (fa * (fa - 1) / 2 > b) --fa;
-            if (fa * (fa + 1) / 2 <= b) ++fa;
-            const int fb = b - fa * (fa - 1) / 2;
-            const int A = node_of[fa], B = node_of[fb];
-            const int u = A < B ? upair_index(A, B, N) : upair_index(B, A, N);
-            at[x] = (6 * fa + rr) * ld + 6 * fb + cc;
-            v[x] = __ldcg(blk + (size_t)u * kUPairBlk + 42 + (A < B ? rr * 6 + cc : cc * 6 + rr));
+            for (int x = 0; x < kBlocks; ++x) {
+                const int u = u0 + x * nw;
+                fa[x] = fb[x] = -1;
+                if (u < U) {
+                    fa[x] = free_of[A];
+                    fb[x] = free_of[B];
+                    B += nw;
+                    settle();
+                }
+                v[x] = __ldcg(reinterpret_cast<const double2*>(blk + (size_t)min(u, U - 1) * kUPairBlk + 42) + min(lane, 17));
+            }
+#pragma unroll
+            for (int x = 0; x < kBlocks; ++x)
+                if (lane < 18 && fa[x] >= 0 && fb[x] >= 0) {
+                    double* to = H + (6 * fb[x] + cc) * ld + 6 * fa[x] + rr;
+                    to[0] = v[x].x;
+                    to[ld] = v[x].y;
+                }
         }
-#pragma unroll
-        for (int x = 0; x < kFly; ++x)
-            if (at[x] >= 0) H[at[x]] = v[x];
     }
     // diagonal blocks and gradient: one thread per (free node, value), values
     // 0-20 the unique block entries, 21-26 the gradient entries (all the
@@ -651,8 +681,9 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
             cf[4 * lane + 1 + warp] = c;
             if (warp == 0) cf[4 * lane] = fma(xi[5], xi[5], fma(xi[4], xi[4], xi[3] * xi[3]));
         }
-        if (costs_due && warp == cost_warp) write_costs();
+        if (costs_due && warp == cost_warp) add_costs();
         __syncthreads();
+        if (costs_due && warp == cost_warp) store_costs();
         for (int q = tid; q < 12 * nf; q += nt) {
             // rotation entries (f, r, c < 3) first, then the translations
             int f, r, c;
