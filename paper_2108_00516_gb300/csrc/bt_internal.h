@@ -3,10 +3,9 @@
 // Layout in HBM (all device buffers are owned by a bt_graph):
 //   per stored frame (storage precision P of the graph: FP32, BF16 or FP16)
 //     tgt   [H*W]  (z, nx, ny, nz) per pixel, read by the projective gather
-//                  (Eq. 3).  FP32: float4, z = 0 where the pixel cannot be a
-//                  dense target (not masked / no depth / no normal), 16 B.
-//                  BF16/FP16: 4 x 16 bit (z - zref, nx, ny, nz), z - zref =
-//                  NaN where invalid, 8 B; zref = the frame's mean valid depth
+//                  (Eq. 3), z = NaN where the pixel cannot be a dense target
+//                  (not masked / no depth / no normal).  FP32: float4, 16 B.
+//                  BF16/FP16: 4 x 16 bit (z - zref, nx, ny, nz), 8 B; zref = the frame's mean valid depth
 //     src_p [M]    back-projected source points of the M valid masked pixels,
 //                  increasing pixel order: float4 (px, py, pz, 0) or
 //                  4 x 16 bit (px, py, pz - zref, 0)
@@ -32,12 +31,10 @@ namespace bt {
 constexpr int kThreads = 256;                 // reduce CTAs, sparse CTAs, prep CTAs
 constexpr int kPixPerThread = 4;              // prep
 // Dense residual CTA shapes (threads x source pixels per thread); the tile of
-// a CTA is their product.  A thread takes its pixels of one target in
-// batches of up to 4 (the gathers of a batch are in flight together) and
-// reduces its sums across the warp once per target, so more pixels per
-// thread spread that reduction over more pixel pairs.  Shape
-// BT_SINGLE_GRAPH_SHAPE (256 x 4) is the single-graph path's; the batched
-// solver's autotuner picks among all of them.
+// a CTA is their product.  A warp reduces its sums across its lanes once per
+// target, so more pixels per thread spread that reduction over more pixel
+// pairs.  Shape BT_SINGLE_GRAPH_SHAPE (256 x 4) is the single-graph path's;
+// the batched solver's autotuner picks among all of them.
 constexpr int kNumShapes = 6;     // BT_NUM_SHAPES
 constexpr int kSingleShape = BT_SINGLE_GRAPH_SHAPE;   // CTA shape of the single-graph solve (bt_solve)
 constexpr int kShapeThreads[kNumShapes] = {128, 128, 256, 64, 64, 32};

@@ -7,8 +7,8 @@
 //   reduce_kernel   one CTA per unordered node pair turns the FP32 partials of
 //                   both directions and the pair's correspondence set into
 //                   FP64 6x6 blocks; the last CTA to finish assembles the
-//                   normal equations over the free nodes, runs the FP64
-//                   Cholesky solve and the FP64 se(3) update.
+//                   normal equations over the free nodes, solves them
+//                   (bt_ldlt.h) and runs the FP64 se(3) update.
 //
 // Perturbations are right perturbations, T_i <- T_i exp(d_i) (see
 // bt_residual.cu for why every iterate equals the left-perturbation one).
@@ -366,8 +366,9 @@ __device__ double se3_exp_entry(const double* xi, const double* cf, int r, int c
 }
 
 // Last CTA: energies, then (full) assembly of H and g over the free nodes,
-// the solve of H dx = -g (square-root-free Cholesky in double-float
-// arithmetic, bt_ldlt.h; or PCG, the paper's inner solver, in FP64), and finally
+// the solve of H dx = -g (FP32 inverse with double-float corrections or
+// double-float Cholesky, bt_ldlt.h; or PCG, the paper's inner solver, in FP64),
+// and finally
 // T <- T exp(dx).
 // The first global reads of the last CTA, issued by every CTA of the reduce
 // kernel before its pair stage: the last CTA is only known after the
