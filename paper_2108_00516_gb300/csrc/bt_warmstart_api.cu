@@ -32,8 +32,8 @@ struct bt_warmstart {
     int64_t n_points = 0, cap_points = 0;
     int n_samples = 0, cap_samples = 0;
     // launch scratch
-    DevBuf ids, y, maxima, cache, rec, grad, loss;
-    DevBuf app_samples, app_y, app_maxima, app_graphs, app_scratch, app_status, app_items;
+    DevBuf ids, out, cache, rec, grad, loss;             // out: pooled maxima of every set, then its outputs
+    DevBuf app_samples, app_out, app_graphs, app_scratch, app_status, app_items;
     PinBuf pin_app, pin_status;   // staging of the apply tables and the per-graph status
     // fault word of the forward pass (mapped pinned host memory: the kernel
     // writes it, the host reads it after the call's synchronisation)
@@ -53,8 +53,8 @@ struct bt_warmstart {
     ~bt_warmstart()
     {
         if (stream) cudaStreamSynchronize(stream);
-        for (DevBuf* b : {&master, &wb, &m, &v, &pool_p, &pool_q, &samples, &stage, &items, &ids, &y, &maxima, &cache, &rec,
-                          &grad, &loss, &app_samples, &app_y, &app_maxima, &app_graphs, &app_scratch, &app_status,
+        for (DevBuf* b : {&master, &wb, &m, &v, &pool_p, &pool_q, &samples, &stage, &items, &ids, &out, &cache, &rec,
+                          &grad, &loss, &app_samples, &app_out, &app_graphs, &app_scratch, &app_status,
                           &app_items})
             b->release();
         pin_app.release();
@@ -65,6 +65,11 @@ struct bt_warmstart {
 };
 
 namespace {
+
+// A forward pass's scratch and outputs in one buffer: the pooled maxima of n
+// sets, then their outputs.
+size_t out_bytes(int n) { return W::pool_bytes(n) + sizeof(float) * W::kOut * (size_t)n; }
+float* outputs(const DevBuf& b, int n) { return reinterpret_cast<float*>(b.as<char>() + W::pool_bytes(n)); }
 
 // Grows a device buffer to `bytes`, keeping its first `keep` bytes.
 int grow(DevBuf& b, size_t bytes, size_t keep, cudaStream_t s, void** old_out = nullptr)
@@ -147,8 +152,7 @@ int gradient_pass(bt_warmstart* ws, const int32_t* ids, int n)
     int st = upload_ids(ws, ids, n);
     if (st != BT_OK) return st;
     cudaStream_t s = ws->stream;
-    BT_CUDA(ws->y.ensure(sizeof(float) * W::kOut * (size_t)n), "alloc y");
-    BT_CUDA(ws->maxima.ensure(W::pool_bytes(n)), "alloc pooled features");
+    BT_CUDA(ws->out.ensure(out_bytes(n)), "alloc outputs");
     BT_CUDA(ws->cache.ensure(sizeof(W::Cache) * (size_t)n), "alloc cache");
     BT_CUDA(ws->rec.ensure(sizeof(W::BwdRec) * (size_t)n), "alloc gradient contributions");
     BT_CUDA(ws->grad.ensure(sizeof(float) * W::kNumParams), "alloc gradient");
@@ -156,7 +160,7 @@ int gradient_pass(bt_warmstart* ws, const int32_t* ids, int n)
     const W::Net net = ws->net();
     const W::Sample* smp = ws->samples.as<W::Sample>();
     const int* d_ids = ws->ids.as<int>();
-    BT_CUDA(W::launch_forward(net, smp, d_ids, n, ws->maxima.as<unsigned long long>(), ws->y.as<float>(),
+    BT_CUDA(W::launch_forward(net, smp, d_ids, n, ws->out.as<unsigned long long>(), outputs(ws->out, n),
                               ws->cache.as<W::Cache>(), s),
             "launch forward");
     BT_CUDA(W::launch_backward(net, smp, d_ids, n, ws->cache.as<W::Cache>(), ws->rec.as<W::BwdRec>(),
@@ -226,8 +230,7 @@ int enqueue_apply(bt_warmstart* ws, bt_graph* const* gs, int n_graphs, double* c
     const int S = (int)smp.size();
     BT_CUDA(ws->app_samples.ensure(sizeof(W::Sample) * (size_t)std::max(S, 1)), "alloc samples");
     BT_CUDA(ws->app_items.ensure(sizeof(W::PrepItem) * (size_t)std::max(S, 1)), "alloc items");
-    BT_CUDA(ws->app_y.ensure(sizeof(float) * W::kOut * (size_t)std::max(S, 1)), "alloc outputs");
-    BT_CUDA(ws->app_maxima.ensure(W::pool_bytes(std::max(S, 1))), "alloc pooled features");
+    BT_CUDA(ws->app_out.ensure(out_bytes(std::max(S, 1))), "alloc outputs");
     BT_CUDA(ws->app_scratch.ensure(sizeof(double) * W::kAvgScratch * (size_t)std::max(S, 1)), "alloc scratch");
     BT_CUDA(ws->app_graphs.ensure(sizeof(W::AvgGraph) * (size_t)n_graphs), "alloc graphs");
     BT_CUDA(ws->app_status.ensure(sizeof(int) * (size_t)n_graphs), "alloc status");
@@ -239,7 +242,7 @@ int enqueue_apply(bt_warmstart* ws, bt_graph* const* gs, int n_graphs, double* c
         a.n_free = g->args.n_free;
         a.nodes = g->args.nodes;
         a.edges = g->args.edges;
-        a.y = ws->app_y.as<float>() + (size_t)first[k] * W::kOut;
+        a.y = outputs(ws->app_out, S) + (size_t)first[k] * W::kOut;
         a.smp = ws->app_samples.as<W::Sample>() + first[k];
         a.pose = pose[k];
         a.scratch = ws->app_scratch.as<double>() + (size_t)first[k] * W::kAvgScratch;
@@ -277,7 +280,7 @@ int launch_apply(bt_warmstart* ws, int S, int n_graphs, int max_free, cudaStream
 {
     W::Sample* d_smp = ws->app_samples.as<W::Sample>();
     BT_CUDA(W::launch_prep(d_smp, ws->app_items.as<W::PrepItem>(), S, s), "launch prep");
-    BT_CUDA(W::launch_forward(ws->net(), d_smp, nullptr, S, ws->app_maxima.as<unsigned long long>(), ws->app_y.as<float>(),
+    BT_CUDA(W::launch_forward(ws->net(), d_smp, nullptr, S, ws->app_out.as<unsigned long long>(), outputs(ws->app_out, S),
                               nullptr, s),
             "launch forward");
     BT_CUDA(W::launch_average(ws->app_graphs.as<W::AvgGraph>(), n_graphs, max_free, s), "launch average");
@@ -595,12 +598,11 @@ int bt_warmstart_predict(bt_warmstart* ws, const int32_t* ids, int32_t n, float*
     if (n == 0) return BT_OK;
     st = upload_ids(ws, ids, n);
     if (st != BT_OK) return st;
-    BT_CUDA(ws->y.ensure(sizeof(float) * W::kOut * (size_t)n), "alloc y");
-    BT_CUDA(ws->maxima.ensure(W::pool_bytes(n)), "alloc pooled features");
+    BT_CUDA(ws->out.ensure(out_bytes(n)), "alloc outputs");
     BT_CUDA(W::launch_forward(ws->net(), ws->samples.as<W::Sample>(), ws->ids.as<int>(), n,
-                              ws->maxima.as<unsigned long long>(), ws->y.as<float>(), nullptr, ws->stream),
+                              ws->out.as<unsigned long long>(), outputs(ws->out, n), nullptr, ws->stream),
             "launch forward");
-    BT_CUDA(cudaMemcpyAsync(y_out, ws->y.p, sizeof(float) * W::kOut * (size_t)n, cudaMemcpyDeviceToHost, ws->stream),
+    BT_CUDA(cudaMemcpyAsync(y_out, outputs(ws->out, n), sizeof(float) * W::kOut * (size_t)n, cudaMemcpyDeviceToHost, ws->stream),
             "read outputs");
     BT_CUDA(cudaStreamSynchronize(ws->stream), "bt_warmstart_predict: synchronize");
     return take_fault(ws, "bt_warmstart_predict");
