@@ -1,6 +1,6 @@
 // bt_ldlt.h -- solve of a symmetric positive-definite FP64 system H x = y by
 // one CTA of 256 threads: by an FP32 inverse and corrections from the
-// double-float residual (18 .. 120 unknowns), or, for other sizes and where
+// double-float residual (up to 120 unknowns), or, for larger ones and where
 // the corrections do not settle, by the square-root-free Cholesky
 // factorisation H = L D L^T with a one-panel look-ahead (forward substitution
 // L z = y carried along), D w = z, and a blocked back substitution L^T x = w.
@@ -200,7 +200,7 @@ struct LdltNoIdle {
 
 // Systems that are solved by their FP32 inverse: its entries stay in the
 // threads' registers, and its panels have to fit the factorisation's.
-constexpr int kInvMinN = 18, kInvMaxN = 120;
+constexpr int kInvMaxN = 120;
 
 #ifdef __CUDACC__
 // H x = b by the FP32 inverse W of the scaled system and corrections of x from
@@ -595,13 +595,14 @@ __device__ __forceinline__ bool ldlt_solve(double* __restrict__ H, int ld, int n
         for (int i = lane; i < n; i += 32) yf[i] = ff_from_f64(y[i], shift[i] + e);
     }
     __syncthreads();
-    if (n >= kInvMinN && n <= kInvMaxN && *fail == 0) {
+    if (n <= kInvMaxN && *fail == 0) {
         float* buf = reinterpret_cast<float*>(pan);
         float2* p = reinterpret_cast<float2*>(sc.part);
         // rows (with padding) of the row groups, by size
-        const int rows = n <= 30 ? inv_stride(6) * 5 : n <= 60 ? inv_stride(18) * 4 : n <= 96 ? 48 * 2 : 60 * 2;
+        const int rows = n <= 12 ? inv_stride(6) * 2 : n <= 30 ? inv_stride(6) * 5 : n <= 60 ? inv_stride(18) * 4 : n <= 96 ? 48 * 2 : 60 * 2;
         float2* x = reinterpret_cast<float2*>(buf + 2 * kPan * (rows + n));
-        const bool done = n <= 30   ? inverse_solve<6, 5>(F, ld, n, yf, buf, p, x)
+        const bool done = n <= 12   ? inverse_solve<6, 2>(F, ld, n, yf, buf, p, x)
+                          : n <= 30 ? inverse_solve<6, 5>(F, ld, n, yf, buf, p, x)
                           : n <= 60 ? inverse_solve<18, 4>(F, ld, n, yf, buf, p, x)
                           : n <= 96 ? inverse_solve<48, 2>(F, ld, n, yf, buf, p, x)
                                     : inverse_solve<60, 2>(F, ld, n, yf, buf, p, x);
