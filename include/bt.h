@@ -193,7 +193,7 @@ int bt_get_poses(const bt_graph* g, double* poses);
  * IV-D over the active nodes -- per iteration: dense association and
  * point-to-plane residuals for every ordered pair, Huber point-to-point
  * residuals for every correspondence set, reduction into 6x6 blocks,
- * assembly of the normal equations over the non-fixed nodes, FP64 Cholesky
+ * assembly of the normal equations over the non-fixed nodes, their exact
  * solve, FP64 se(3) update -- then evaluates E at the final poses.  The new
  * poses are stored in the graph (the memory write-back of Sec. IV-D) and, if
  * poses_out != NULL, copied to it (n_active x 16 doubles, host).  rep may be

@@ -17,13 +17,14 @@
 // value inside the FP32 exponent range).
 // Error of the solution against an 80-bit one, relative to its largest entry
 // (60 Gauss-Newton systems, worst of each size): inverse and corrections
-// 4e-14 .. 1.5e-13 for 24 .. 120 unknowns, factorisation 8e-13; an FP64
-// factorisation with pivots' reciprocals good to 1e-12: 7e-13 .. 2.5e-12.
-// Measured (one CTA, cycles, whole solve, inverse against factorisation): n =
-// 18: 9.8 k against 9.0 k, n = 54: 23 k against 28 k, n = 114: 104 k against
-// 104 k of which 14 k are the back substitution's; FP64 factorisation: 13 k,
-// 55 k, 236 k.  One pivot a step instead of six, without the redundant 6 x 6
-// factorisations: 32 k at n = 54, 135 k at n = 114.
+// 3e-14 .. 1.5e-13 for 18 .. 120 unknowns, factorisation up to 3.6e-13 there
+// and 6e-13 at 138; an FP64 factorisation with pivots' reciprocals good to
+// 1e-12: 7e-13 .. 2.5e-12.
+// Measured in the solve kernel (cycles of one solve, inverse against
+// factorisation with back substitution): n = 6: 8.0 k against 10.7 k, n = 18:
+// 11.0 k against 16.5 k, n = 54: 24.4 k against 36.1 k, n = 114: 106 k against
+// 136 k.  One pivot a step instead of six, without the redundant 6 x 6
+// factorisations: 33 k at n = 54, 138 k at n = 114.
 #pragma once
 
 #include "bt_internal.h"

@@ -172,7 +172,8 @@ __device__ void eigenvectors4_f32(float (&A)[4][4], float (&V)[4][4])
 // each of which shrinks the error by the single-precision error of V over the
 // gap to the next eigenvalue (about 1e-6: three corrections).  A correction is
 // ~46 FP64 instructions; the all-FP64 Jacobi iteration is ~9000, and on this
-// part a warp-wide FP64 instruction takes 64 cycles of its sub-partition.
+// part a warp-wide FP64 instruction takes 64 cycles of its sub-partition (fits
+// of 9 sets x 256 samples: 123 -> 24 us).
 // Returns false, v unset, where the gap is below 2e-6 of the largest entry or
 // the corrections do not settle: the caller then runs the FP64 iteration.
 __device__ bool top_eigenvector4_refined(const double (&N)[4][4], double (&v)[4])
