@@ -111,6 +111,10 @@ int reserve(bt_warmstart* ws, int64_t add_pts, int add_sets)
         int st = grow(ws->samples, sizeof(W::Sample) * (size_t)cap, sizeof(W::Sample) * (size_t)ws->n_samples, s);
         if (st != BT_OK) return st;
         ws->cap_samples = cap;
+        // outputs of the first few thousand sets with the room for the sets
+        // themselves: a mapping of megabytes (~0.2 ms) stays out of the first
+        // forward pass (larger ones grow it there)
+        if (!ws->out.p) BT_CUDA(ws->out.ensure(out_bytes(std::min(cap, 4096))), "alloc outputs");
     }
     return BT_OK;
 }
