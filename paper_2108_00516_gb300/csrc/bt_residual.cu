@@ -231,8 +231,11 @@ __global__ void __launch_bounds__(kThreads) prep_write_kernel(
                     reinterpret_cast<float4*>(tgt_v)[pix] =
                         ok ? make_float4(zz, nn.x, nn.y, nn.z) : make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
                 } else {
+                    // nor can one much nearer than the mean depth whose offset
+                    // comes back (decode_target) as a depth that is not positive
                     ushort4 t;
-                    t.x = ok ? to16<P>(zz - zref) : nan16<P>();
+                    const unsigned short dz = to16<P>(zz - zref);
+                    t.x = ok && zref + from16<P>(dz) > 0.f ? dz : nan16<P>();
                     t.y = ok ? to16<P>(nn.x) : (unsigned short)0;
                     t.z = ok ? to16<P>(nn.y) : (unsigned short)0;
                     t.w = ok ? to16<P>(nn.z) : (unsigned short)0;
