@@ -856,10 +856,13 @@ __global__ void __launch_bounds__(kBwdThreads)
         const float4 xa = *reinterpret_cast<const float4*>(sxr + ch * 8);
         const float2 xb = *reinterpret_cast<const float2*>(sxr + ch * 8 + 4);
         const float xc[6] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y};
-        const float w = z1_unit(w1, b1, xc) > 0.f ? sdz2[ch] * w2[q] : 0.f;
+        // added only where the unit is active: the row's features need not be
+        // finite where it is not (a NaN point's layer-1 outputs are all zero)
+        const float d = sdz2[ch], w = d * w2[q];
+        const bool on = z1_unit(w1, b1, xc) > 0.f && d != 0.f;
 #pragma unroll
-        for (int k = 0; k < 6; ++k) a[k] = __fmaf_rn(w, xc[k], a[k]);
-        a[6] += w;
+        for (int k = 0; k < 6; ++k) a[k] = on ? __fmaf_rn(w, xc[k], a[k]) : a[k];
+        a[6] = on ? a[6] + w : a[6];
     }
 #pragma unroll
     for (int k = 0; k < 7; ++k) spart[seg][j][k] = a[k];
@@ -966,7 +969,7 @@ __global__ void __launch_bounds__(kSumThreads, 1)
                     const int s = s0 + u * kSumGroups;
                     const float* R = reinterpret_cast<const float*>(rec + min(s, n - 1));
                     v[u] = s < n ? __ldcg(R + at) : 0.f;
-                    f[u] = fac >= 0 ? __ldcg(R + fac) : 1.f;
+                    f[u] = s >= n ? 0.f : fac >= 0 ? __ldcg(R + fac) : 1.f;
                 }
 #pragma unroll
                 for (int u = 0; u < 8; ++u) a = __fmaf_rn(v[u], f[u], a);
