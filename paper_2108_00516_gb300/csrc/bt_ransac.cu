@@ -265,11 +265,12 @@ __device__ void fit_from_moments(const double (&S)[3][3], const double (&pc)[3],
 }
 
 // x / 3: the product with the rounded reciprocal, corrected by its exact
-// remainder (a full FP64 division is ~10 times as many instructions).
+// remainder (a full FP64 division is ~10 times as many instructions).  The
+// remainder of an infinite product is NaN: the product is the quotient then.
 __device__ __forceinline__ double third(double x)
 {
-    const double q = x * (1.0 / 3.0);
-    return fma(fma(-3.0, q, x), 1.0 / 3.0, q);
+    const double q = x * (1.0 / 3.0), r = fma(-3.0, q, x);
+    return r == r ? fma(r, 1.0 / 3.0, q) : q;
 }
 
 constexpr int kHypThreads = 32;      // one warp a CTA: the FP64 units of all SMs share the samples

@@ -1,6 +1,8 @@
 """Correspondences that are not finite: what they leave untouched stays
 finite.  A point p that is NaN takes no part in the maxima of the warm start's
-network (its layer-1 outputs are zero), so it has no part in the gradient."""
+network (its layer-1 outputs are zero), so it has no part in the gradient; a
+3-point sample with an infinite target point has no rotation and an infinite
+translation."""
 import numpy as np
 import pytest
 
@@ -70,3 +72,14 @@ def test_nan_point_has_no_part_in_the_gradient(bt, n, bad):
         a, b = g[offs[k]:offs[k + 1]].astype(np.float64), go[offs[k]:offs[k + 1]]
         assert np.isfinite(a).all(), name
         assert np.linalg.norm(a - b) <= 2e-3 * np.linalg.norm(b), name
+
+
+@pytest.mark.parametrize("value", [np.inf, -np.inf])
+def test_infinite_target_point(bt, value):
+    p = np.array([[0, 0, 0.5], [0.1, 0, 0.5], [0, 0.1, 0.5]], np.float32)
+    q = p.copy()
+    q[1, 0] = value
+    M, count = bt.ransac(p, q, hypotheses=16, seed=1, inlier_dist=0.01, refine=False)
+    assert count == 0 and np.array_equal(M[:3, :3], np.eye(3))
+    # the centroid's first component is infinite, the others as they are
+    assert M[0, 3] == value and np.abs(M[1:3, 3]).max() <= 4 * 2.0**-53
