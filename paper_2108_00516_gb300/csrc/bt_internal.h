@@ -73,10 +73,11 @@ struct Control {
     unsigned int counter;   // last-block detection of the reduce kernel
     int status;             // 0 ok, -4 singular (sticky for the solve)
     unsigned checked;       // BT_CHECKED builds: bits of the index checks that failed (kChk*)
-    int pad;
+    int declined;           // 1: an iteration's system was left to the factorisation (bt_ldlt.h)
     // SM clock cycles spent by the last CTA, summed over the solve's
-    // iterations: [0] gather + assembly, [1] factorisation (with forward
-    // substitution), [2] back substitution, [3] pose update + transforms
+    // iterations: [0] gather + assembly, [1] solve by the inverse, or
+    // factorisation with forward substitution, [2] its write-back, or back
+    // substitution, [3] pose update + transforms
     unsigned long long clk[4];
 };
 

@@ -1,30 +1,33 @@
 // bt_ldlt.h -- solve of a symmetric positive-definite FP64 system H x = y by
 // one CTA of 256 threads: by an FP32 inverse and corrections from the
-// double-float residual (up to 120 unknowns), or, for larger ones and where
-// the corrections do not settle, by the square-root-free Cholesky
-// factorisation H = L D L^T with a one-panel look-ahead (forward substitution
+// double-float residual, or, where the inverse declines (pivots too small or
+// corrections that do not settle), in FP64 by the square-root-free Cholesky
+// factorisation H = L D L^T with a one-column look-ahead (forward substitution
 // L z = y carried along), D w = z, and a blocked back substitution L^T x = w.
 // Used by the Gauss-Newton step of Sec. IV-D (bt_solve.cu) and by the learned
 // warm start's relative-pose averaging (bt_warmstart.cu).
 //
-// Arithmetic: the system, the right-hand side and the solution are pairs of
-// FP32 numbers h + l (double-float, 48 bits), on the FP32 pipes.  On GB300 a
-// dependent FP64 operation costs ~64 cycles or more and a warp-wide FP64
-// instruction holds its sub-partition's DP unit for ~64 cycles whatever the
-// number of active lanes; a double-float multiply-subtract is 12 FP32
-// instructions with a dependent chain of ~30 cycles.  The system is first
+// On GB300 a dependent FP64 operation costs ~64 cycles or more and a warp-wide
+// FP64 instruction holds its sub-partition's DP unit for ~64 cycles whatever
+// the number of active lanes.  The inverse therefore runs on the FP32 pipes,
+// and so do its corrections: there the system, the right-hand side and the
+// solution are pairs of FP32 numbers h + l (double-float, 48 bits), the system
 // scaled by powers of two to a diagonal in [1, 4) (exact, and it keeps every
-// value inside the FP32 exponent range).
+// value inside the FP32 exponent range).  The factorisation is arranged for
+// short dependency chains and for many lanes behind each FP64 instruction.
+//
+// Measured in the solve kernel (chains of correspondence sets, the diagonal
+// scaled away; cycles of one solve, inverse against factorisation): n = 6:
+// 7.6 k against 9.1 k, n = 18: 12.2 k against 16.1 k, n = 54: 25 k against 56 k,
+// n = 114: 80 k against 233 k, n = 138: 138 k against 366 k.  Trying the inverse
+// in vain costs 4.5 k, 22 k and about 90 k cycles at n = 6, 54 and 114.  One
+// pivot a step of the inverse instead of six: 33 k at n = 54, 138 k at n = 114.
 // Error of the solution against an 80-bit one, relative to its largest entry
-// (60 Gauss-Newton systems, worst of each size): inverse and corrections
-// 3e-14 .. 1.5e-13 for 18 .. 120 unknowns, factorisation up to 3.6e-13 there
-// and 6e-13 at 138; an FP64 factorisation with pivots' reciprocals good to
-// 1e-12: 7e-13 .. 2.5e-12.
-// Measured in the solve kernel (cycles of one solve, inverse against
-// factorisation with back substitution): n = 6: 8.0 k against 10.7 k, n = 18:
-// 11.0 k against 16.5 k, n = 54: 24.4 k against 36.1 k, n = 114: 106 k against
-// 136 k.  One pivot a step instead of six, without the redundant 6 x 6
-// factorisations: 33 k at n = 54, 138 k at n = 114.
+// (worst of the systems of 6 .. 138 unknowns with condition numbers in the
+// given range): where the inverse is taken, up to 1e3: 9e-13 (factorisation
+// 2e-11), 1e3 .. 1e4: 1e-11 (4e-10), 1e4 .. 1e5: 1e-11 (4e-10); where it
+// declines, 1e5 .. 9e5: 2e-8.  A factorisation in double-float numbers took
+// half the cycles of the FP64 one, but left errors of up to 9e-6 there.
 #pragma once
 
 #include "bt_internal.h"
@@ -71,37 +74,12 @@ __host__ __device__ __forceinline__ float2 ff_msub_acc(float2 c, float2 a, float
     return make_float2(s, ff_add_(w, ff_sub_(c.y, e)));
 }
 
-// a b, not renormalised.
-__host__ __device__ __forceinline__ float2 ff_mul_acc(float2 a, float2 b)
-{
-    const float p = ff_mul_(a.x, b.x);
-    float e = ff_fma_(a.x, b.x, -p);
-    e = ff_fma_(a.x, b.y, e);
-    return make_float2(p, ff_fma_(a.y, b.x, e));
-}
-
 __host__ __device__ __forceinline__ float2 ff_add(float2 a, float2 b)
 {
     const float s = ff_add_(a.x, b.x);
     const float v = ff_sub_(s, a.x);
     const float w = ff_add_(ff_sub_(a.x, ff_sub_(s, v)), ff_sub_(b.x, v));
     return ff_norm(s, ff_add_(w, ff_add_(a.y, b.y)));
-}
-
-// 1 / d, not renormalised: the hardware approximation r0 (relative error
-// below 2^-22) and its remainder e = 1 - d r0, as r0 (1 + e + e^2); relative
-// error below 2^-44.  The leading part is ready as soon as r0 is.
-__host__ __device__ __forceinline__ float2 ff_rcp(float2 d)
-{
-#ifdef __CUDA_ARCH__
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d.x));
-#else
-    const float r = 1.0f / d.x;
-#endif
-    float e = ff_fma_(-d.x, r, 1.0f);
-    e = ff_fma_(-d.y, r, e);
-    return make_float2(r, ff_mul_(r, ff_fma_(e, e, e)));
 }
 
 // Exponent field of an FP64 number (0 for zero and subnormal numbers).
@@ -167,60 +145,99 @@ __host__ __device__ __forceinline__ double ff_to_f64(float2 v, int k)
 // (256 threads), which needs r0 < n <= 256.
 constexpr int kLdltMaxN = 6 * (kMaxNodes - 1);
 static_assert(kLdltMaxN <= 256, "ldlt_solve: at most 256 unknowns for one 256-thread CTA");
-// Columns factorised between two barriers: one node's unknowns.
+// Unknowns eliminated between two barriers of the inverse: one node's.
 constexpr int kPan = 6;
-// Rows below the panel's own six that one warp takes through a panel.
-constexpr int kPanRows = 32 - kPan;
-static_assert((kLdltMaxN + 1 - kPan + kPanRows - 1) / kPanRows <= 8, "a panel's rows fit the CTA's eight warps");
+
+// Row groups of the inverse by size of the system: entries of a column in a
+// thread's registers (a multiple of six) and groups, one warp a group and
+// block of 32 columns.
+struct InvShape {
+    int rows, groups;
+};
+__host__ __device__ constexpr InvShape inv_shape(int n)
+{
+    return n <= 12 ? InvShape{6, 2} : n <= 30 ? InvShape{6, 5} : n <= 60 ? InvShape{18, 4} : n <= 96 ? InvShape{48, 2}
+         : n <= 120 ? InvShape{60, 2} : InvShape{138, 1};
+}
+static_assert(kLdltMaxN <= 138, "the inverse holds the largest system");
+__host__ __device__ constexpr int inv_stride(int kR) { return (kR + 3) & ~3; }      // of a row group, in floats
+// Two panels of six columns and six rows, the solution, the right-hand side.
+__host__ __device__ constexpr size_t inv_floats(int n)
+{
+    return 2 * kPan * (size_t)(inv_stride(inv_shape(n).rows) * inv_shape(n).groups + n) + 4 * (size_t)n;
+}
 
 // Shared-memory scratch of ldlt_solve for an n x n system.
 struct LdltScratch {
-    double* pan;    // [ldlt_pan_doubles(n)]: columns u and l = u / D of a panel by row, double-buffered (16-byte aligned)
-    int* shift;     // [2 ldlt_shift_doubles(n)]: power-of-two scaling of each row and of y, two work counters
-    double* part;   // [256]    partial dot products of the back substitution
+    double* work;   // [ldlt_work_doubles(n)], 16-byte aligned: the inverse's panels and vectors; the factorisation's
+                    // scaled look-ahead column, double-buffered [2][n], and (row, column) table of the trailing triangle
+    double* rD;     // [n]      1 / D_k
+    double* part;   // [256]    partial dot products
+    int* shift;     // [n + 1]  power-of-two scaling of each row and of y
 };
-__host__ __device__ constexpr size_t ldlt_pan_doubles(size_t n) { return 4 * kPan * (n + 1); }
-__host__ __device__ constexpr size_t ldlt_shift_doubles(size_t n) { return (n + 4) / 2; }
+__host__ __device__ constexpr size_t ldlt_work_doubles(int n)
+{
+    const size_t inv = (inv_floats(n) + 1) / 2, fac = 2 * (size_t)n + ((size_t)n * (n + 1) / 2 + 1) / 2;
+    return inv > fac ? inv : fac;
+}
+__host__ __device__ constexpr size_t ldlt_shift_doubles(size_t n) { return (n + 2) / 2; }
 
-// H: n x n (n a multiple of 6, at most kLdltMaxN) FP64 in shared memory,
-// row-major with leading dimension ld = n + 1, lower triangle filled;
-// overwritten (H and the scratch hold double-floats during the call).  y =
-// H + n ld: right-hand side, overwritten with x (FP64).  *fail (shared
-// memory, zero on entry) is set when a pivot is not positive; x is then
-// meaningless, and the caller reads *fail after the call (the call ends with
-// a barrier).  t_mid: every thread's clock after the factorisation.
-// idle(warp): called once by each of warps 1-7 while warp 0 alone runs the
-// first block of the back substitution (work the caller has for otherwise
-// idle warps; it must not touch H, y or the scratch, and is not called when
-// a pivot failed).  Returns whether idle was called for (false: the system
-// was solved by its FP32 inverse, without a time when warps are idle).  All
-// threads of the CTA (blockDim.x == 256) must call it.
+// H: n x n (n a multiple of 6, at most kLdltMaxN) in shared memory, row-major
+// with leading dimension ld = n + 1, lower triangle filled; the rest of it is
+// overwritten.  y: [n] right-hand side in shared memory, overwritten with x.
+// *fail (shared memory, zero on entry) is set when a pivot is not positive; x
+// is then meaningless, and the caller reads *fail after the call (the call
+// ends with a barrier).  inverse: whether to try the inverse first (a system
+// whose predecessor was declined will most often be declined too).  t_mid:
+// every thread's clock after the inverse's solve, or after the factorisation
+// and D w = z.  idle(warp): called once by each of warps 1-7 while warp 0
+// alone runs the first block of the back substitution (work the caller has for
+// otherwise idle warps; it must not touch H, y or the scratch, and is not
+// called when a pivot failed).  Returns whether the system was factorised, and
+// idle called for (false: solved by the inverse, without a time when warps are
+// idle).  All threads of the CTA (blockDim.x == 256) must call it.
 struct LdltNoIdle {
     __device__ void operator()(int) const {}
 };
 
-// Systems that are solved by their FP32 inverse: its entries stay in the
-// threads' registers, and its panels have to fit the factorisation's.
-constexpr int kInvMaxN = 120;
-
 #ifdef __CUDACC__
+// 1/d for a positive FP64 pivot: the hardware approximation (rcp.approx.f64,
+// relative error below 1e-6 on GB300) refined by one Newton step
+// r <- r + r (1 - d r), which leaves a relative error below 1e-12 (measured
+// on 1M pivots spanning 1e-6 .. 1e6) -- ample for a factorisation whose
+// results are compared at 1e-5, and two dependent FP64 operations shorter
+// than the correctly rounded reciprocal on the column chain.
+__device__ __forceinline__ double rcp_fp64(double d)
+{
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+    const double e = fma(-d, r, 1.0);
+    return fma(r, e, r);
+}
+
+// Trailing rows from which warp 4 joins the bulk update (see ldlt_solve).
+#ifndef BT_LDLT_WIDE_ROWS
+#define BT_LDLT_WIDE_ROWS 30
+#endif
+constexpr int kWideBulkRows = BT_LDLT_WIDE_ROWS;
+
 // H x = b by the FP32 inverse W of the scaled system and corrections of x from
-// its double-float residual, x += W (b - H x).  The scaled normal equations of
-// a pose graph in the object's frame have condition numbers of 20 .. 60, so W
-// is good to about 1e-6 and two corrections reach the accuracy of the
-// double-float residual, without the n dependent double-float pivots of the
-// factorisation below.  W is formed by Gauss-Jordan elimination in steps of
-// six unknowns, one barrier a step: lane = column, warps = column blocks x kG
-// row groups, kR entries of a column in a thread's registers (kR a multiple of
-// six, so that a panel's rows lie in one group); the panel (six columns, six
-// rows) of the next step goes through shared memory, and every thread
-// factorises the 6 x 6 pivot block for itself.
-// Returns false, F and b untouched, when a pivot is below 2^-10 (the diagonal
-// is in [1, 4)), so that the system may not be positive definite, or when the
-// corrections do not shrink by at least four each; the caller then factorises.
-// F: lower triangle, leading dimension ld; buf: 12 (inv_stride(kR) kG + n)
-// floats (16-byte aligned); part: kG n; x: n.
-__host__ __device__ constexpr int inv_stride(int kR) { return (kR + 3) & ~3; }                 // of a row group, in floats
+// its double-float residual, x += W (b - H x), until they settle (at most
+// eight).  The normal equations of dense graphs in the object's frame have
+// scaled condition numbers of 20 .. 60 (six graphs of 18 .. 138 unknowns;
+// chains of correspondence sets reach 1e3): there W is good to about 1e-6 and
+// two corrections reach the accuracy of the double-float residual, without the
+// n dependent pivots of the factorisation below.  W is formed by Gauss-Jordan
+// elimination in steps of six unknowns, one barrier a step: lane = column,
+// warps = column blocks x kG row groups, kR entries of a column in a thread's
+// registers (kR a multiple of six, so that a panel's rows lie in one group);
+// the panel (six columns, six rows) of the next step goes through shared
+// memory, and every thread factorises the 6 x 6 pivot block for itself.
+// Returns false when a pivot is below 2^-10 (the diagonal is in [1, 4)), so
+// that the system may not be positive definite, or when the corrections do not
+// shrink by at least four each; the caller then factorises.
+// F: upper triangle of the scaled system, leading dimension ld; buf: panels,
+// 12 (inv_stride(kR) kG + n) floats (16-byte aligned); part: kG n; x: n.
 template <int kR, int kG>
 __device__ __forceinline__ bool inverse_solve(const float2* __restrict__ F, int ld, int n, const float2* __restrict__ b,
                                               float* __restrict__ buf, float2* __restrict__ part,
@@ -255,7 +272,7 @@ __device__ __forceinline__ bool inverse_solve(const float2* __restrict__ F, int 
 #pragma unroll
         for (int r = 0; r < kS; ++r) {
             const int i = i0 + r;
-            w[r] = r < kR && i < n ? F[max(i, jc) * ld + min(i, jc)].x : 0.f;
+            w[r] = r < kR && i < n ? F[min(i, jc) * ld + max(i, jc)].x : 0.f;
         }
         publish(0, 0);
     }
@@ -387,13 +404,13 @@ __device__ __forceinline__ bool inverse_solve(const float2* __restrict__ F, int 
         if (active) {
             float2 s0 = g == 0 ? b[jc] : make_float2(0.f, 0.f), s1 = make_float2(0.f, 0.f);
             const int k1 = min(i0 + kR, n);
-            // H_jk: row j of the triangle up to the diagonal, column j below it
+            // H_jk: row k of the upper triangle up to column j, row j after it
             int k = i0;
             for (; k + 1 < k1; k += 2) {
-                s0 = ff_msub_acc(s0, F[max(k, jc) * ld + min(k, jc)], x[k]);
-                s1 = ff_msub_acc(s1, F[max(k + 1, jc) * ld + min(k + 1, jc)], x[k + 1]);
+                s0 = ff_msub_acc(s0, F[min(k, jc) * ld + max(k, jc)], x[k]);
+                s1 = ff_msub_acc(s1, F[min(k + 1, jc) * ld + max(k + 1, jc)], x[k + 1]);
             }
-            if (k < k1) s0 = ff_msub_acc(s0, F[max(k, jc) * ld + min(k, jc)], x[k]);
+            if (k < k1) s0 = ff_msub_acc(s0, F[min(k, jc) * ld + max(k, jc)], x[k]);
             if (j < n) part[g * n + j] = ff_add(s0, s1);
         }
         __syncthreads();
@@ -408,270 +425,230 @@ __device__ __forceinline__ bool inverse_solve(const float2* __restrict__ F, int 
     return false;
 }
 
-// The six values of row i of a panel buffer.
-__device__ __forceinline__ void pan_load(const float2* pan, int i, float2 (&v)[kPan])
-{
-    const float4* p = reinterpret_cast<const float4*>(pan + i * kPan);
-#pragma unroll
-    for (int q = 0; q < kPan / 2; ++q) {
-        const float4 x = p[q];
-        v[2 * q] = make_float2(x.x, x.y);
-        v[2 * q + 1] = make_float2(x.z, x.w);
-    }
-}
-
-__device__ __forceinline__ void pan_store(float2* pan, int i, const float2 (&v)[kPan])
-{
-    float4* p = reinterpret_cast<float4*>(pan + i * kPan);
-#pragma unroll
-    for (int q = 0; q < kPan / 2; ++q) p[q] = make_float4(v[2 * q].x, v[2 * q].y, v[2 * q + 1].x, v[2 * q + 1].y);
-}
-
-// Warp w's share of the panel of columns c0 .. c0 + 5: lanes 0-5 hold the
-// panel's own rows (the same in every warp: the six pivots are formed by
-// each warp for itself, which saves a barrier and a shared-memory round trip
-// inside the panel), lanes 6-31 the rows c0 + 6 + 26 w onwards (row n is the
-// right-hand side).  First the previous panel (pu, pl; NULL for the first) is
-// applied to these six columns, then per column the pivot and the panel's
-// other entries of its row come by shuffle and every lane forms 1 / D
-// itself.  On the chain from pivot to pivot lie one shuffle, the reciprocal
-// and two products; everything that renormalises runs beside it.  Written:
-// u and l by row, L transposed into the upper triangle, w = z / D (the l of
-// row n) over the finished entries of y.
-__device__ __forceinline__ void ldlt_panel(float2* F, int ld, int n, int c0, int w, const float2* pu, const float2* pl,
-                                           float2* wu, float2* wl, int* fail)
-{
-    const int lane = threadIdx.x & 31;
-    const bool diag = lane < kPan;
-    const int i = c0 + lane + (diag ? 0 : kPanRows * w);
-    const int ic = min(i, n);
-    float2 a[kPan], l[kPan];
-#pragma unroll
-    for (int c = 0; c < kPan; ++c) a[c] = lane >= c ? F[ic * ld + c0 + c] : make_float2(0.f, 0.f);
-    if (pu) {
-        pan_load(pl, ic, l);
-#pragma unroll
-        for (int c = 0; c < kPan; ++c) {
-            float2 u[kPan];
-            pan_load(pu, c0 + c, u);
-#pragma unroll
-            for (int q = 0; q < kPan; ++q) a[c] = ff_msub_acc(a[c], l[q], u[q]);
-        }
-    }
-    bool ok = true;
-#pragma unroll
-    for (int p = 0; p < kPan; ++p) {
-        float2 u[kPan];
-#pragma unroll
-        for (int c = p; c < kPan; ++c)
-            u[c] = make_float2(__shfl_sync(0xffffffffu, a[p].x, c), __shfl_sync(0xffffffffu, a[p].y, c));
-        a[p] = ff_norm(a[p].x, a[p].y);
-        ok = ok && u[p].x > 0.f && u[p].x < INFINITY;
-        const float2 r = ff_rcp(u[p]);
-        l[p] = ff_mul_acc(a[p], r);
-#pragma unroll
-        for (int c = p + 1; c < kPan; ++c) a[c] = ff_msub_acc(a[c], l[p], ff_norm(u[c].x, u[c].y));
-    }
-    if (!ok && lane == 0) *fail = 1;
-#pragma unroll
-    for (int c = 0; c < kPan; ++c) l[c] = ff_norm(l[c].x, l[c].y);
-    if (!diag && i <= n) {
-        pan_store(wu, i, a);
-        pan_store(wl, i, l);
-    }
-    if (i == n) {
-#pragma unroll
-        for (int c = 0; c < kPan; ++c) F[n * ld + c0 + c] = l[c];
-    } else if (i < n && (!diag || w == 0)) {
-#pragma unroll
-        for (int c = 0; c < kPan; ++c)
-            if (i > c0 + c) F[(c0 + c) * ld + i] = l[c];
-    }
-}
-
-// Applies a panel (pu, pl) to the trailing columns c1 .. n - 1, rows down to
-// n: tiles of 2 x 2 entries, 32 tiles a warp at a time from the counter, so
-// that warps join when their part of the next panel is done.  12
-// instructions a product leave the FP32 pipes the limit; a tile reads 16
-// 16-byte words of shared memory for its 24 products (one entry a thread: 14
-// for six, more than the shared memory delivers at that rate).
-__device__ __forceinline__ void ldlt_trailing(float2* F, int ld, int n, int c1, const float2* pu, const float2* pl,
-                                              int* counter)
-{
-    const int lane = threadIdx.x & 31;
-    const int h = (n - c1) >> 1, tiles = h * (h + 3) / 2;      // column pairs; row pairs h + 1, the last with row n alone
-    for (;;) {
-        int t0 = 0;
-        if (lane == 0) t0 = atomicAdd(counter, 32);
-        t0 = __shfl_sync(0xffffffffu, t0, 0);
-        if (t0 >= tiles) return;
-        const int t = t0 + lane;
-        if (t >= tiles) continue;
-        // tiles numbered from the last column pair back: t = r (r + 3) / 2 + c
-        // for column pair h - 1 - r and row pair h - c; r from the square
-        // root, corrected by one step either way (t < 2^12)
-        int r = (int)((sqrtf(8.0f * (float)t + 9.0f) - 3.0f) * 0.5f);
-        if (r * (r + 3) / 2 > t) --r;
-        if ((r + 1) * (r + 4) / 2 <= t) ++r;
-        const int j = c1 + 2 * (h - 1 - r), i = c1 + 2 * (h - (t - r * (r + 3) / 2));
-        const int i1 = min(i + 1, n);
-        float2* f0 = F + i * ld + j;
-        float2* f1 = F + i1 * ld + j;
-        float2 v00 = f0[0], v01 = f0[1], v10 = f1[0], v11 = f1[1];
-        const float4* u0 = reinterpret_cast<const float4*>(pu + j * kPan);
-        const float4* l0 = reinterpret_cast<const float4*>(pl + i * kPan);
-        const float4* l1 = reinterpret_cast<const float4*>(pl + i1 * kPan);
-#pragma unroll
-        for (int q = 0; q < kPan / 2; ++q) {
-            const float4 ua = u0[q], ub = u0[q + kPan / 2], la = l0[q], lb = l1[q];
-            v00 = ff_msub_acc(v00, make_float2(la.x, la.y), make_float2(ua.x, ua.y));
-            v01 = ff_msub_acc(v01, make_float2(la.x, la.y), make_float2(ub.x, ub.y));
-            v10 = ff_msub_acc(v10, make_float2(lb.x, lb.y), make_float2(ua.x, ua.y));
-            v11 = ff_msub_acc(v11, make_float2(lb.x, lb.y), make_float2(ub.x, ub.y));
-            v00 = ff_msub_acc(v00, make_float2(la.z, la.w), make_float2(ua.z, ua.w));
-            v01 = ff_msub_acc(v01, make_float2(la.z, la.w), make_float2(ub.z, ub.w));
-            v10 = ff_msub_acc(v10, make_float2(lb.z, lb.w), make_float2(ua.z, ua.w));
-            v11 = ff_msub_acc(v11, make_float2(lb.z, lb.w), make_float2(ub.z, ub.w));
-        }
-        f0[0] = v00;
-        if (i > j) f0[1] = v01;
-        if (i < n) {
-            f1[0] = v10;
-            f1[1] = v11;
-        }
-    }
-}
-
 template <typename Idle = LdltNoIdle>
 __device__ __forceinline__ bool ldlt_solve(double* __restrict__ H, int ld, int n, double* __restrict__ y,
-                                           const LdltScratch& sc, int* fail, unsigned long long& t_mid,
+                                           const LdltScratch& sc, bool inverse, int* fail, unsigned long long& t_mid,
                                            const Idle& idle = Idle())
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x;
-    float2* F = reinterpret_cast<float2*>(H);
-    float2* yf = reinterpret_cast<float2*>(y);     // row n of F
-    float2* pan = reinterpret_cast<float2*>(sc.pan);
-    const int pan_len = kPan * (n + 1);            // buffer b: u at pan + 2 b pan_len, l after it
-    int* shift = sc.shift;
-    // scaling: row i by 2^shift[i], so that the diagonal lies in [1, 4), and
-    // the right-hand side so that its largest entry lies in [1, 2)
-    for (int i = tid; i < n; i += nt) {
-        const double d = H[i * ld + i];
-        const int f = f64_exponent(d);
-        if (f == 0 || f == 0x7ff || __double2hiint(d) < 0) *fail = 1;     // not positive (or not finite)
-        shift[i] = -((f - 1023) >> 1);
-    }
-    __syncthreads();
-    for (int i = warp; i < n; i += nt >> 5) {
-        // a row's parts together: the compiler keeps loads behind the stores
-        // to the same memory
-        constexpr int kParts = (kLdltMaxN + 31) / 32;
-        double h[kParts];
-        int e[kParts];
-#pragma unroll
-        for (int q = 0; q < kParts; ++q) {
-            const int j = min(lane + 32 * q, i);
-            h[q] = H[i * ld + j];
-            e[q] = shift[j];
-        }
-        const int si = shift[i];
-#pragma unroll
-        for (int q = 0; q < kParts; ++q) {
-            const int j = lane + 32 * q;
-            if (32 * q > i) break;
-            const float2 f = ff_from_f64(h[q], si + e[q]);
-            if (j <= i) F[i * ld + j] = f;
-        }
-    }
-    if (warp == 7) {
-        int e = -100000;
-        for (int i = lane; i < n; i += 32) {
-            const int f = f64_exponent(y[i]);
-            if (f != 0 && f != 0x7ff) e = max(e, f - 1023 + shift[i]);
-        }
-#pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, off));
-        e = e > -100000 ? -e : 0;
-        if (lane == 0) shift[n] = e;
-        for (int i = lane; i < n; i += 32) yf[i] = ff_from_f64(y[i], shift[i] + e);
-    }
-    __syncthreads();
-    if (n <= kInvMaxN && *fail == 0) {
-        float* buf = reinterpret_cast<float*>(pan);
+    if (inverse) {
+        // the scaled system beside H: entry (i, j), i >= j, at F[j ld + i], the
+        // places right of H's diagonal (H and y stay as they are for the
+        // factorisation)
+        float2* F = reinterpret_cast<float2*>(H) + 1;
+        float* buf = reinterpret_cast<float*>(sc.work);
+        float2* x = reinterpret_cast<float2*>(buf + inv_floats(n)) - 2 * n;
+        float2* b = x + n;
         float2* p = reinterpret_cast<float2*>(sc.part);
-        // rows (with padding) of the row groups, by size
-        const int rows = n <= 12 ? inv_stride(6) * 2 : n <= 30 ? inv_stride(6) * 5 : n <= 60 ? inv_stride(18) * 4 : n <= 96 ? 48 * 2 : 60 * 2;
-        float2* x = reinterpret_cast<float2*>(buf + 2 * kPan * (rows + n));
-        const bool done = n <= 12   ? inverse_solve<6, 2>(F, ld, n, yf, buf, p, x)
-                          : n <= 30 ? inverse_solve<6, 5>(F, ld, n, yf, buf, p, x)
-                          : n <= 60 ? inverse_solve<18, 4>(F, ld, n, yf, buf, p, x)
-                          : n <= 96 ? inverse_solve<48, 2>(F, ld, n, yf, buf, p, x)
-                                    : inverse_solve<60, 2>(F, ld, n, yf, buf, p, x);
-        if (done) {
-            t_mid = clock64();
-            for (int i = tid; i < n; i += nt) y[i] = ff_to_f64(x[i], shift[i] - shift[n]);
+        int* shift = sc.shift;
+        // row i by 2^shift[i], so that the diagonal lies in [1, 4), and the
+        // right-hand side so that its largest entry lies in [1, 2)
+        bool bad = false;
+        for (int i = tid; i < n; i += nt) {
+            const double d = H[i * ld + i];
+            const int f = f64_exponent(d);
+            bad = bad || f == 0 || f == 0x7ff || __double2hiint(d) < 0;     // not positive, or not finite
+            shift[i] = -((f - 1023) >> 1);
+        }
+        if (!__syncthreads_or(bad)) {
+            for (int i = warp; i < n; i += nt >> 5) {
+                // a row's parts together: the compiler keeps loads behind the stores
+                // to the same memory
+                constexpr int kParts = (kLdltMaxN + 31) / 32;
+                double h[kParts];
+                int e[kParts];
+#pragma unroll
+                for (int q = 0; q < kParts; ++q) {
+                    const int j = min(lane + 32 * q, i);
+                    h[q] = H[i * ld + j];
+                    e[q] = shift[j];
+                }
+                const int si = shift[i];
+#pragma unroll
+                for (int q = 0; q < kParts; ++q) {
+                    const int j = lane + 32 * q;
+                    if (32 * q > i) break;
+                    const float2 f = ff_from_f64(h[q], si + e[q]);
+                    if (j <= i) F[j * ld + i] = f;
+                }
+            }
+            if (warp == 7) {
+                int e = -100000;
+                for (int i = lane; i < n; i += 32) {
+                    const int f = f64_exponent(y[i]);
+                    if (f != 0 && f != 0x7ff) e = max(e, f - 1023 + shift[i]);
+                }
+#pragma unroll
+                for (int off = 16; off >= 1; off >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, off));
+                e = e > -100000 ? -e : 0;
+                if (lane == 0) shift[n] = e;
+                for (int i = lane; i < n; i += 32) b[i] = ff_from_f64(y[i], shift[i] + e);
+            }
             __syncthreads();
-            return false;
+            const bool done = n <= 12    ? inverse_solve<6, 2>(F, ld, n, b, buf, p, x)
+                              : n <= 30  ? inverse_solve<6, 5>(F, ld, n, b, buf, p, x)
+                              : n <= 60  ? inverse_solve<18, 4>(F, ld, n, b, buf, p, x)
+                              : n <= 96  ? inverse_solve<48, 2>(F, ld, n, b, buf, p, x)
+                              : n <= 120 ? inverse_solve<60, 2>(F, ld, n, b, buf, p, x)
+                                         : inverse_solve<138, 1>(F, ld, n, b, buf, p, x);
+            if (done) {
+                t_mid = clock64();
+                for (int i = tid; i < n; i += nt) y[i] = ff_to_f64(x[i], shift[i] - shift[n]);
+                __syncthreads();
+                return false;
+            }
         }
         __syncthreads();
     }
-    // LDL^T in panels of six columns (one node), the right-hand side carried
-    // along as row n, one barrier a panel: the warps that hold the panel's
-    // rows bring it up to date and factorise it -- the serial chain of the
-    // solve -- while the others apply the panel before it to the rest of the
-    // trailing triangle, where the first ones then join.  L is stored
-    // transposed in the upper triangle, L_ik at (k, i).  A failed pivot sets
-    // *fail; the loop still runs to the end (same bounds, discarded values).
-    for (int c0 = 0; c0 < n; c0 += kPan) {
-        const int b = (c0 / kPan) & 1;
-        float2* wu = pan + 2 * b * pan_len;
-        const float2* pu = pan + 2 * (b ^ 1) * pan_len;      // the panel before this one
-        if (kPanRows * warp < n + 1 - kPan - c0)
-            ldlt_panel(F, ld, n, c0, warp, c0 > 0 ? pu : nullptr, pu + pan_len, wu, wu + pan_len, fail);
-        if (c0 > 0) ldlt_trailing(F, ld, n, c0 + kPan, pu, pu + pan_len, shift + n + 1 + b);
-        if (tid == 0) shift[n + 1 + (b ^ 1)] = 0;            // the next panel's counter
+    double* rD = sc.rD;
+    double* colb = sc.work;
+    int* tab = reinterpret_cast<int*>(sc.work + 2 * n);
+    // LDL^T with a one-column look-ahead, one barrier per column.  At step k
+    // warp 0 prepares column k+1 -- its update by column k, the pivot
+    // D_{k+1} and reciprocal, and the scaled l_{i,k+1} -- while warps
+    // {1,2,3,5,6,7} (no FP64 pipe shared with warp 0) apply column k to the
+    // trailing triangle of rows and columns >= k+2 and carry the forward
+    // substitution.  The scaled column is double-buffered; L is stored
+    // transposed in the upper triangle, L_ik at (k, i).  A failed pivot
+    // (not positive) sets *fail and a zero reciprocal; the loop still runs
+    // to the end (same bounds, finite or discarded values), which keeps a
+    // shared-memory read and a branch off every column of the chain.
+    for (int ip = tid; ip < n; ip += nt)
+        for (int jp = 0; jp <= ip; ++jp) tab[ip * (ip + 1) / 2 + jp] = (ip << 16) | jp;
+    if (warp == 0) {
+        double r = 0.0;
+        if (lane == 0) {
+            const double d = H[0];
+            if (!(d > 0.0)) *fail = 1; else r = rcp_fp64(d);
+            rD[0] = r;
+        }
+        r = __shfl_sync(0xffffffffu, r, 0);
+        for (int i = 1 + lane; i < n; i += 32) {
+            const double l = H[i * ld] * r;
+            colb[i] = l;
+            H[i] = l;
+        }
+    }
+    __syncthreads();
+    // bulk warps: {1,2,3,5,6,7}, and also warp 4 while the trailing triangle
+    // is large (the early columns, where the bulk update and not warp 0's
+    // chain sets the pace; warp 4 shares warp 0's FP64 unit, which has slack
+    // there)
+    const int bt6 = (warp != 0 && warp != 4 && warp < 8) ? (warp < 4 ? warp - 1 : warp - 2) * 32 + lane : -1;
+    const int bt7 = (warp != 0 && warp < 8) ? (warp - 1) * 32 + lane : -1;
+    for (int k = 0; k < n - 1; ++k) {
+        const double* ck = colb + (k & 1) * n;        // l_{i,k}
+        double* cn = colb + ((k + 1) & 1) * n;        // l_{i,k+1}, written now
+        const bool wide = n - k - 2 >= kWideBulkRows;
+        const int nbulk = wide ? 7 * 32 : 6 * 32;
+        const int bt = wide ? bt7 : bt6;
+        const bool bulk = bt >= 0;
+        if (warp == 0) {
+            // column p = k + 1, rows i = p .. n-1 in slots of 32: u_i = H_ip -
+            // l_ik H_pk (the pivot is u_p), then every lane forms 1 / u_p
+            // itself (no divergent branch, no second broadcast) and scales
+            const int p = k + 1;
+            const double hpk = H[p * ld + k];         // unscaled H_{k+1,k}
+            const int nq = (n - p + 31) >> 5;         // active slots (warp-uniform)
+            constexpr int kRows = (kLdltMaxN + 31) / 32;
+            double hv[kRows], cv[kRows], u[kRows];
+#pragma unroll
+            for (int q = 0; q < kRows; ++q) {
+                if (q >= nq) break;
+                const int i = p + lane + 32 * q;
+                hv[q] = i < n ? H[i * ld + p] : 0.0;
+                cv[q] = i < n ? ck[i] : 0.0;
+            }
+#pragma unroll
+            for (int q = 0; q < kRows; ++q) {
+                if (q >= nq) break;
+                u[q] = hv[q] - cv[q] * hpk;
+            }
+            const double h = __shfl_sync(0xffffffffu, u[0], 0);
+            // h > 0 as an integer test on the bits (positive, not NaN): no
+            // FP64 compare on the chain
+            const long long hb = __double_as_longlong(h);
+            const bool ok = hb > 0ll && hb <= 0x7ff0000000000000ll;
+            const double rp = ok ? rcp_fp64(h) : 0.0;
+            if (lane == 0) {
+                if (!ok) *fail = 1;
+                H[p * ld + p] = h;
+                rD[p] = rp;
+            }
+#pragma unroll
+            for (int q = 0; q < kRows; ++q) {
+                if (q >= nq) break;
+                const int i = p + lane + 32 * q;
+                if (i > p && i < n) {
+                    const double l = u[q] * rp;
+                    H[i * ld + p] = u[q];
+                    cn[i] = l;
+                    H[p * ld + i] = l;
+                }
+            }
+        } else if (bulk) {
+            const int m1 = n - k - 2, tri = m1 * (m1 + 1) / 2;
+            const double zk = y[k];
+            for (int i = k + 1 + bt; i < n; i += nbulk) y[i] -= ck[i] * zk;
+            int t = bt;
+            for (; t + nbulk < tri; t += 2 * nbulk) {
+                const int e0 = tab[t], e1 = tab[t + nbulk];
+                const int i0 = k + 2 + (e0 >> 16), j0 = k + 2 + (e0 & 0xffff);
+                const int i1 = k + 2 + (e1 >> 16), j1 = k + 2 + (e1 & 0xffff);
+                const double a0 = H[i0 * ld + j0], a1 = H[i1 * ld + j1];
+                const double l0 = ck[i0], l1 = ck[i1];
+                const double b0 = H[j0 * ld + k], b1 = H[j1 * ld + k];
+                H[i0 * ld + j0] = a0 - l0 * b0;
+                H[i1 * ld + j1] = a1 - l1 * b1;
+            }
+            for (; t < tri; t += nbulk) {
+                const int e = tab[t];
+                const int i = k + 2 + (e >> 16), j = k + 2 + (e & 0xffff);
+                H[i * ld + j] -= ck[i] * H[j * ld + k];
+            }
+        }
         __syncthreads();
     }
+    for (int i = tid; i < n; i += nt) y[i] *= rD[i];   // D w = z
+    __syncthreads();
     t_mid = clock64();
     const bool failed = *fail != 0;
     // L^T x = w, unit diagonal (L_ki is stored at (i, k)), in blocks of 32
     // unknowns from the last block up.  Warp 0 runs the chain of one block
     // with the block's values in registers, lane l holding row r0 + l: x_k
-    // is broadcast from its lane with a shuffle.  The rows above the block
-    // then take the block's unknowns as dot products, split into column
-    // chunks over several warps (partial sums in shared memory, added per
-    // row).
-    float2* part = reinterpret_cast<float2*>(sc.part);
+    // is broadcast from its lane with a shuffle, and the FP64 instructions
+    // issued do not grow with the size of the system.  The rows above the
+    // block then take the
+    // block's unknowns as dot products, split into column chunks over
+    // several warps (partial sums in shared memory, added per row).
+    double* part = sc.part;
     for (int r0 = ((n - 1) >> 5) << 5; r0 >= 0; r0 -= 32) {
         const int r1 = min(n, r0 + 32);
         if (warp == 0) {
             const int i = r0 + lane;
-            const float2 zero = make_float2(0.f, 0.f);
-            float2 wv = i < r1 ? yf[i] : zero;
+            double wv = i < r1 ? y[i] : 0.0;
+            int k = r1 - 1;
             // two unknowns a step: x_k is final; every lane forms
             // x_{k-1} = w_{k-1} - L_{k,k-1} x_k itself from the broadcast
-            // values (the same operation its owner would apply), so the
-            // chain is one shuffle and two multiply-subtracts deep per two
-            // unknowns; the next step's values of L are read ahead.  (An odd
-            // number of unknowns in the block starts one row past it, where
-            // L and w are taken as zero.)
-            const float2* row = F + min(i, n - 1) * ld + r0;
-            int k = (r1 - r0 - 1) | 1;
-            auto at = [&](int q) { return lane < q && r0 + q < r1 ? row[q] : zero; };
-            float2 hk = at(k), hk1 = at(k - 1);
-            for (; k > 0; k -= 2) {
-                const float2 nk = at(k - 2), nk1 = at(k - 3);
-                const float2 lk = make_float2(__shfl_sync(0xffffffffu, hk.x, k - 1), __shfl_sync(0xffffffffu, hk.y, k - 1));
-                const float2 xk = make_float2(__shfl_sync(0xffffffffu, wv.x, k), __shfl_sync(0xffffffffu, wv.y, k));
-                const float2 wk1 = make_float2(__shfl_sync(0xffffffffu, wv.x, k - 1),
-                                               __shfl_sync(0xffffffffu, wv.y, k - 1));
-                const float2 xk1 = ff_msub_acc(wk1, lk, xk);
-                wv = ff_msub_acc(wv, hk, xk);
-                wv = ff_msub_acc(wv, hk1, xk1);
-                hk = nk;
-                hk1 = nk1;
+            // values (the same FMA its owner would apply), so the chain is
+            // one shuffle and two FMAs deep per two unknowns; each row takes
+            // x_k, then x_{k-1}, exactly as in the one-at-a-time order
+            for (; k > r0 + 1; k -= 2) {
+                const double hk = i < k ? H[i * ld + k] : 0.0;
+                const double hk1 = i < k - 1 ? H[i * ld + k - 1] : 0.0;
+                const double lk = H[(k - 1) * ld + k];        // L_{k,k-1}
+                const double xk = __shfl_sync(0xffffffffu, wv, k - r0);
+                const double wk1 = __shfl_sync(0xffffffffu, wv, k - 1 - r0);
+                const double xk1 = fma(-lk, xk, wk1);
+                if (i < k) wv = fma(-hk, xk, wv);
+                if (i < k - 1) wv = fma(-hk1, xk1, wv);
             }
-            if (i < r1) yf[i] = ff_norm(wv.x, wv.y);
+            if (k == r0 + 1) {
+                const double hk = i < k ? H[i * ld + k] : 0.0;
+                const double xk = __shfl_sync(0xffffffffu, wv, k - r0);
+                if (i < k) wv = fma(-hk, xk, wv);
+            }
+            if (i < r1) y[i] = wv;
         } else if (r0 + 32 >= n && !failed) {
             idle(warp);
         }
@@ -680,28 +657,23 @@ __device__ __forceinline__ bool ldlt_solve(double* __restrict__ H, int ld, int n
         const int chunks = min(4, 256 / r0);      // r0 <= 128: at least 2
         if (tid < chunks * r0) {
             const int i = tid % r0, c = tid / r0;
-            float2 s0 = make_float2(0.f, 0.f), s1 = s0;
+            double s0 = 0.0, s1 = 0.0;
             int k = r0 + c;
             for (; k + chunks < r1; k += 2 * chunks) {
-                s0 = ff_msub_acc(s0, F[i * ld + k], yf[k]);
-                s1 = ff_msub_acc(s1, F[i * ld + k + chunks], yf[k + chunks]);
+                s0 = fma(H[i * ld + k], y[k], s0);
+                s1 = fma(H[i * ld + k + chunks], y[k + chunks], s1);
             }
-            if (k < r1) s0 = ff_msub_acc(s0, F[i * ld + k], yf[k]);
-            part[c * r0 + i] = ff_add(s0, s1);
+            if (k < r1) s0 = fma(H[i * ld + k], y[k], s0);
+            part[c * r0 + i] = s0 + s1;
         }
         __syncthreads();
         for (int i = tid; i < r0; i += nt) {
-            float2 s = part[i];
-            for (int c = 1; c < chunks; ++c) s = ff_add(s, part[c * r0 + i]);
-            yf[i] = ff_add(yf[i], s);
+            double s = part[i];
+            for (int c = 1; c < chunks; ++c) s += part[c * r0 + i];
+            y[i] -= s;
         }
         __syncthreads();
     }
-    for (int i = tid; i < n; i += nt) {
-        const float2 x = yf[i];
-        y[i] = ff_to_f64(x, shift[i] - shift[n]);
-    }
-    __syncthreads();
     return true;
 }
 #endif

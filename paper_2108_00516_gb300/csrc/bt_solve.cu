@@ -1,7 +1,7 @@
 // bt_solve.cu -- sm_103a kernels of the pose-graph solve (BundleTrack, Sec. IV-D):
 // single-precision transforms of the FP64 poses, the reduction of the residual
 // pass's FP32 partials into FP64 6x6 blocks, the assembly of the normal
-// equations, the Cholesky (LDL^T) solve and the FP64 se(3) update, for one
+// equations, their solve and the FP64 se(3) update, for one
 // graph (reduce_kernel) or a batch of graphs (batch_*_kernel).
 //
 //   reduce_kernel   one CTA per unordered node pair turns the FP32 partials of
@@ -366,20 +366,19 @@ __device__ double se3_exp_entry(const double* xi, const double* cf, int r, int c
 }
 
 // Last CTA: energies, then (full) assembly of H and g over the free nodes,
-// the solve of H dx = -g (FP32 inverse with double-float corrections or
-// double-float Cholesky, bt_ldlt.h; or PCG, the paper's inner solver, in FP64),
-// and finally
+// the solve of H dx = -g (FP32 inverse with double-float corrections or FP64
+// Cholesky, bt_ldlt.h; or PCG, the paper's inner solver, in FP64), and finally
 // T <- T exp(dx).
 // The first global reads of the last CTA, issued by every CTA of the reduce
 // kernel before its pair stage: the last CTA is only known after the
-// hand-off, and these values (the sticky status of earlier iterations, the
-// nodes' free indices, the poses) do not change within the kernel, so their
+// hand-off, and these values (what earlier iterations left in the control
+// block, the nodes' free indices, the poses) do not change within the kernel, so their
 // L2 round trip overlaps the pair stage instead of following the hand-off.
 // Thread t holds pose entries t and t + blockDim.x (12 N <= 2 * 256) and the
 // free index of node t.
 static_assert(12 * kMaxNodes <= 2 * kThreads && kMaxNodes <= kThreads, "final_prefetch: two pose entries a thread");
 struct FinalPrefetch {
-    int status;
+    int status, declined;
     int free_idx;
     double pose0, pose1;
 };
@@ -387,10 +386,11 @@ struct FinalPrefetch {
 template <bool kFull>
 __device__ __forceinline__ FinalPrefetch final_prefetch(const SolveArgs& a)
 {
-    FinalPrefetch pf{0, -1, 0.0, 0.0};
+    FinalPrefetch pf{0, 0, -1, 0.0, 0.0};
     if (!kFull) return pf;
     const int tid = threadIdx.x, nt = blockDim.x, N = a.N;
     pf.status = __ldcg(&a.ctrl->status);
+    pf.declined = __ldcg(&a.ctrl->declined);
     if (tid < N) pf.free_idx = __ldcg(&a.nodes[tid].free_idx);
     if (tid < 12 * N) pf.pose0 = __ldcg(a.pose + tid);
     if (tid + nt < 12 * N) pf.pose1 = __ldcg(a.pose + tid + nt);
@@ -451,14 +451,14 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
     }
     unsigned long long t0 = clock64();
     const int ld = n + 1;        // odd leading dimension: conflict-free FP64 rows
-    double* H = sm;              // n*ld: lower triangle H, then L^T in the upper triangle
+    double* H = sm;              // n*ld: lower triangle H; beside it the solve's scaled system, or L^T
     double* y = H + n * ld;      // n
-    double* rD = y + n;          // n: scratch (PCG, the update)
+    double* rD = y + n;          // n: 1 / D_k; scratch (PCG, the update)
     double* ps = rD + n;         // 12 * N poses
     double* tinv = ps + 12 * kMaxNodes;   // 12 * N
-    // tinv + 12 * kMaxNodes: the solve's panels and scaling exponents (bt_ldlt.h)
+    // tinv + 12 * kMaxNodes: the solve's scratch and scaling exponents (bt_ldlt.h)
     double* colb = tinv + 12 * kMaxNodes;    // 16-byte aligned: n is even
-    double* shift = colb + ldlt_pan_doubles(n);
+    double* shift = colb + ldlt_work_doubles(n);
     int* node_of = reinterpret_cast<int*>(shift + ldlt_shift_doubles(n));
     double* scratch = reinterpret_cast<double*>(node_of + kMaxNodes);      // 264 doubles
     __shared__ int s_fail, free_of[kMaxNodes];
@@ -647,17 +647,21 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
         __syncthreads();
         t2 = t3 = clock64();
     } else {
-    // by the FP32 inverse and corrections, or LDL^T in panels of six columns,
-    // D w = z, blocked L^T dx = w (bt_ldlt.h)
+    // by the FP32 inverse and corrections, or LDL^T with a one-column
+    // look-ahead, D w = z, blocked L^T dx = w (bt_ldlt.h)
     LdltScratch sc;
-    sc.pan = colb;
+    sc.work = colb;
+    sc.rD = rD;
     sc.shift = reinterpret_cast<int*>(shift);
     sc.part = scratch;
     // the factorisation leaves the last warp time to add the energies up while
-    // warp 0 runs the first block of the back substitution alone
-    costs_due = !ldlt_solve(H, ld, n, y, sc, &s_fail, t2, [&](int w) {
+    // warp 0 runs the first block of the back substitution alone.  The systems
+    // of a solve's iterations are much alike: where one was left to the
+    // factorisation, the later ones go straight to it
+    costs_due = !ldlt_solve(H, ld, n, y, sc, pf.declined == 0, &s_fail, t2, [&](int w) {
         if (w == cost_warp) write_costs();
     });
+    if (!costs_due && tid == 0) a.ctrl->declined = 1;
     if (s_fail) {
         if (tid == 0) a.ctrl->status = -4;
         if (warp == cost_warp) write_costs();
@@ -671,7 +675,8 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
     // three sub-partitions), the entries of exp(dx_A) (one thread each), the
     // products T_A exp(dx_A) (one thread each).  The solve's scratch, rD
     // and tinv are free now (after PCG the last warp adds up the energies
-    // meanwhile; the Cholesky path has done so during its back substitution).
+    // meanwhile, as after the inverse; the factorisation has had it done during
+    // its back substitution).
     {
         double* cf = rD;       // [nf][4]: th^2, A, B, C
         double* E = colb;      // [nf][12]
@@ -754,9 +759,9 @@ __global__ void __launch_bounds__(kThreads, 1) reduce_kernel(SolveArgs a, int it
 size_t reduce_smem_bytes(int n_free)
 {
     const size_t n = 6 * (size_t)n_free;
-    // H, y, two poses' worth a node, the solve's panels and exponents, the
+    // H, y, two poses' worth a node, the solve's scratch and exponents, the
     // node table, 256 partial sums + 8 warp sums
-    const size_t fin = (n * (n + 1) + 2 * n + 24 * (size_t)kMaxNodes + ldlt_pan_doubles(n) + ldlt_shift_doubles(n) + 264) *
+    const size_t fin = (n * (n + 1) + 2 * n + 24 * (size_t)kMaxNodes + ldlt_work_doubles((int)n) + ldlt_shift_doubles(n) + 264) *
                            sizeof(double) + kMaxNodes * sizeof(int);
     const size_t ph1 = kPairSmemDoubles * sizeof(double);
     return fin > ph1 ? fin : ph1;

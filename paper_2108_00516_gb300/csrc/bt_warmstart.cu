@@ -1244,9 +1244,10 @@ __global__ void __launch_bounds__(kAvgThreads) average_kernel(const AvgGraph* __
     double* H = sT + 12 * N;                 // [n][ld]
     double* b = H + (size_t)n * ld;          // [n]
     LdltScratch sc;                          // the solve's scratch (bt_ldlt.h)
-    sc.pan = b + n;                          // 16-byte aligned: n is even
-    sc.part = sc.pan + ldlt_pan_doubles(n);  // [256]
-    int* eof = reinterpret_cast<int*>(sc.part + 256);   // [N][N]
+    sc.work = b + n;                         // 16-byte aligned: n is even
+    sc.part = sc.work + ldlt_work_doubles(n);  // [256]
+    sc.rD = sc.part + 256;                   // [n]
+    int* eof = reinterpret_cast<int*>(sc.rD + n);       // [N][N]
     int* freenode = eof + N * N;             // [nf]
     sc.shift = freenode + nf;
     const double Wd[6] = {1.0 / (kSU * kSU), 1.0 / (kSU * kSU), 1.0 / (kSU * kSU),
@@ -1384,12 +1385,12 @@ __global__ void __launch_bounds__(kAvgThreads) average_kernel(const AvgGraph* __
         b[r] = v;
     }
     __syncthreads();
-    // 4-5. H d = b by LDL^T in double-float arithmetic (bt_ldlt.h); a
-    // pivot that is not positive, or a solution that is not finite, leaves
-    // the poses as they were
+    // 4-5. H d = b by the FP32 inverse with double-float corrections, or
+    // FP64 LDL^T where it declines (bt_ldlt.h); a pivot that is not positive,
+    // or a solution that is not finite, leaves the poses as they were
     if (n > 0) {
         unsigned long long t_unused;
-        ldlt_solve(H, ld, n, b, sc, &s_sing, t_unused);
+        ldlt_solve(H, ld, n, b, sc, true, &s_sing, t_unused);
         for (int i = tid; i < n; i += kAvgThreads)
             if (!isfinite(b[i])) s_sing = 1;
         __syncthreads();
@@ -1469,7 +1470,7 @@ cudaError_t launch_adam(Net net, const float* grad, float lr, float beta1, float
 size_t average_smem_bytes(int max_free, int max_N)
 {
     const size_t n = 6 * (size_t)max_free;
-    return sizeof(double) * (24 * (size_t)max_N + n * (n + 1) + n + ldlt_pan_doubles(n) + 256 + ldlt_shift_doubles(n)) +
+    return sizeof(double) * (24 * (size_t)max_N + n * (n + 1) + 2 * n + ldlt_work_doubles((int)n) + 256 + ldlt_shift_doubles(n)) +
            sizeof(int) * ((size_t)max_N * max_N + max_free) + 16;
 }
 
