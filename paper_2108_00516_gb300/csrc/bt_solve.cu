@@ -735,7 +735,7 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
 template <bool kFull>
 __global__ void __launch_bounds__(kThreads, 1) reduce_kernel(SolveArgs a, int iter)
 {
-    extern __shared__ double sm[];
+    extern __shared__ __align__(16) double sm[];
     __shared__ int s_last;
     const int b = blockIdx.x;
     // the previous update's poses and status: written before the residual
@@ -813,7 +813,7 @@ template <bool kFull>
 __global__ void __launch_bounds__(kThreads, 1) batch_solve_kernel(const SolveArgs* __restrict__ args, int iter)
 {
     pdl_wait_and_release();
-    extern __shared__ double smd[];
+    extern __shared__ __align__(16) double smd[];
     __shared__ SolveArgs sa;
     if (threadIdx.x == 0) sa = args[blockIdx.x];
     __syncthreads();

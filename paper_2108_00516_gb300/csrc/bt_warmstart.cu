@@ -1234,7 +1234,7 @@ __device__ __forceinline__ void tri_rc(int q, int& r, int& c)
 
 __global__ void __launch_bounds__(kAvgThreads) average_kernel(const AvgGraph* __restrict__ graphs)
 {
-    extern __shared__ double asm_[];
+    extern __shared__ __align__(16) double asm_[];
     __shared__ int s_sing;
     const AvgGraph G = graphs[blockIdx.x];
     const int N = G.N, E = G.n_edges, nf = G.n_free, n = 6 * nf, ld = n + 1;
