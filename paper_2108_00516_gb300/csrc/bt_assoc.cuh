@@ -76,8 +76,8 @@ __device__ __forceinline__ bool assoc_project(const PairK& k, float px, float py
     const float2 uv = __ffma2_rn(__fmul2_rn(qxy, k.f), make_float2(rz, rz), k.ch);
     constexpr float kRound = 12582912.0f;
     const float2 b = __fadd2_rd(uv, make_float2(kRound, kRound));
-    iu = __float_as_int(b.x) - 0x4B400000;
-    iv = __float_as_int(b.y) - 0x4B400000;
+    iu = (int)(__float_as_uint(b.x) - 0x4B400000u);      // modulo 2^32: any pattern may come here
+    iv = (int)(__float_as_uint(b.y) - 0x4B400000u);
     uvf = __fadd2_rn(b, make_float2(-kRound, -kRound));
     return qz > 1e-30f && (unsigned)iu < (unsigned)k.W && (unsigned)iv < (unsigned)k.H;
 }
