@@ -86,13 +86,22 @@ int grow(DevBuf& b, size_t bytes, size_t keep, cudaStream_t s, void** old_out = 
     return BT_OK;
 }
 
+// A handle's first room: 4096 sets (a minibatch, or the sets of a batch of
+// graphs, is a few thousand at most) of 256 points each, 25 MB, and the scratch
+// and outputs of a forward pass over all of them, 8.5 MB.  The latter is part
+// of it because the mapping of that many megabytes takes ~0.2 ms, which the
+// first pass would otherwise wait for; the pass that first takes more sets
+// than that grows it.
+constexpr int kFirstSets = 4096;
+constexpr int64_t kFirstPoints = 256 * (int64_t)kFirstSets;
+
 // Room for `add_pts` more points and `add_sets` more samples; sample point
 // pointers are rebased when the pools move.
 int reserve(bt_warmstart* ws, int64_t add_pts, int add_sets)
 {
     cudaStream_t s = ws->stream;
     if (ws->n_points + add_pts > ws->cap_points) {
-        int64_t cap = std::max<int64_t>(ws->cap_points * 2, std::max<int64_t>(ws->n_points + add_pts, 1 << 20));
+        int64_t cap = std::max<int64_t>(ws->cap_points * 2, std::max<int64_t>(ws->n_points + add_pts, kFirstPoints));
         void *old_p, *old_q;
         const size_t keep = sizeof(float) * 3 * (size_t)ws->n_points;
         int st = grow(ws->pool_p, sizeof(float) * 3 * (size_t)cap, keep, s, &old_p);
@@ -107,14 +116,11 @@ int reserve(bt_warmstart* ws, int64_t add_pts, int add_sets)
         ws->cap_points = cap;
     }
     if (ws->n_samples + add_sets > ws->cap_samples) {
-        int cap = std::max(ws->cap_samples * 2, std::max(ws->n_samples + add_sets, 4096));
+        int cap = std::max(ws->cap_samples * 2, std::max(ws->n_samples + add_sets, kFirstSets));
         int st = grow(ws->samples, sizeof(W::Sample) * (size_t)cap, sizeof(W::Sample) * (size_t)ws->n_samples, s);
         if (st != BT_OK) return st;
         ws->cap_samples = cap;
-        // outputs of the first few thousand sets with the room for the sets
-        // themselves: a mapping of megabytes (~0.2 ms) stays out of the first
-        // forward pass (larger ones grow it there)
-        if (!ws->out.p) BT_CUDA(ws->out.ensure(out_bytes(std::min(cap, 4096))), "alloc outputs");
+        if (!ws->out.p) BT_CUDA(ws->out.ensure(out_bytes(kFirstSets)), "alloc outputs");
     }
     return BT_OK;
 }
