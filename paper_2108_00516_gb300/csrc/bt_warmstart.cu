@@ -751,7 +751,7 @@ int num_sms()
 
 // ---------------------------------------------------------------------------
 // Backward pass: one CTA per set of the minibatch leaves what the set
-// contributes to the gradient in factored form (a BwdRec of 11.5 KiB), and
+// contributes to the gradient in factored form (a BwdRec of 12.5 KiB), and
 // one launch over the parameters sums the contributions of all sets.  The
 // gradients of layers 2, 3 and 4 are sums of outer products over the sets, so
 // writing them out per set first (264 KiB a set, read back by the sum) cost
@@ -1426,8 +1426,6 @@ cudaError_t launch_to_bf16(Net net, cudaStream_t s)
     to_bf16_kernel<<<(kNumParams + 255) / 256, 256, 0, s>>>(net);
     return cudaGetLastError();
 }
-
-size_t forward_smem_bytes() { return Fwd::Total; }
 
 template <bool kTrain>
 static cudaError_t launch_forward_t(Net net, const Sample* smp, const int* ids, int n, unsigned long long* pool,

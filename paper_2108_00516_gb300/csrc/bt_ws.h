@@ -85,6 +85,7 @@ struct __align__(16) BwdRec {
     float dy[kOut];
     float loss, pad;
 };
+static_assert(sizeof(BwdRec) == 12832, "12.5 KiB a set");
 
 // One graph of an averaging launch.
 struct AvgGraph {
@@ -105,7 +106,6 @@ cudaError_t launch_to_bf16(Net net, cudaStream_t s);
 inline size_t pool_bytes(int n) { return sizeof(unsigned long long) * kH2 * (size_t)n; }
 cudaError_t launch_forward(Net net, const Sample* smp, const int* ids, int n, unsigned long long* pool, float* y_out,
                            Cache* cache, cudaStream_t s);
-size_t forward_smem_bytes();
 // Gradient of the mean loss 1/2 |y - y*|^2 over n sets (sum over the sets in a
 // fixed order) and the loss (FP64); rec [n] is scratch.
 cudaError_t launch_backward(Net net, const Sample* smp, const int* ids, int n, Cache* cache, BwdRec* rec,
