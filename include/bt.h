@@ -400,7 +400,10 @@ int bt_batch_solve_warm(bt_batch* b, bt_warmstart* ws, int32_t iters, int32_t fa
  * camera i to camera j, q ~ rel_out p (pts_i, pts_j: count x 3 floats, host
  * or device); inliers_out (may be NULL) gets the inlier count.  With fewer
  * than 3 points or only degenerate samples rel_out is the identity and the
- * count 0.  Enqueued on cuda_stream and synchronised.
+ * count 0.  Enqueued on cuda_stream and synchronised.  The call's device
+ * scratch (about 100 bytes a sample and set) is one block of the device memory
+ * cache below, a power of two from 64 KiB to 64 MiB, which stays there idle
+ * afterwards; a larger one is allocated and freed by the call.
  * Errors: BT_ERR_INVALID, BT_ERR_CUDA, BT_ERR_OOM. */
 int bt_ransac(const float* pts_i, const float* pts_j, int32_t count, int32_t mem_kind, int32_t hypotheses,
               uint64_t seed, double inlier_dist, int32_t refine, double* rel_out, int32_t* inliers_out,
@@ -506,8 +509,10 @@ typedef struct {
     int64_t sparse_pairs;       /* correspondences of timed residual launches */
     /* SM clock cycles of the solve stage (the last CTA of each Gauss-Newton
      * iteration): [0] gathering the pair blocks and assembling H, g;
-     * [1] Cholesky factorisation with the forward substitution; [2] back
-     * substitution; [3] pose update and single-precision transforms */
+     * [1] the solve of H dx = -g by the inverse and its corrections, or, where
+     * the inverse declines, its attempt and the Cholesky factorisation with
+     * the forward substitution; [2] writing dx, or the back substitution;
+     * [3] pose update and single-precision transforms */
     int64_t solve_phase_cycles[4];
 } bt_profile;
 
@@ -527,7 +532,8 @@ int bt_profile_read(const bt_graph* g, bt_profile* out);
  * blocks to a process-wide cache of idle blocks, from which later graphs
  * take blocks of the same size class before allocating, so a series of
  * graphs reuses device memory instead of allocating and freeing it (cudaFree
- * synchronises the device).  Thread-safe.
+ * synchronises the device).  The scratch of bt_ransac and bt_ransac_init comes
+ * from it and goes back to it within the call.  Thread-safe.
  *
  * bt_device_cache_bytes: bytes of idle cached blocks.
  * bt_device_cache_trim: frees the idle blocks above 64 KiB (the smaller
