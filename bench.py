@@ -684,7 +684,8 @@ def run_ours(args):
                "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32",
                "data": "synthetic (seeded ray-cast box+ellipsoid sequence; no dataset)",
                "config": {"workload": WORKLOAD, "graphs_per_step": len(graphs), "iters": it,
-                          "max_nodes": 10, "solve_precision": "FP32 residual pass, FP64 assembly/Cholesky/exp",
+                          "max_nodes": 10, "solve_precision": "FP32 residual pass, FP64 assembly; solve by an FP32 inverse "
+                                             "corrected to FP64 accuracy or FP64 Cholesky; FP64 exp",
                           "l2": f"flushed ({L2_FLUSH_BYTES >> 20} MiB write) before every timed step; "
                                 f"sequence inputs {sum(seq.frame(t).depth.nbytes * 5 for t in range(seq.n)) / 1e9:.1f} GB "
                                 f"on device > L2",

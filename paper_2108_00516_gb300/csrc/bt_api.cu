@@ -609,7 +609,7 @@ int bt_add_frame(bt_graph* g, const float* depth, const float* normals, const ui
     f.dev_m2 = static_cast<int*>(m2);
     const float ifx = 1.0f / K->fx, ify = 1.0f / K->fy;
     // (M, zref) land in a mapped pinned slot, written by the preparation's
-    // scan kernel itself (no separate read-back copy), read at the next
+    // second kernel itself (no separate read-back copy), read at the next
     // topology build after a stream synchronisation
     if (e == cudaSuccess) {
         f.slot = g->free_slots.back();
