@@ -861,7 +861,7 @@ int batch_build(bt_batch* b, int shape)
     std::vector<bt::SolveArgs> args;
     std::vector<int2> wres, wpair;
     b->max_N = 1;
-    b->max_free = 0;
+    b->solve_smem = 0;
     b->pixels_per_pass = 0;
     for (size_t k = 0; k < b->graphs.size(); ++k) {
         bt_graph* g = b->graphs[k];
@@ -878,7 +878,7 @@ int batch_build(bt_batch* b, int shape)
         for (int t = 0; t < a.n_tiles; ++t) wres.push_back(make_int2((int)k, a.n_edges + t));
         for (int u = 0; u < a.n_upairs; ++u) wpair.push_back(make_int2((int)k, u));
         b->max_N = std::max(b->max_N, a.N);
-        b->max_free = std::max(b->max_free, a.n_free);
+        b->solve_smem = std::max(b->solve_smem, bt::reduce_smem_bytes(a.n_free));
         b->pixels_per_pass += g->pixels_per_pass;
     }
     cudaStream_t s = b->stream;
@@ -964,7 +964,7 @@ int batch_enqueue(bt_batch* b, int iters, int shape)
                                           b->precision, s),
                 "batch residual");
         BT_CUDA(bt::launch_batch_pairs(A, b->d_work_pair.as<int2>(), b->n_work_pair, full, s), "batch pairs");
-        BT_CUDA(bt::launch_batch_solve(A, G, b->max_free, full, p, s), "batch solve");
+        BT_CUDA(bt::launch_batch_solve(A, G, b->solve_smem, full, p, s), "batch solve");
     }
     return BT_OK;
 }

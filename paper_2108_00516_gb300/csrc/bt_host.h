@@ -343,7 +343,7 @@ struct bt_batch {
     std::vector<uint64_t> topo_versions; // the graphs' table versions h_args was built from
     uint64_t build_id = 0;               // unique per batch_build in the process (never 0 once built)
     int n_work_res = 0, n_work_pair = 0, max_N = 1;
-    int max_free = 0;
+    size_t solve_smem = 0;
     int64_t pixels_per_pass = 0;
     cudaGraphExec_t exec = nullptr;
     int exec_iters = -1, exec_shape = -1;

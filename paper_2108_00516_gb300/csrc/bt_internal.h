@@ -205,7 +205,7 @@ cudaError_t launch_batch_residual(const SolveArgs* args_dev, const int2* work_re
                                   bool full, int shape, int precision, cudaStream_t s);
 cudaError_t launch_batch_pairs(const SolveArgs* args_dev, const int2* work_pair, int n_work, bool full,
                                cudaStream_t s);
-cudaError_t launch_batch_solve(const SolveArgs* args_dev, int n_graphs, int max_free, bool full, int iter,
+cudaError_t launch_batch_solve(const SolveArgs* args_dev, int n_graphs, size_t smem, bool full, int iter,
                                cudaStream_t s);
 // Sets every kernel's shared-memory attribute (call before a stream capture).
 void prepare_launch_attributes();

@@ -150,9 +150,7 @@ constexpr int kPan = 6;
 
 // Row groups of the inverse by size of the system: entries of a column in a
 // thread's registers (a multiple of six) and groups, one warp a group and
-// block of 32 columns.  The largest shape takes a kernel of its own (kLarge):
-// beside the others it costs 250 registers instead of 180 and 0.5 % of a
-// ten-view solve.
+// block of 32 columns.
 struct InvShape {
     int rows, groups;
 };
@@ -162,7 +160,6 @@ __host__ __device__ constexpr InvShape inv_shape(int n)
          : n <= 120 ? InvShape{60, 2} : InvShape{138, 1};
 }
 static_assert(kLdltMaxN <= 138, "the inverse holds the largest system");
-__host__ __device__ constexpr bool ldlt_large(int n) { return n > 120; }
 __host__ __device__ constexpr int inv_stride(int kR) { return (kR + 3) & ~3; }      // of a row group, in floats
 // Two panels of six columns and six rows, the solution, the right-hand side.
 __host__ __device__ constexpr size_t inv_floats(int n)
@@ -191,8 +188,7 @@ __host__ __device__ constexpr size_t ldlt_shift_doubles(size_t n) { return (n + 
 // *fail (shared memory, zero on entry) is set when a pivot is not positive; x
 // is then meaningless, and the caller reads *fail after the call (the call
 // ends with a barrier).  inverse: whether to try the inverse first (a system
-// whose predecessor was declined will most often be declined too).  kLarge:
-// whether n may exceed 120 (without it such a system would be factorised).  t_mid:
+// whose predecessor was declined will most often be declined too).  t_mid:
 // every thread's clock after the inverse's solve, or after the factorisation
 // and D w = z.  idle(warp): called once by each of warps 1-7 while warp 0
 // alone runs the first block of the back substitution (work the caller has for
@@ -429,7 +425,7 @@ __device__ __forceinline__ bool inverse_solve(const float2* __restrict__ F, int 
     return false;
 }
 
-template <bool kLarge, typename Idle = LdltNoIdle>
+template <typename Idle = LdltNoIdle>
 __device__ __forceinline__ bool ldlt_solve(double* __restrict__ H, int ld, int n, double* __restrict__ y,
                                            const LdltScratch& sc, bool inverse, int* fail, unsigned long long& t_mid,
                                            const Idle& idle = Idle())
@@ -489,13 +485,12 @@ __device__ __forceinline__ bool ldlt_solve(double* __restrict__ H, int ld, int n
                 for (int i = lane; i < n; i += 32) b[i] = ff_from_f64(y[i], shift[i] + e);
             }
             __syncthreads();
-            bool done = false;
-            if (n <= 12) done = inverse_solve<6, 2>(F, ld, n, b, buf, p, x);
-            else if (n <= 30) done = inverse_solve<6, 5>(F, ld, n, b, buf, p, x);
-            else if (n <= 60) done = inverse_solve<18, 4>(F, ld, n, b, buf, p, x);
-            else if (n <= 96) done = inverse_solve<48, 2>(F, ld, n, b, buf, p, x);
-            else if (n <= 120) done = inverse_solve<60, 2>(F, ld, n, b, buf, p, x);
-            else if constexpr (kLarge) done = inverse_solve<138, 1>(F, ld, n, b, buf, p, x);
+            const bool done = n <= 12    ? inverse_solve<6, 2>(F, ld, n, b, buf, p, x)
+                              : n <= 30  ? inverse_solve<6, 5>(F, ld, n, b, buf, p, x)
+                              : n <= 60  ? inverse_solve<18, 4>(F, ld, n, b, buf, p, x)
+                              : n <= 96  ? inverse_solve<48, 2>(F, ld, n, b, buf, p, x)
+                              : n <= 120 ? inverse_solve<60, 2>(F, ld, n, b, buf, p, x)
+                                         : inverse_solve<138, 1>(F, ld, n, b, buf, p, x);
             if (done) {
                 t_mid = clock64();
                 for (int i = tid; i < n; i += nt) y[i] = ff_to_f64(x[i], shift[i] - shift[n]);

@@ -397,7 +397,7 @@ __device__ __forceinline__ FinalPrefetch final_prefetch(const SolveArgs& a)
     return pf;
 }
 
-template <bool kFull, bool kLarge>
+template <bool kFull>
 __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const FinalPrefetch& pf)
 {
     const int N = a.N, U = a.n_upairs;
@@ -658,7 +658,7 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
     // warp 0 runs the first block of the back substitution alone.  The systems
     // of a solve's iterations are much alike: where one was left to the
     // factorisation, the later ones go straight to it
-    costs_due = !ldlt_solve<kLarge>(H, ld, n, y, sc, pf.declined == 0, &s_fail, t2, [&](int w) {
+    costs_due = !ldlt_solve(H, ld, n, y, sc, pf.declined == 0, &s_fail, t2, [&](int w) {
         if (w == cost_warp) write_costs();
     });
     if (!costs_due && tid == 0) a.ctrl->declined = 1;
@@ -732,7 +732,7 @@ __device__ void final_phase(const SolveArgs& a, int iter, double* sm, const Fina
     }
 }
 
-template <bool kFull, bool kLarge>
+template <bool kFull>
 __global__ void __launch_bounds__(kThreads, 1) reduce_kernel(SolveArgs a, int iter)
 {
     extern __shared__ __align__(16) double sm[];
@@ -753,7 +753,7 @@ __global__ void __launch_bounds__(kThreads, 1) reduce_kernel(SolveArgs a, int it
     if (!s_last) return;
     __threadfence();
     if (threadIdx.x == 0) a.ctrl->counter = 0u;
-    final_phase<kFull, kLarge>(a, iter, sm, pf);
+    final_phase<kFull>(a, iter, sm, pf);
 }
 
 size_t reduce_smem_bytes(int n_free)
@@ -767,25 +767,19 @@ size_t reduce_smem_bytes(int n_free)
     return fin > ph1 ? fin : ph1;
 }
 
-template <typename... K>
-static void set_solve_smem(K*... kernels)
-{
-    (cudaFuncSetAttribute(kernels, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kReduceSmemMax), ...);
-}
-
 cudaError_t launch_reduce(const SolveArgs& a, bool full, int iter, cudaStream_t s)
 {
     static const bool attr_set = [] {      // once per process, thread-safe
-        set_solve_smem(reduce_kernel<true, false>, reduce_kernel<true, true>, reduce_kernel<false, false>);
+        cudaFuncSetAttribute(reduce_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kReduceSmemMax);
+        cudaFuncSetAttribute(reduce_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kReduceSmemMax);
         return true;
     }();
     (void)attr_set;
     const int grid = a.n_upairs > 0 ? a.n_upairs : 1;
     const size_t smem = reduce_smem_bytes(a.n_free);
-    auto kernel = !full                      ? reduce_kernel<false, false>
-                  : ldlt_large(6 * a.n_free) ? reduce_kernel<true, true>
-                                             : reduce_kernel<true, false>;
-    return launch_chained(kernel, dim3(grid), dim3(kThreads), smem, s, a, iter);
+    if (full)
+        return launch_chained(reduce_kernel<true>, dim3(grid), dim3(kThreads), smem, s, a, iter);
+    return launch_chained(reduce_kernel<false>, dim3(grid), dim3(kThreads), smem, s, a, iter);
 }
 
 // ---------------------------------------------------------------------------
@@ -815,7 +809,7 @@ __global__ void __launch_bounds__(kThreads) batch_pair_kernel(const SolveArgs* _
     reduce_upair<kFull>(sa, w.y, sm);
 }
 
-template <bool kFull, bool kLarge>
+template <bool kFull>
 __global__ void __launch_bounds__(kThreads, 1) batch_solve_kernel(const SolveArgs* __restrict__ args, int iter)
 {
     pdl_wait_and_release();
@@ -823,7 +817,7 @@ __global__ void __launch_bounds__(kThreads, 1) batch_solve_kernel(const SolveArg
     __shared__ SolveArgs sa;
     if (threadIdx.x == 0) sa = args[blockIdx.x];
     __syncthreads();
-    final_phase<kFull, kLarge>(sa, iter, smd, final_prefetch<kFull>(sa));
+    final_phase<kFull>(sa, iter, smd, final_prefetch<kFull>(sa));
 }
 
 cudaError_t launch_batch_xforms(const SolveArgs* args_dev, int n_graphs, cudaStream_t s)
@@ -841,26 +835,28 @@ cudaError_t launch_batch_pairs(const SolveArgs* args_dev, const int2* work_pair,
     return launch_chained(batch_pair_kernel<false>, dim3(n_work), dim3(kThreads), 0, s, args_dev, work_pair);
 }
 
-cudaError_t launch_batch_solve(const SolveArgs* args_dev, int n_graphs, int max_free, bool full, int iter,
+cudaError_t launch_batch_solve(const SolveArgs* args_dev, int n_graphs, size_t smem, bool full, int iter,
                                cudaStream_t s)
 {
     static const bool attr_set = [] {      // once per process, thread-safe
-        set_solve_smem(batch_solve_kernel<true, false>, batch_solve_kernel<true, true>, batch_solve_kernel<false, false>);
+        cudaFuncSetAttribute(batch_solve_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kReduceSmemMax);
+        cudaFuncSetAttribute(batch_solve_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kReduceSmemMax);
         return true;
     }();
     (void)attr_set;
     if (n_graphs == 0) return cudaSuccess;
-    auto kernel = !full                      ? batch_solve_kernel<false, false>
-                  : ldlt_large(6 * max_free) ? batch_solve_kernel<true, true>
-                                             : batch_solve_kernel<true, false>;
-    return launch_chained(kernel, dim3(n_graphs), dim3(kThreads), reduce_smem_bytes(max_free), s, args_dev, iter);
+    if (full)
+        return launch_chained(batch_solve_kernel<true>, dim3(n_graphs), dim3(kThreads), smem, s, args_dev, iter);
+    return launch_chained(batch_solve_kernel<false>, dim3(n_graphs), dim3(kThreads), smem, s, args_dev, iter);
 }
 
 void prepare_launch_attributes()
 {
     prepare_residual_attributes();
-    set_solve_smem(batch_solve_kernel<true, false>, batch_solve_kernel<true, true>, batch_solve_kernel<false, false>);
-    set_solve_smem(reduce_kernel<true, false>, reduce_kernel<true, true>, reduce_kernel<false, false>);
+    cudaFuncSetAttribute(batch_solve_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kReduceSmemMax);
+    cudaFuncSetAttribute(batch_solve_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kReduceSmemMax);
+    cudaFuncSetAttribute(reduce_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kReduceSmemMax);
+    cudaFuncSetAttribute(reduce_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kReduceSmemMax);
 }
 
 }  // namespace bt

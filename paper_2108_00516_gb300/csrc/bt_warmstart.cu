@@ -1232,7 +1232,6 @@ __device__ __forceinline__ void tri_rc(int q, int& r, int& c)
     c = q - r * (r + 1) / 2;
 }
 
-template <bool kLarge>
 __global__ void __launch_bounds__(kAvgThreads) average_kernel(const AvgGraph* __restrict__ graphs)
 {
     extern __shared__ __align__(16) double asm_[];
@@ -1391,7 +1390,7 @@ __global__ void __launch_bounds__(kAvgThreads) average_kernel(const AvgGraph* __
     // or a solution that is not finite, leaves the poses as they were
     if (n > 0) {
         unsigned long long t_unused;
-        ldlt_solve<kLarge>(H, ld, n, b, sc, true, &s_sing, t_unused);
+        ldlt_solve(H, ld, n, b, sc, true, &s_sing, t_unused);
         for (int i = tid; i < n; i += kAvgThreads)
             if (!isfinite(b[i])) s_sing = 1;
         __syncthreads();
@@ -1478,14 +1477,12 @@ cudaError_t launch_average(const AvgGraph* graphs, int n_graphs, int max_free, c
     if (n_graphs <= 0) return cudaSuccess;
     const size_t smem = average_smem_bytes(max_free, kMaxNodes);
     static const bool attr = [] {         // once per process, thread-safe
-        for (auto k : {average_kernel<false>, average_kernel<true>})
-            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)average_smem_bytes(kMaxNodes - 1, kMaxNodes));
+        cudaFuncSetAttribute(average_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)average_smem_bytes(kMaxNodes - 1, kMaxNodes));
         return true;
     }();
     (void)attr;
-    if (ldlt_large(6 * max_free)) average_kernel<true><<<n_graphs, kAvgThreads, smem, s>>>(graphs);
-    else average_kernel<false><<<n_graphs, kAvgThreads, smem, s>>>(graphs);
+    average_kernel<<<n_graphs, kAvgThreads, smem, s>>>(graphs);
     return cudaGetLastError();
 }
 
